@@ -1,0 +1,337 @@
+// Products of spectra modulo 31-bit primes: the transforms of the fused estimator for
+// lengths N = 2^10 .. 2^22.  Included by sk_estimate.cu only.
+//
+// A length-N transform of a counter vector is split as N = R x 1024 (element n = 1024 n1 + n2,
+// frequency nu = k1 + R k2):
+//   k_ntt_cols  reads the int64 counters, reduces them modulo the prime, transforms the columns
+//               (over n1, length R), multiplies by w_N^(n2 k1) and stores [k1][n2] residues;
+//   k_ntt_rows  gives one warp the rows k1 of all r relations of one output: each row's
+//               1024-point transform (32 x 32) stays in the warp's registers with one
+//               shared-memory transposition, the r spectra are multiplied as they appear and
+//               only their sum over nu leaves the SM.
+// A relation whose spectrum is taken at -nu is transformed with the inverse root instead, so
+// that all factors of a product sit in the same lane and register.  All primes of an estimate
+// run in one launch (grid y).
+//
+// Bound: integer issue.  Per element and prime about 75 instructions in the column pass and 60
+// in the row pass against 12 bytes read and 4 written; a separate residue pass, spectra written
+// back and products in their own kernel cost 4.3 passes over the residues more.
+//
+// Residues are plain (not in Montgomery form); the twiddles are in Montgomery form with
+// R = 2^32, so x (*) w is again a plain residue.  The r - 1 products of spectra each bring a
+// factor 2^-32, which the host takes out of the final sums.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace sk {
+namespace ntt {
+
+constexpr int kMaxPrimes = 9;
+constexpr int kLogRow = 10;                 // row length 1024
+constexpr int kMinLog = 10, kMaxLog = 22;   // transform lengths
+
+struct PrimeConst {
+  uint32_t p, pinv;       // pinv = -p^-1 mod 2^32
+  uint32_t r2;            // 2^64 mod p
+  uint32_t w64[2][32];    // w_64^j, j < 32 (Montgomery form): [0] forward, [1] inverse root
+};
+__constant__ PrimeConst c_prime[kMaxPrimes];
+
+// Powers of the roots of unity, Montgomery form, [prime][direction]:
+__device__ uint32_t g_root[kMaxPrimes][2][4096];                           // w_4096^e
+__device__ uint32_t g_low[kMaxPrimes][2][kMaxLog - kMinLog + 1][1024];     // w_N^e, e < 1024
+__device__ uint32_t g_row[kMaxPrimes][2][1024];                            // w_1024^(c b) at 32 c + b
+
+struct Mod {
+  uint32_t p, pinv;
+};
+
+// a + b, a - b mod p for a, b < p < 2^31: the wrapped candidate is the larger one
+__device__ __forceinline__ uint32_t add(uint32_t a, uint32_t b, Mod q) {
+  const uint32_t s = a + b;
+  return min(s, s - q.p);
+}
+__device__ __forceinline__ uint32_t sub(uint32_t a, uint32_t b, Mod q) {
+  const uint32_t s = a - b;
+  return min(s, s + q.p);
+}
+// a b 2^-32 mod p for a b < 2^32 * 2^31 (Montgomery): t + q p < 2^64, its high word < 2p
+__device__ __forceinline__ uint32_t mul(uint32_t a, uint32_t b, Mod q) {
+  const uint64_t t = (uint64_t)a * b;
+  const uint32_t m = (uint32_t)t * q.pinv;
+  const uint32_t u = (uint32_t)((t + (uint64_t)m * q.p) >> 32);
+  return min(u, u - q.p);
+}
+
+// c mod p.  |c| < 2^30 < p in two instructions; any int64 through two Montgomery products
+// per half of |c| = h 2^32 + l.
+__device__ __forceinline__ uint32_t residue(int64_t c, Mod q, uint32_t r2) {
+  if ((uint64_t)(c + (1ll << 30)) < (1ull << 31)) {
+    const uint32_t x = (uint32_t)c;
+    return min(x, x + q.p);
+  }
+  const uint64_t mag = c < 0 ? 0ull - (uint64_t)c : (uint64_t)c;
+  const uint32_t v = add(mul(mul((uint32_t)mag, r2, q), 1u, q), mul((uint32_t)(mag >> 32), r2, q), q);
+  return c < 0 && v ? q.p - v : v;
+}
+
+constexpr int rev_bits(int k, int bits) {
+  int r = 0;
+  for (int i = 0; i < bits; i++) r |= ((k >> i) & 1) << (bits - 1 - i);
+  return r;
+}
+
+// 2^LOG-point DFT in registers, natural order in and out; w64[j] = w_64^j.  Radix-2 decimation
+// in frequency; the difference of a butterfly with a twiddle is left in (0, 2p) for mul.
+template <int LOG>
+__device__ __forceinline__ void dft(uint32_t (&x)[1 << LOG], const uint32_t* w64, Mod q) {
+  constexpr int N = 1 << LOG;
+#pragma unroll
+  for (int st = 0; st < LOG; st++) {
+    const int h = N >> (st + 1);
+#pragma unroll
+    for (int blk = 0; blk < N; blk += 2 * h) {
+#pragma unroll
+      for (int j = 0; j < h; j++) {
+        const uint32_t u = x[blk + j], v = x[blk + j + h];
+        x[blk + j] = add(u, v, q);
+        x[blk + j + h] = j == 0 ? sub(u, v, q) : mul(u - v + q.p, w64[(j << st) << (6 - LOG)], q);
+      }
+    }
+  }
+  uint32_t y[N];
+#pragma unroll
+  for (int k = 0; k < N; k++) y[k] = x[rev_bits(k, LOG)];
+#pragma unroll
+  for (int k = 0; k < N; k++) x[k] = y[k];
+}
+
+// Vectors of one launch: vector v is base[v / per] + (v % per) m (m int64 counters, taken as
+// zero from m to N); its direction (1: inverse root) is dirs[v] or bit v / per of negmask.
+struct ColArgs {
+  const int64_t* const* base;
+  int per;
+  int64_t m;
+  unsigned long long negmask;
+  const uint8_t* dirs;
+  int logR;
+  uint32_t* V;              // [prime][stride vectors][N]
+  int64_t stride;           // vectors per prime in V
+  int prime0;               // prime of grid y = 0
+  int nvec[kMaxPrimes];     // vectors of each prime (leading ones)
+};
+
+__device__ __forceinline__ int dir_of(const ColArgs& a, int64_t v) {
+  return a.dirs ? a.dirs[v] : (int)((a.negmask >> (v / a.per)) & 1ull);
+}
+
+// w_N^e for e < N = R 1024
+__device__ __forceinline__ uint32_t root_pow(int prime, int dir, int logR, uint32_t e, Mod q) {
+  const uint32_t lo = g_low[prime][dir][logR][e & 1023u], hi = e >> kLogRow;
+  return hi ? mul(lo, g_root[prime][dir][hi << (12 - logR)], q) : lo;
+}
+
+// R = 2^(LA + LB).  A thread of a CTA of 256 holds one A- or B-point DFT (A <= B) of one of cb =
+// 256 / A columns: the counters go from global memory into registers, through one shared-memory
+// exchange between the two levels and back to global memory.  LA = 0: R = B points per thread,
+// no exchange.  64-byte column segments are read and 32-byte ones written at least, so tiles
+// wider than eight columns would not save sectors.
+template <int LA, int LB>
+__global__ void __launch_bounds__(256, (LB <= 5 ? 3 : 2)) k_ntt_cols(const __grid_constant__ ColArgs a) {
+  constexpr int A = 1 << LA, B = 1 << LB, LR = LA + LB;
+  constexpr int LCB = LA ? 8 - LA : 8, CB = 1 << LCB;
+  const int prime = a.prime0 + (int)blockIdx.y;
+  const int64_t vec = blockIdx.x >> (kLogRow - LCB);
+  if (vec >= a.nvec[prime]) return;
+  const int n2 = (int)(blockIdx.x & ((1u << (kLogRow - LCB)) - 1u)) * CB + (int)(threadIdx.x & (CB - 1));
+  const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
+  const uint32_t r2 = c_prime[prime].r2;
+  const int dir = dir_of(a, vec);
+  const uint32_t* w64 = c_prime[prime].w64[dir];
+  const int64_t* src = a.base[vec / a.per] + (vec % a.per) * a.m + n2;
+  uint32_t* dst = a.V + (((int64_t)blockIdx.y * a.stride + vec) << (LR + kLogRow)) + n2;
+  const int64_t left = a.m - n2;   // counters of this column: rows n1 with 1024 n1 < left
+  extern __shared__ uint32_t s_col[];
+  const int c = (int)(threadIdx.x >> LCB);   // this thread's k1 residue at the second level
+  uint32_t x[B];
+  if constexpr (LA > 0) {
+    // [c][b] twiddles w_R^(c b), then the exchange tile: element (c, b) of column v at
+    // (c (B + 1) + b) CB + v, which keeps writes (b, v fast) and reads (c, v fast) conflict-free
+    uint32_t* tw = s_col;
+    uint32_t* ex = s_col + A * B;
+    for (int i = threadIdx.x; i < A * B; i += 256)
+      tw[i] = g_root[prime][dir][((i >> LB) * (i & (B - 1))) << (12 - LR)];
+    __syncthreads();
+    const int v = (int)(threadIdx.x & (CB - 1));
+#pragma unroll
+    for (int s = 0; s < B / A; s++) {
+      const int b = (int)(threadIdx.x >> LCB) + A * s;
+      uint32_t y[A];
+#pragma unroll
+      for (int i = 0; i < A; i++) {
+        const int64_t at = (int64_t)(B * i + b) << kLogRow;
+        y[i] = at < left ? residue(__ldg(src + at), q, r2) : 0u;
+      }
+      dft<LA>(y, w64, q);
+#pragma unroll
+      for (int i = 0; i < A; i++) ex[(i * (B + 1) + b) * CB + v] = i ? mul(y[i], tw[i * B + b], q) : y[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < B; b++) x[b] = ex[(c * (B + 1) + b) * CB + v];
+  } else {
+#pragma unroll
+    for (int i = 0; i < B; i++) {
+      const int64_t at = (int64_t)i << kLogRow;
+      x[i] = at < left ? residue(__ldg(src + at), q, r2) : 0u;
+    }
+  }
+  dft<LB>(x, w64, q);
+  // x[e] is row k1 = c + A e: times w_N^(n2 k1), advanced in two chains of step w_N^(2 A n2)
+  if constexpr (LR > 0) {
+    const uint32_t k0 = LA ? (uint32_t)c : 0u;
+    uint32_t w0 = root_pow(prime, dir, LR, (uint32_t)n2 * k0, q);
+    const uint32_t st = root_pow(prime, dir, LR, (uint32_t)n2 * A, q);
+    uint32_t w1 = mul(w0, st, q);
+    const uint32_t st2 = mul(st, st, q);
+#pragma unroll
+    for (int e = 0; e < B; e += 2) {
+      dst[(int64_t)(k0 + A * e) << kLogRow] = mul(x[e], w0, q);
+      dst[(int64_t)(k0 + A * (e + 1)) << kLogRow] = mul(x[e + 1], w1, q);
+      if (e + 2 < B) {
+        w0 = mul(w0, st2, q);
+        w1 = mul(w1, st2, q);
+      }
+    }
+  } else {
+    dst[0] = x[0];
+  }
+}
+
+// One output: the product over its r vectors base + k step (k < r).
+struct Out {
+  int64_t base, step;
+  int r;
+  unsigned long long negmask;   // bit k: vector k was transformed with the inverse root
+};
+
+struct RowArgs {
+  const uint32_t* V;
+  int64_t stride;
+  int logR, prime0;
+  const Out* outs;            // nullptr: output o is {o, one.step, one.r, one.negmask}
+  Out one;
+  int nout[kMaxPrimes];
+  unsigned long long* sums;   // [out][kMaxPrimes] += sum over nu of the product (residues < p)
+};
+
+// 8 warps, one row k1 each; sums of at most 2^22 residues below 2^31 fit 64 bits.
+__global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ RowArgs a) {
+  __shared__ uint32_t s_tw[2][1024];
+  __shared__ uint32_t s_ex[8][32 * 33];
+  __shared__ unsigned long long s_sum[8];
+  const int prime = a.prime0 + (int)blockIdx.y;
+  const int R = 1 << a.logR;
+  const int lcta = a.logR > 3 ? a.logR - 3 : 0;   // log2 CTAs per output
+  const int64_t o = blockIdx.x >> lcta;
+  if (o >= a.nout[prime]) return;
+  const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
+  const int k1 = (int)(blockIdx.x & ((1u << lcta) - 1u)) * 8 + warp;
+  const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
+  for (int i = threadIdx.x; i < 2048; i += 256) ((uint32_t*)s_tw)[i] = ((const uint32_t*)g_row[prime])[i];
+  __syncthreads();
+  unsigned long long sum = 0;
+  if (k1 < R) {
+    Out f;
+    if (a.outs) {
+      f = a.outs[o];
+    } else {
+      f = a.one;
+      f.base = o;
+    }
+    const uint32_t* row =
+        a.V + (((int64_t)blockIdx.y * a.stride + f.base) << (a.logR + kLogRow)) + ((int64_t)k1 << kLogRow) + lane;
+    const int64_t rstep = f.step << (a.logR + kLogRow);
+    uint32_t* ex = s_ex[warp];
+    uint32_t prod[32], x[32];
+#pragma unroll
+    for (int i = 0; i < 32; i++) x[i] = __ldcs(row + 32 * i);
+    for (int k = 0; k < f.r; k++) {
+      const int dir = (int)((f.negmask >> k) & 1ull);
+      const uint32_t* w64 = c_prime[prime].w64[dir];
+      const uint32_t* tw = s_tw[dir];
+      dft<5>(x, w64, q);
+#pragma unroll
+      for (int i = 0; i < 32; i++) ex[i * 33 + lane] = i ? mul(x[i], tw[i * 32 + lane], q) : x[i];
+      __syncwarp();
+      uint32_t y[32];
+#pragma unroll
+      for (int i = 0; i < 32; i++) y[i] = ex[lane * 33 + i];
+      __syncwarp();
+      row += rstep;
+      if (k + 1 < f.r) {   // the next vector's row, in flight during this one's second level
+#pragma unroll
+        for (int i = 0; i < 32; i++) x[i] = __ldcs(row + 32 * i);
+      }
+      dft<5>(y, w64, q);
+      if (k == 0) {
+#pragma unroll
+        for (int i = 0; i < 32; i++) prod[i] = y[i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; i++) prod[i] = mul(prod[i], y[i], q);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; i++) sum += prod[i];
+  }
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, s);
+  if (lane == 0) s_sum[warp] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) sum += s_sum[w];
+    atomicAdd(a.sums + o * kMaxPrimes + prime, sum);
+  }
+}
+
+template <int LA, int LB>
+cudaError_t launch_cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+  constexpr int LCB = LA ? 8 - LA : 8;
+  const size_t smem = LA ? ((size_t)(1 << (LA + LB)) + ((size_t)(1 << LA) * ((1 << LB) + 1) << LCB)) * 4 : 0;
+  const cudaError_t e = fit_dynamic_smem((const void*)k_ntt_cols<LA, LB>, smem);
+  if (e != cudaSuccess) return e;
+  k_ntt_cols<LA, LB><<<dim3((unsigned)(nvec << (kLogRow - LCB)), (unsigned)primes), 256, smem, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+inline cudaError_t cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+  switch (a.logR) {
+    case 0: return launch_cols<0, 0>(a, nvec, primes, st);
+    case 1: return launch_cols<0, 1>(a, nvec, primes, st);
+    case 2: return launch_cols<0, 2>(a, nvec, primes, st);
+    case 3: return launch_cols<0, 3>(a, nvec, primes, st);
+    case 4: return launch_cols<0, 4>(a, nvec, primes, st);
+    case 5: return launch_cols<0, 5>(a, nvec, primes, st);
+    case 6: return launch_cols<3, 3>(a, nvec, primes, st);
+    case 7: return launch_cols<3, 4>(a, nvec, primes, st);
+    case 8: return launch_cols<4, 4>(a, nvec, primes, st);
+    case 9: return launch_cols<4, 5>(a, nvec, primes, st);
+    case 10: return launch_cols<5, 5>(a, nvec, primes, st);
+    case 11: return launch_cols<5, 6>(a, nvec, primes, st);
+    default: return launch_cols<6, 6>(a, nvec, primes, st);
+  }
+}
+
+inline cudaError_t rows(const RowArgs& a, int64_t nout, int primes, cudaStream_t st) {
+  const int lcta = a.logR > 3 ? a.logR - 3 : 0;
+  k_ntt_rows<<<dim3((unsigned)(nout << lcta), (unsigned)primes), 256, 0, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace ntt
+}  // namespace sk
