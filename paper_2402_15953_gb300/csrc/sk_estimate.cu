@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "sk_internal.h"
+#include "sk_ntt.cuh"
 
 namespace sk {
 namespace {
@@ -1696,7 +1697,7 @@ uint32_t fu_to_mont(uint64_t v, uint32_t p) { return (uint32_t)(((unsigned __int
 // host work that every estimate would otherwise repeat): w, a root of unity of order exactly
 // M, its inverse, and in Montgomery form w, w^-1, w^(M/4), w^(-M/4), M^-1 and 1.
 struct FuWidth {
-  uint64_t w = 1, winv = 1;
+  uint64_t w = 1, winv = 1, minv_p = 1;   // minv_p = M^-1 mod p (plain)
   uint32_t w_m = 0, winv_m = 0, r4 = 0, r4i = 0, minv = 0, one = 0;
 };
 
@@ -1718,7 +1719,8 @@ const FuWidth& fu_width(int i, int64_t M) {
       f.winv_m = fu_to_mont(f.winv, pr[k].p);
       f.r4 = M >= 4 ? fu_to_mont(fu_powmod(f.w, (uint64_t)M / 4, p), pr[k].p) : f.one;
       f.r4i = M >= 4 ? fu_to_mont(fu_powmod(f.winv, (uint64_t)M / 4, p), pr[k].p) : f.one;
-      f.minv = fu_to_mont(fu_powmod((uint64_t)M % p, p - 2, p), pr[k].p);
+      f.minv_p = fu_powmod((uint64_t)M % p, p - 2, p);
+      f.minv = fu_to_mont(f.minv_p, pr[k].p);
     }
     it = cache.emplace(M, std::move(v)).first;
   }
@@ -1991,6 +1993,58 @@ bool fu_eligible(const sk_set* s, unsigned long long* negmask) {
   return true;
 }
 
+// Fills the current device's root tables of sk_ntt.cuh (about 1.3 MB, a few milliseconds of
+// host arithmetic, once per device and process).
+cudaError_t ntt_constants() {
+  const std::vector<FuPrime>& pr = fu_primes();
+  constexpr int NP = ntt::kMaxPrimes, NL = ntt::kMaxLog - ntt::kMinLog + 1;
+  static_assert(NP == kFuMaxPrimes, "one table per CRT prime");
+  std::vector<uint32_t> root((size_t)NP * 2 * 4096), low((size_t)NP * 2 * NL * 1024), row((size_t)NP * 2 * 1024);
+  std::vector<ntt::PrimeConst> pc(NP);
+  for (int i = 0; i < NP; i++) {
+    const uint64_t p = pr[i].p;
+    pc[i].p = pr[i].p;
+    pc[i].pinv = pr[i].pinv;
+    pc[i].r2 = pr[i].r2;
+    for (int dir = 0; dir < 2; dir++) {
+      // w_n^e for e < count, Montgomery form, w_n = g^(+-(p - 1) / n)
+      auto powers = [&](int64_t n, int count, uint32_t* out) {
+        uint64_t w = fu_powmod(pr[i].g, (p - 1) / (uint64_t)n, p);
+        if (dir) w = fu_powmod(w, p - 2, p);
+        uint64_t v = (1ull << 32) % p;
+        for (int e = 0; e < count; e++, v = v * w % p) out[e] = (uint32_t)v;
+      };
+      uint32_t* r = &root[((size_t)i * 2 + dir) * 4096];
+      powers(4096, 4096, r);
+      for (int k = 0; k < NL; k++)
+        powers((int64_t)1 << (ntt::kMinLog + k), 1024, &low[(((size_t)i * 2 + dir) * NL + k) * 1024]);
+      for (int e = 0; e < 1024; e++) row[((size_t)i * 2 + dir) * 1024 + e] = r[4 * ((e >> 5) * (e & 31))];
+      for (int j = 0; j < 32; j++) pc[i].w64[dir][j] = r[64 * j];
+    }
+  }
+  cudaError_t e = cudaMemcpyToSymbol(ntt::g_root, root.data(), root.size() * 4);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_low, low.data(), low.size() * 4);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_row, row.data(), row.size() * 4);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::c_prime, pc.data(), pc.size() * sizeof(ntt::PrimeConst));
+  return e;
+}
+
+// The residue of a row estimate mod prime i from its sum of products of r spectra (which
+// carries 2^(-32 (r - 1)), see sk_ntt.cuh): sum 2^(32 (r - 1)) / M mod p.
+uint32_t ntt_row_residue(int i, int64_t M, int r, unsigned long long sum) {
+  const uint64_t p = fu_primes()[i].p;
+  const uint64_t f = fu_powmod((1ull << 32) % p, (uint64_t)(r - 1), p) * fu_width(i, M).minv_p % p;
+  return (uint32_t)(sum % p * f % p);
+}
+
+// Residue vectors one launch holds at a time: every prime's while they fit 256 MiB (small
+// estimates are bound by their launches), else two primes' (the least that keeps the second
+// prime's blocks behind the first's last wave).
+int ntt_primes_at_once(size_t words, int np) {
+  const size_t budget = (size_t)256 << 20;
+  return (int)std::min<size_t>(np, std::max<size_t>(2, budget / (words * sizeof(uint32_t))));
+}
+
 std::mutex g_fu_const_mutex;
 bool g_fu_const_ready[64] = {false};
 
@@ -2012,6 +2066,7 @@ cudaError_t fu_constants(bool* ready) {
     }
     cudaError_t e = cudaMemcpyToSymbol(c_fu_p, ps, sizeof(ps));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_fu_pinv, pis, sizeof(pis));
+    if (e == cudaSuccess) e = ntt_constants();
     if (e != cudaSuccess) return e;
     g_fu_const_ready[dev] = true;
   }
@@ -2031,17 +2086,17 @@ struct FuSetup {
   int np = 0;
 };
 
-sk_status fu_setup(sk_set* s, int64_t M, bool pairwise, cudaStream_t st, FuSetup* f) {
+sk_status fu_setup(sk_set* s, int64_t M, bool pairwise, bool tables, cudaStream_t st, FuSetup* f) {
   const int64_t m = s->m;
   const int r = s->r, d = s->d;
   const std::vector<FuPrime>& pr = fu_primes();
   SK_CK(fu_rel_table(s, st));
-  // scratch: norm partials [r][d][l1ch][2] doubles | residues [d][9] | partials [d][nchunk]
+  // scratch: norm partials [r][d][l1ch][2] doubles | residues or 64-bit sums [d][9] | partials [d][nchunk]
   int nchunk = 1;
   while ((int64_t)nchunk * 2 * 256 <= M && (int64_t)d * nchunk * 2 <= 4096) nchunk *= 2;
   const int l1ch = fu_l1_chunks((int64_t)r * d, m);
   const size_t l1_bytes = ((size_t)r * d * l1ch * 16 + 255) & ~(size_t)255;
-  const size_t res_bytes = ((size_t)d * kFuMaxPrimes * 4 + 255) & ~(size_t)255;
+  const size_t res_bytes = ((size_t)d * kFuMaxPrimes * 8 + 255) & ~(size_t)255;
   const size_t part_bytes = ((size_t)d * nchunk * 4 + 255) & ~(size_t)255;
   SK_CK(ensure(s->scratch, l1_bytes + res_bytes + part_bytes, st));
   double* d_l1 = (double*)s->scratch.ptr;
@@ -2057,7 +2112,7 @@ sk_status fu_setup(sk_set* s, int64_t M, bool pairwise, cudaStream_t st, FuSetup
   double cover = 0.0;
   while (np < kFuMaxPrimes && cover < bits + 3.0) cover += pr[np++].log2p;
   f->np = cover < bits + 3.0 ? 0 : np;
-  if (f->np && (s->fu_m != M || !s->d_fu_tw)) {
+  if (f->np && tables && (s->fu_m != M || !s->d_fu_tw)) {
     s->fu_np = 0;
     SK_CK(table_alloc((void**)&s->d_fu_tw, (size_t)kFuMaxPrimes * M * sizeof(uint32_t), st));
     s->fu_m = M;
@@ -2065,26 +2120,31 @@ sk_status fu_setup(sk_set* s, int64_t M, bool pairwise, cudaStream_t st, FuSetup
   return SK_OK;
 }
 
-// Reads the residues back, reconstructs each row by CRT and fills *out.
-sk_status fu_finish(sk_set* s, const FuSetup& f, sk_estimate* out, cudaStream_t st) {
+// Reconstructs each row from its residues [d][kFuMaxPrimes] by CRT and fills *out.
+sk_status fu_fill(const sk_set* s, const uint32_t* res, int np, sk_estimate* out) {
   const int d = s->d;
   const std::vector<FuPrime>& pr = fu_primes();
-  s->fu_np = std::max(s->fu_np, f.np);
-  std::vector<uint32_t> res((size_t)d * kFuMaxPrimes);
-  SK_CK(cudaMemcpyAsync(res.data(), f.d_res, res.size() * 4, cudaMemcpyDeviceToHost, st));
-  SK_CK(cudaStreamSynchronize(st));
   I256 rows[SK_MAX_ROWS], sorted[SK_MAX_ROWS];
   for (int row = 0; row < d; row++)
-    if (!fu_crt(res.data() + (size_t)row * kFuMaxPrimes, f.np, pr, &rows[row])) return SK_ERR_OVERFLOW;
+    if (!fu_crt(res + (size_t)row * kFuMaxPrimes, np, pr, &rows[row])) return SK_ERR_OVERFLOW;
   std::memcpy(sorted, rows, sizeof(I256) * d);
   std::sort(sorted, sorted + d, [](const I256& a, const I256& b) { return i256_lt(a, b); });
   fill_estimate(out, rows, sorted, d);
   out->max_residual = 0.0;
-  out->max_limbs = f.np;      // CRT primes
+  out->max_limbs = np;      // CRT primes
   out->limb_bits = 0;
   out->corr_steps = s->corr_steps;
   out->retries = 0;
   return SK_OK;
+}
+
+// Reads the residues back and fills *out.
+sk_status fu_finish(sk_set* s, const FuSetup& f, sk_estimate* out, cudaStream_t st) {
+  s->fu_np = std::max(s->fu_np, f.np);
+  std::vector<uint32_t> res((size_t)s->d * kFuMaxPrimes);
+  SK_CK(cudaMemcpyAsync(res.data(), f.d_res, res.size() * 4, cudaMemcpyDeviceToHost, st));
+  SK_CK(cudaStreamSynchronize(st));
+  return fu_fill(s, res.data(), f.np, out);
 }
 
 // Twiddles of prime PI for length M (once per set and length).
@@ -2190,11 +2250,55 @@ sk_status run_estimate_pairwise(sk_set* s, sk_estimate* out, cudaStream_t st, bo
     SK_CK_ST(run_estimate_pairwise_small(s, out, negmask, st, done));
     if (*done) return SK_OK;
   }
+  const bool wide = m >= (1ll << ntt::kMinLog);
   FuSetup f;
-  SK_CK_ST(fu_setup(s, m, true, st, &f));
+  SK_CK_ST(fu_setup(s, m, true, !wide, st, &f));
   if (!f.np) return SK_OK;   // beyond nine primes: the GF(q) steps handle it
   const std::vector<FuPrime>& pr = fu_primes();
   const size_t words = (size_t)s->r * s->d * m;
+  if (wide) {
+    const int at_once = ntt_primes_at_once(words, f.np);
+    SK_CK(ensure(s->fft_scratch, (size_t)at_once * words * sizeof(uint32_t), st));
+    unsigned long long* d_sums = (unsigned long long*)f.d_res;   // [d][kFuMaxPrimes]
+    const size_t nsum = (size_t)s->d * kFuMaxPrimes;
+    SK_CK(cudaMemsetAsync(d_sums, 0, nsum * 8, st));
+    ntt::ColArgs ca;
+    ca.base = s->d_fu_rel;
+    ca.per = s->d;
+    ca.m = m;
+    ca.negmask = negmask;
+    ca.dirs = nullptr;
+    ca.logR = ilog2(m) - ntt::kLogRow;
+    ca.V = (uint32_t*)s->fft_scratch.ptr;
+    ca.stride = (int64_t)s->r * s->d;
+    ntt::RowArgs ra;
+    ra.V = ca.V;
+    ra.stride = ca.stride;
+    ra.logR = ca.logR;
+    ra.outs = nullptr;
+    ra.one = {0, s->d, s->r, negmask};
+    ra.sums = d_sums;
+    for (int i = 0; i < kFuMaxPrimes; i++) {
+      ca.nvec[i] = (int)ca.stride;
+      ra.nout[i] = s->d;
+    }
+    for (int i = 0; i < f.np; i += at_once) {
+      ca.prime0 = ra.prime0 = i;
+      SK_CK(ntt::cols(ca, ca.stride, std::min(at_once, f.np - i), st));
+      SK_CK(ntt::rows(ra, s->d, std::min(at_once, f.np - i), st));
+    }
+    std::vector<unsigned long long> sums(nsum);
+    SK_CK(cudaMemcpyAsync(sums.data(), d_sums, nsum * 8, cudaMemcpyDeviceToHost, st));
+    SK_CK(cudaStreamSynchronize(st));
+    std::vector<uint32_t> res(nsum);
+    for (size_t k = 0; k < nsum; k++) {
+      const int i = (int)(k % kFuMaxPrimes);
+      res[k] = i < f.np ? ntt_row_residue(i, m, s->r, sums[k]) : 0u;
+    }
+    SK_CK_ST(fu_fill(s, res.data(), f.np, out));
+    *done = true;
+    return SK_OK;
+  }
   SK_CK(ensure(s->fft_scratch, 2 * words * sizeof(uint32_t), st));
   uint32_t* V = (uint32_t*)s->fft_scratch.ptr;
   uint32_t* Wb = V + words;
@@ -2354,7 +2458,7 @@ sk_status run_estimate_crt(sk_set* s, sk_estimate* out, cudaStream_t st, bool* d
   const int64_t M = (m & (m - 1)) == 0 ? m : (int64_t)1 << ilog2(2 * m - 1);
   if (M < 2 || M > (1ll << 22) || s->n_slots + 1 > 64) return SK_OK;
   FuSetup f;
-  SK_CK_ST(fu_setup(s, M, false, st, &f));
+  SK_CK_ST(fu_setup(s, M, false, true, st, &f));
   if (!f.np) return SK_OK;
   const std::vector<FuPrime>& pr = fu_primes();
   const size_t dM = (size_t)s->d * M;
