@@ -2983,6 +2983,185 @@ int many_workers() {
   return x < 1 ? 1 : (x > 16 ? 16 : x);
 }
 
+// The groups of width >= 2^10 (sk_ntt.cuh), all of them between two host synchronisations: the
+// norms of every group's vectors first, read back together; then each group's passes with its
+// sets ordered by the primes their own rows need, so that prime i runs only the leading sets
+// that need more than i; then every output's sums read back together.  One set of metadata
+// buffers serves all groups; the residue vectors of a group reuse the previous group's block
+// (stream order).  A set beyond nine primes is left to the caller (done stays 0).
+sk_status ntt_groups(sk_set** sets, const std::map<int64_t, std::vector<int>>& groups, sk_estimate* out,
+                     std::vector<char>& done, cudaStream_t st) {
+  const std::vector<FuPrime>& pr = fu_primes();
+  struct Member {
+    int i;                        // index into sets
+    int np = 0;                   // primes its rows need
+    int64_t vec = 0;              // its first vector in the norms
+    unsigned long long negmask = 0;
+  };
+  struct Group {
+    int64_t M, vec0, nvec;        // its vectors in the norms
+    int nch;                      // norm chunks per vector
+    size_t part0;                 // its first norm partial
+    std::vector<Member> sets;
+    int np = 0;
+    size_t out0 = 0;              // its first output
+    int nvec_at[kFuMaxPrimes] = {0}, nout_at[kFuMaxPrimes] = {0};
+  };
+  std::vector<Group> gs;
+  std::vector<const int64_t*> rows;
+  size_t parts = 0;
+  for (const auto& g : groups) {
+    Group x;
+    x.M = g.first;
+    x.vec0 = (int64_t)rows.size();
+    for (int i : g.second) {
+      Member mb;
+      mb.i = i;
+      mb.vec = (int64_t)rows.size();
+      fu_eligible(sets[i], &mb.negmask);
+      for (int k = 0; k < sets[i]->r; k++)
+        for (int row = 0; row < sets[i]->d; row++) rows.push_back(sets[i]->rel_ctr[k] + (int64_t)row * x.M);
+      x.sets.push_back(mb);
+    }
+    x.nvec = (int64_t)rows.size() - x.vec0;
+    x.nch = fu_l1_chunks(x.nvec, x.M);
+    x.part0 = parts;
+    parts += (size_t)2 * x.nvec * x.nch;
+    gs.push_back(std::move(x));
+  }
+  size_t nout = 0;
+  for (const Group& g : gs)
+    for (const Member& mb : g.sets) nout += sets[mb.i]->d;
+  // metadata: row pointers | directions | outputs (refilled in the second phase's order), then
+  // norm partials | sums
+  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t b_rows = al(rows.size() * sizeof(void*)), b_dirs = al(rows.size()), b_outs = al(nout * sizeof(ntt::Out)),
+               b_part = al(parts * 8), b_sums = al(nout * kFuMaxPrimes * 8);
+  char* blk = nullptr;
+  SK_CK(pool_malloc_async((void**)&blk, b_rows + b_dirs + b_outs + b_part + b_sums, st));
+  const int64_t** d_rows = (const int64_t**)blk;
+  uint8_t* d_dirs = (uint8_t*)(blk + b_rows);
+  ntt::Out* d_outs = (ntt::Out*)(blk + b_rows + b_dirs);
+  double* d_part = (double*)(blk + b_rows + b_dirs + b_outs);
+  unsigned long long* d_sums = (unsigned long long*)((char*)d_part + b_part);
+  uint32_t* V = nullptr;
+  std::vector<unsigned long long> sums(nout * kFuMaxPrimes);
+  auto run = [&]() -> sk_status {
+    SK_CK(cudaMemcpyAsync(d_rows, rows.data(), rows.size() * sizeof(void*), cudaMemcpyHostToDevice, st));
+    for (const Group& g : gs) {
+      k_fu_norms<<<(unsigned)(g.nvec * g.nch), 256, 0, st>>>(d_rows + g.vec0, 1, g.M, g.nch, d_part + g.part0);
+      count_launch();
+      SK_CK(cudaGetLastError());
+    }
+    std::vector<double> part(parts);
+    SK_CK(cudaMemcpyAsync(part.data(), d_part, parts * 8, cudaMemcpyDeviceToHost, st));
+    SK_CK(cudaStreamSynchronize(st));
+    // each set's primes; the second phase's vectors and outputs
+    std::vector<char> meta(b_rows + b_dirs + b_outs);
+    const int64_t** h_rows = (const int64_t**)meta.data();
+    uint8_t* h_dirs = (uint8_t*)(meta.data() + b_rows);
+    ntt::Out* h_outs = (ntt::Out*)(meta.data() + b_rows + b_dirs);
+    size_t v_words = 0, o = 0;
+    for (Group& g : gs) {
+      for (Member& mb : g.sets) {
+        const sk_set* s = sets[mb.i];
+        std::vector<double> l1((size_t)s->r * s->d, 0.0), l2((size_t)s->r * s->d, 0.0);
+        for (size_t v = 0; v < l1.size(); v++) {
+          const double* p = &part[g.part0 + 2 * (size_t)(mb.vec - g.vec0 + (int64_t)v) * g.nch];
+          for (int c = 0; c < g.nch; c++) {
+            l1[v] += p[2 * c];
+            l2[v] += p[2 * c + 1];
+          }
+          l2[v] = std::sqrt(l2[v]);
+        }
+        double bits = 0.0, cover = 0.0;
+        for (int row = 0; row < s->d; row++) bits = std::max(bits, fu_row_bits(&l1[row], &l2[row], s->r, s->d, true));
+        while (mb.np < kFuMaxPrimes && cover < bits + 3.0) cover += pr[mb.np++].log2p;
+        if (cover < bits + 3.0) mb.np = 0;
+      }
+      std::stable_sort(g.sets.begin(), g.sets.end(), [](const Member& x, const Member& y) { return x.np > y.np; });
+      g.np = g.sets[0].np;
+      g.out0 = o;
+      int64_t base = 0;
+      for (const Member& mb : g.sets) {
+        if (mb.np == 0) break;
+        const sk_set* s = sets[mb.i];
+        for (int k = 0; k < s->r; k++)
+          for (int row = 0; row < s->d; row++) {
+            h_rows[g.vec0 + base + (int64_t)k * s->d + row] = s->rel_ctr[k] + (int64_t)row * g.M;
+            h_dirs[g.vec0 + base + (int64_t)k * s->d + row] = (uint8_t)((mb.negmask >> k) & 1ull);
+          }
+        for (int row = 0; row < s->d; row++) h_outs[o++] = {base + row, s->d, s->r, mb.negmask};
+        base += (int64_t)s->r * s->d;
+        for (int i = 0; i < mb.np; i++) {
+          g.nvec_at[i] = (int)base;
+          g.nout_at[i] = (int)(o - g.out0);
+        }
+      }
+      const size_t words = (size_t)g.nvec_at[0] * g.M;
+      if (words) v_words = std::max(v_words, words * ntt_primes_at_once(words, g.np));
+    }
+    if (!v_words) return SK_OK;
+    SK_CK(cudaMemcpyAsync(blk, meta.data(), meta.size(), cudaMemcpyHostToDevice, st));
+    SK_CK(cudaMemsetAsync(d_sums, 0, b_sums, st));
+    SK_CK(pool_malloc_async((void**)&V, v_words * sizeof(uint32_t), st));
+    for (const Group& g : gs) {
+      if (!g.np) continue;
+      ntt::ColArgs ca;
+      ca.base = d_rows + g.vec0;
+      ca.per = 1;
+      ca.m = g.M;
+      ca.negmask = 0;
+      ca.dirs = d_dirs + g.vec0;
+      ca.logR = ilog2(g.M) - ntt::kLogRow;
+      ca.V = V;
+      ca.stride = g.nvec_at[0];
+      ntt::RowArgs ra;
+      ra.V = V;
+      ra.stride = ca.stride;
+      ra.logR = ca.logR;
+      ra.outs = d_outs + g.out0;
+      ra.one = {0, 0, 0, 0};
+      ra.sums = d_sums + g.out0 * kFuMaxPrimes;
+      for (int i = 0; i < kFuMaxPrimes; i++) {
+        ca.nvec[i] = g.nvec_at[i];
+        ra.nout[i] = g.nout_at[i];
+      }
+      const int at_once = ntt_primes_at_once((size_t)ca.stride * g.M, g.np);
+      for (int i = 0; i < g.np; i += at_once) {
+        ca.prime0 = ra.prime0 = i;
+        SK_CK(ntt::cols(ca, g.nvec_at[i], std::min(at_once, g.np - i), st));
+        SK_CK(ntt::rows(ra, g.nout_at[i], std::min(at_once, g.np - i), st));
+      }
+    }
+    SK_CK(cudaMemcpyAsync(sums.data(), d_sums, sums.size() * 8, cudaMemcpyDeviceToHost, st));
+    SK_CK(cudaStreamSynchronize(st));
+    return SK_OK;
+  };
+  const sk_status status = run();
+  cudaError_t ef = cudaFreeAsync(blk, st);
+  if (V) {
+    const cudaError_t ev = cudaFreeAsync(V, st);
+    if (ef == cudaSuccess) ef = ev;
+  }
+  if (status != SK_OK) return status;
+  if (ef != cudaSuccess) return set_status_from_cuda(ef);
+  for (const Group& g : gs) {
+    size_t o = g.out0;
+    for (const Member& mb : g.sets) {
+      if (mb.np == 0) break;
+      const sk_set* s = sets[mb.i];
+      std::vector<uint32_t> res((size_t)s->d * kFuMaxPrimes, 0u);
+      for (int row = 0; row < s->d; row++, o++)
+        for (int i = 0; i < mb.np; i++)
+          res[(size_t)row * kFuMaxPrimes + i] = ntt_row_residue(i, g.M, s->r, sums[o * kFuMaxPrimes + i]);
+      SK_CK_ST(fu_fill(s, res.data(), mb.np, &out[mb.i]));
+      done[mb.i] = 1;
+    }
+  }
+  return SK_OK;
+}
+
 sk_status run_estimate_many(sk_set** sets, int n, sk_estimate* out, cudaStream_t st) {
   std::vector<char> done(n, 0);
   std::vector<sk_status> status(n, SK_OK);
@@ -2998,10 +3177,16 @@ sk_status run_estimate_many(sk_set** sets, int n, sk_estimate* out, cudaStream_t
         fu_eligible(s, &nm))
       groups[m].push_back(i);
   }
+  std::map<int64_t, std::vector<int>> wide;
   for (auto& g : groups) {
+    if (g.first >= (1ll << ntt::kMinLog)) {
+      wide[g.first] = std::move(g.second);
+      continue;
+    }
     const sk_status gs = fu_group(sets, g.second, g.first, out, done, st);
     if (gs != SK_OK) return gs;
   }
+  if (!wide.empty()) SK_CK_ST(ntt_groups(sets, wide, out, done, st));
   // everything else: per-set estimates on worker streams, after the caller's queued work
   std::vector<int> rest;
   for (int i = 0; i < n; i++)
