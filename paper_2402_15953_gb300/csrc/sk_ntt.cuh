@@ -13,9 +13,11 @@
 // that all factors of a product sit in the same lane and register.  All primes of an estimate
 // run in one launch (grid y).
 //
-// Bound: integer issue.  Per element and prime about 75 instructions in the column pass and 60
-// in the row pass against 12 bytes read and 4 written; a separate residue pass, spectra written
-// back and products in their own kernel cost 4.3 passes over the residues more.
+// Bound: the integer multiplier (a modular product is two 32 x 32 -> 64-bit multiplies and one
+// 32-bit one; ncu: 64 % of the pipe in the row pass, 50 % issue).  m = 2^20 and 2^16: 3.1 ns per
+// 1024 elements and prime in the column pass, 2.3 ns in the row pass, against 1.8 and 0.6 ns for
+// their bytes at the measured copy rate.  The chain of eight at m = 2^20, d = 16 (6 primes): 4.17 ms,
+// 11.4 ms with residues, spectra and products each in their own pass over memory.
 //
 // Residues are plain (not in Montgomery form); the twiddles are in Montgomery form with
 // R = 2^32, so x (*) w is again a plain residue.  The r - 1 products of spectra each bring a
@@ -65,16 +67,37 @@ __device__ __forceinline__ uint32_t mul(uint32_t a, uint32_t b, Mod q) {
   return min(u, u - q.p);
 }
 
-// c mod p.  |c| < 2^30 < p in two instructions; any int64 through two Montgomery products
-// per half of |c| = h 2^32 + l.
+// c mod p for any int64, |c| = h 2^32 + l: two Montgomery products for l, one for h
 __device__ __forceinline__ uint32_t residue(int64_t c, Mod q, uint32_t r2) {
-  if ((uint64_t)(c + (1ll << 30)) < (1ull << 31)) {
-    const uint32_t x = (uint32_t)c;
-    return min(x, x + q.p);
-  }
   const uint64_t mag = c < 0 ? 0ull - (uint64_t)c : (uint64_t)c;
   const uint32_t v = add(mul(mul((uint32_t)mag, r2, q), 1u, q), mul((uint32_t)(mag >> 32), r2, q), q);
   return c < 0 && v ? q.p - v : v;
+}
+
+// x[i] = src[i stride] mod p for i < K, zero where i stride >= left: the loads of a batch of up
+// to 16 are in flight together, and one branch per batch decides between the short reduction
+// (every |c| < 2^30) and the general one.  With a branch per element each load waited for the
+// one before it (column pass 7.1 ns per 1024 elements).
+template <int K>
+__device__ __forceinline__ void load_residues(uint32_t (&x)[K], const int64_t* __restrict__ src, int64_t stride,
+                                              int64_t left, Mod q, uint32_t r2) {
+  constexpr int U = K < 16 ? K : 16;
+#pragma unroll
+  for (int i0 = 0; i0 < K; i0 += U) {
+    int64_t c[U];
+#pragma unroll
+    for (int i = 0; i < U; i++) c[i] = (i0 + i) * stride < left ? __ldg(src + (i0 + i) * stride) : 0;
+    uint64_t far = 0;   // bits 31 and up: some |c| >= 2^30
+#pragma unroll
+    for (int i = 0; i < U; i++) far |= (uint64_t)(c[i] + (1ll << 30));
+    if (far < (1ull << 31)) {
+#pragma unroll
+      for (int i = 0; i < U; i++) x[i0 + i] = min((uint32_t)c[i], (uint32_t)c[i] + q.p);
+    } else {
+#pragma unroll
+      for (int i = 0; i < U; i++) x[i0 + i] = residue(c[i], q, r2);
+    }
+  }
 }
 
 constexpr int rev_bits(int k, int bits) {
@@ -139,7 +162,7 @@ __device__ __forceinline__ uint32_t root_pow(int prime, int dir, int logR, uint3
 // no exchange.  64-byte column segments are read and 32-byte ones written at least, so tiles
 // wider than eight columns would not save sectors.
 template <int LA, int LB>
-__global__ void __launch_bounds__(256, (LB <= 5 ? 3 : 2)) k_ntt_cols(const __grid_constant__ ColArgs a) {
+__global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __grid_constant__ ColArgs a) {
   constexpr int A = 1 << LA, B = 1 << LB, LR = LA + LB;
   constexpr int LCB = LA ? 8 - LA : 8, CB = 1 << LCB;
   const int prime = a.prime0 + (int)blockIdx.y;
@@ -169,11 +192,8 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 3 : 2)) k_ntt_cols(const __gri
     for (int s = 0; s < B / A; s++) {
       const int b = (int)(threadIdx.x >> LCB) + A * s;
       uint32_t y[A];
-#pragma unroll
-      for (int i = 0; i < A; i++) {
-        const int64_t at = (int64_t)(B * i + b) << kLogRow;
-        y[i] = at < left ? residue(__ldg(src + at), q, r2) : 0u;
-      }
+      const int64_t at = (int64_t)b << kLogRow;
+      load_residues<A>(y, src + at, (int64_t)B << kLogRow, left - at, q, r2);
       dft<LA>(y, w64, q);
 #pragma unroll
       for (int i = 0; i < A; i++) ex[(i * (B + 1) + b) * CB + v] = i ? mul(y[i], tw[i * B + b], q) : y[i];
@@ -182,11 +202,7 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 3 : 2)) k_ntt_cols(const __gri
 #pragma unroll
     for (int b = 0; b < B; b++) x[b] = ex[(c * (B + 1) + b) * CB + v];
   } else {
-#pragma unroll
-    for (int i = 0; i < B; i++) {
-      const int64_t at = (int64_t)i << kLogRow;
-      x[i] = at < left ? residue(__ldg(src + at), q, r2) : 0u;
-    }
+    load_residues<B>(x, src, 1 << kLogRow, left, q, r2);
   }
   dft<LB>(x, w64, q);
   // x[e] is row k1 = c + A e: times w_N^(n2 k1), advanced in two chains of step w_N^(2 A n2)
@@ -227,11 +243,15 @@ struct RowArgs {
   unsigned long long* sums;   // [out][kMaxPrimes] += sum over nu of the product (residues < p)
 };
 
-// 8 warps, one row k1 each; sums of at most 2^22 residues below 2^31 fit 64 bits.
+// 8 warps, one row k1 each; sums of at most 2^22 residues below 2^31 fit 64 bits.  The running
+// products live in shared memory: with them in registers the kernel spilled at 128 registers
+// (2.40 against 2.24 ns per 1024 elements), and more warps per SM (80 registers) only spilled
+// more (2.6): the multiplier pipe, not the number of warps, sets the rate.
 __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ RowArgs a) {
   __shared__ uint32_t s_tw[2][1024];
   __shared__ uint32_t s_ex[8][32 * 33];
   __shared__ unsigned long long s_sum[8];
+  extern __shared__ uint32_t s_prod[];   // 8 x 1024
   const int prime = a.prime0 + (int)blockIdx.y;
   const int R = 1 << a.logR;
   const int lcta = a.logR > 3 ? a.logR - 3 : 0;   // log2 CTAs per output
@@ -255,7 +275,8 @@ __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ Row
         a.V + (((int64_t)blockIdx.y * a.stride + f.base) << (a.logR + kLogRow)) + ((int64_t)k1 << kLogRow) + lane;
     const int64_t rstep = f.step << (a.logR + kLogRow);
     uint32_t* ex = s_ex[warp];
-    uint32_t prod[32], x[32];
+    uint32_t* prod = s_prod + warp * 1024 + lane;   // this lane's 32 running products, stride 32
+    uint32_t x[32];
 #pragma unroll
     for (int i = 0; i < 32; i++) x[i] = __ldcs(row + 32 * i);
     for (int k = 0; k < f.r; k++) {
@@ -278,14 +299,14 @@ __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ Row
       dft<5>(y, w64, q);
       if (k == 0) {
 #pragma unroll
-        for (int i = 0; i < 32; i++) prod[i] = y[i];
+        for (int i = 0; i < 32; i++) prod[32 * i] = y[i];
       } else {
 #pragma unroll
-        for (int i = 0; i < 32; i++) prod[i] = mul(prod[i], y[i], q);
+        for (int i = 0; i < 32; i++) prod[32 * i] = mul(prod[32 * i], y[i], q);
       }
     }
 #pragma unroll
-    for (int i = 0; i < 32; i++) sum += prod[i];
+    for (int i = 0; i < 32; i++) sum += prod[32 * i];
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, s);
@@ -328,7 +349,10 @@ inline cudaError_t cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t
 
 inline cudaError_t rows(const RowArgs& a, int64_t nout, int primes, cudaStream_t st) {
   const int lcta = a.logR > 3 ? a.logR - 3 : 0;
-  k_ntt_rows<<<dim3((unsigned)(nout << lcta), (unsigned)primes), 256, 0, st>>>(a);
+  constexpr size_t smem = 8 * 1024 * sizeof(uint32_t);
+  const cudaError_t e = allow_dynamic_smem((const void*)k_ntt_rows);   // 74 KB with its static arrays
+  if (e != cudaSuccess) return e;
+  k_ntt_rows<<<dim3((unsigned)(nout << lcta), (unsigned)primes), 256, smem, st>>>(a);
   count_launch();
   return cudaGetLastError();
 }
