@@ -395,6 +395,12 @@ __device__ __forceinline__ void red_shared_if_lt(uint32_t saddr, int v, uint32_t
                ::"r"(saddr), "r"(v), "r"(x), "r"(n) : "memory");
 }
 
+// shared counter at saddr += v when x != 0
+__device__ __forceinline__ void red_shared_if_set(uint32_t saddr, int v, uint32_t x) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.shared.add.s32 [%0], %1;\n\t}"
+               ::"r"(saddr), "r"(v), "r"(x) : "memory");
+}
+
 __device__ __forceinline__ void red_shared(uint32_t saddr, int v) {
   asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
 }
@@ -610,9 +616,10 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
 }
 
 // ---------------------------------------------------------------------------
-// Partitioned update for wide sketches (unit weights, power-of-two 2^17 <= m <= 2^24, d <= 16,
-// at most 5 attributes, declared domains: the chain of eight relations at m = 2^20).  A d x m
-// int64 sketch of 128 MB does not stay in L2, and one 64-bit reduction per (tuple, row) then
+// Partitioned update for the widest sketches (unit weights, power-of-two 2^21 <= m <= 2^24,
+// d <= 16, at most 5 attributes, declared domains; 2^17 <= m <= 2^20 takes k_wide_sort below,
+// whose one-word items have no room for more bins).  A d x m int64 sketch of 128 MB does not
+// stay in L2, and one 64-bit reduction per (tuple, row) then
 // waits on DRAM.  Each row's bins are split into S = m / 2^15 parts of 2^15 bins (the int32
 // counters of one part fill 128 KB of one SM's shared memory); the items of a window are
 // sorted by part in four steps:
@@ -925,6 +932,332 @@ __global__ void __launch_bounds__(1024) k_wide_accum(WideArgs q, unsigned long l
   }
 }
 
+// ---------------------------------------------------------------------------
+// Wide partitioned update for 2^17 <= m <= 2^20 (4 to 32 parts).  The items of a chunk are
+// sorted by part inside the CTA that gathers them and stay where that CTA writes them, so
+// neither a 32-bit item plane nor a scan over all chunks nor a scatter pass is needed:
+//   1. k_wide_sort: a CTA takes kSortChunk tuples and eight rows (half a 64-byte record per
+//      gather; the CTAs of one half run together, so half of the tables fights for L2 at a
+//      time).  Every item is kept in shared memory as bin | sign | rank, the rank within its
+//      (row, part) from the returning shared-memory atomic that counts the part; after a scan
+//      over the parts the row is rewritten in place as 16-bit items in part order and leaves
+//      with 16-byte stores, its part starts in OFF[row][part][chunk];
+//   2. k_wide_list: the work list, a part with more than twice the mean's items spread over
+//      several CTAs by chunk ranges;
+//   3. k_wide_gather: a CTA owns a part of a row as 2^15 int32 counters and collects its
+//      segment of every chunk of its range.  A warp turns up to 32 segments into a list of
+//      16-byte pieces (position, mask of its items) in shared memory, so that every lane has
+//      a piece whatever the segments' lengths.
+// Per tuple and row 2 bytes are written and read once (the sorted form above: 8 written, 8
+// read), and each item passes one atomic with a returned value instead of two.  Inner chain
+// relation of 1e7 tuples, m = 2^20, d = 16: 758 us against 1063 us (table 88, k_wide_sort 420,
+// bound by the L1 data pipe at 77 %: two record gathers and 12 shared-memory wavefronts per warp
+// and row; k_wide_gather 230, waiting on the pieces it loads; 352 + 152 us before its list was
+// ordered for the SMs).
+// ---------------------------------------------------------------------------
+constexpr int kSortLog = 11;
+constexpr int kSortChunk = 1 << kSortLog;   // tuples per CTA: rank 11 bits + bin 20 + sign 1 = one word
+constexpr int kSortRows = 8;                // rows per CTA
+constexpr int kSortMaxParts = 32;
+constexpr int kPieceCap = 384;              // pieces a warp lists at a time (32 mean segments make 290)
+
+struct SortArgs {
+  uint16_t* sorted;    // [d][nchunk][kSortChunk]
+  uint16_t* off;       // [d][S + 1][nchunk] part starts within a chunk's row; [S]: its item count
+  uint32_t* total;     // [d][S] items of the window
+  uint4* plan;         // per CTA: row * S + part, first chunk, end, heavy
+  uint32_t* plan_n;
+  int64_t cnt;         // tuples in the window
+  const int64_t* col[5];
+  int nchunk;
+  int S;
+  int chunk0, group0;  // k_wide_sort: chunk and row group of the launch's first CTA
+};
+
+__global__ void k_wide_clear(uint32_t* total, int n) {
+  const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (k < n) total[k] = 0;
+}
+
+// PAIR: records are a multiple of 32 bytes, so a CTA's eight words arrive with one load.
+template <int A, bool PAIR>
+__global__ void __launch_bounds__(512, 2) k_wide_sort(UpdArgs p, TabArgs t, SortArgs q) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* item = (uint32_t*)smem_raw;   // [row][kSortChunk]
+  __shared__ uint32_t hist[kSortRows * kSortMaxParts];
+  __shared__ uint32_t valid[kSortChunk / 32];
+  const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = q.group0 + (int)blockIdx.y;
+  const int S = q.S, chunk = q.chunk0 + (int)blockIdx.x, row0 = kSortRows * group;
+  const int nr = min(kSortRows, p.d - row0);
+  for (int k = tid; k < kSortRows * kSortMaxParts; k += 512) hist[k] = 0;
+  __syncthreads();
+  const uint32_t mask = (uint32_t)p.m - 1u;
+  const int64_t c0 = (int64_t)chunk << kSortLog;
+  int64_t key[A];
+#pragma unroll
+  for (int u = 0; u < A; u++) key[u] = c0 + tid < q.cnt ? ld_key_stream(q.col[u] + c0 + tid) : -1;
+  bool mine = true;   // all of this thread's tuples are kept
+  for (int i = tid; i < kSortChunk; i += 512) {
+    bool ok = true;
+    const uint4* rec[A];
+#pragma unroll
+    for (int u = 0; u < A; u++) {
+      const bool kin = (uint64_t)key[u] < (uint64_t)p.dom[u];
+      ok = ok && kin;
+      rec[u] = (const uint4*)t.tbl + ((uint64_t)t.base[u] + (kin ? (uint64_t)key[u] : 0ull)) * (uint64_t)t.rvec +
+               2 * group;
+    }
+    if (!ok && c0 + i < q.cnt) record(p.status, SK_ERR_KEY_OUT_OF_DOMAIN);
+    const int64_t nx = c0 + i + 512;
+#pragma unroll
+    for (int u = 0; u < A; u++)
+      key[u] = (i + 512 < kSortChunk && nx < q.cnt) ? ld_key_stream(q.col[u] + nx) : -1;
+    const uint32_t vb = __ballot_sync(0xffffffffu, ok);
+    if (lane == 0) valid[i >> 5] = vb;
+    mine = mine && ok;
+    if (!ok) continue;
+    uint32_t bin[8] = {0, 0, 0, 0, 0, 0, 0, 0}, sg[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    uint32_t w[A][8];
+#pragma unroll
+    for (int u = 0; u < A; u++) {
+      if (PAIR) {
+        ld_record32(rec[u], w[u]);
+      } else {
+        const uint4 x = __ldg(rec[u]), y = nr > 4 ? __ldg(rec[u] + 1) : make_uint4(0u, 0u, 0u, 0u);
+        w[u][0] = x.x, w[u][1] = x.y, w[u][2] = x.z, w[u][3] = x.w;
+        w[u][4] = y.x, w[u][5] = y.y, w[u][6] = y.z, w[u][7] = y.w;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < A; u++)
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        bin[j] += w[u][j];   // the sign bits carry out above the bins
+        sg[j] ^= w[u][j];
+      }
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      if (j >= nr) break;
+      const uint32_t b = bin[j] & mask;
+      const uint32_t rank = atomicAdd(&hist[j * kSortMaxParts + (b >> 15)], 1u);
+      item[(j << kSortLog) + i] = b | ((sg[j] >> 31) << 20) | (rank << 21);
+    }
+  }
+  const bool full = __syncthreads_and(mine);
+  // warp j: row j's part starts
+  if (warp < nr) {
+    const uint32_t n = hist[warp * kSortMaxParts + lane];   // parts at and beyond S hold nothing
+    uint32_t x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    hist[warp * kSortMaxParts + lane] = x - n;
+    const int64_t row = row0 + warp;
+    if (lane < S) {
+      q.off[(row * (S + 1) + lane) * q.nchunk + chunk] = (uint16_t)(x - n);
+      if (lane == S - 1) q.off[(row * (S + 1) + S) * q.nchunk + chunk] = (uint16_t)x;
+      if (n) atomicAdd(q.total + row * S + lane, n);
+    }
+  }
+  __syncthreads();
+  // two warps per row: its items through registers into part order, 16 bits each
+  const int j = warp >> 1, h = warp & 1;
+  constexpr int E = kSortChunk / 64;   // items per lane
+  uint32_t x[E];
+  uint32_t* src = item + (j << kSortLog) + h * (kSortChunk / 2) + lane;
+  if (j < nr) {
+#pragma unroll
+    for (int e = 0; e < E; e++) x[e] = src[32 * e];
+  }
+  __syncthreads();
+  uint16_t* dst = (uint16_t*)(item + (j << kSortLog));
+  if (j < nr) {
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const uint32_t b = x[e] & 0xfffffu;
+      if (full || ((valid[h * E + e] >> lane) & 1u))
+        dst[hist[j * kSortMaxParts + (b >> 15)] + (x[e] >> 21)] =
+            (uint16_t)((b & 0x7fffu) | (((x[e] >> 20) & 1u) << 15));
+    }
+  }
+  __syncthreads();
+  if (j < nr) {
+    const uint4* sv = (const uint4*)(item + (j << kSortLog));
+    uint4* out = (uint4*)(q.sorted + (((int64_t)(row0 + j) * q.nchunk + chunk) << kSortLog));
+    for (int k = h * 32 + lane; k < kSortChunk / 8; k += 64) out[k] = sv[k];
+  }
+}
+
+// Work list, in the order the CTAs start (one per SM at a time): first the parts with more than
+// 5/4 of the mean's items, split into pieces of at most the mean by chunk ranges; then the others
+// whole; the last of them, which would start a wave that leaves most SMs idle, split so that the
+// wave fills.  One CTA of 512 threads, one part (of at most 16 x 32) each.
+__global__ void __launch_bounds__(512) k_wide_list(SortArgs q, int d, int sms, uint32_t maxc) {
+  __shared__ uint32_t s_warp[32];
+  const uint32_t e = threadIdx.x, ne = (uint32_t)(d * q.S);
+  const uint32_t n = e < ne ? q.total[e] : 0u;
+  uint32_t sum, nheavy, nlight;
+  block_excl_scan_1024(n, s_warp, &sum);
+  const uint32_t mean = max(1u, sum / ne);
+  const bool big = n > mean + mean / 4;
+  uint32_t k = big ? min((n + mean - 1) / mean, (uint32_t)q.nchunk) : (n ? 1u : 0u);
+  uint32_t first = block_excl_scan_1024(big ? k : 0u, s_warp, &nheavy);
+  const uint32_t li = block_excl_scan_1024(big ? 0u : k, s_warp, &nlight);
+  if (!big && k) {
+    // whole parts up to a multiple of the SMs, the rest in `cut` pieces each
+    const uint32_t rem = min(nlight, (nheavy + nlight) % (uint32_t)sms);
+    const uint32_t cut = rem ? max(1u, min(min(8u, (uint32_t)q.nchunk), (uint32_t)sms / rem)) : 1u;
+    const uint32_t whole = nlight - rem;
+    first = nheavy + (li < whole ? li : whole + (li - whole) * cut);
+    k = li < whole ? 1u : cut;
+  }
+  for (uint32_t r = 0; r < k && first + r < maxc; r++)
+    q.plan[first + r] = make_uint4(e, (uint32_t)(((uint64_t)q.nchunk * r) / k),
+                                   (uint32_t)(((uint64_t)q.nchunk * (r + 1)) / k), n > 2 * mean ? 1u : 0u);
+  uint32_t entries;
+  block_excl_scan_1024(k, s_warp, &entries);
+  if (threadIdx.x == 0) q.plan_n[0] = min(entries, maxc);
+}
+
+// 32 warps; shared memory: 2^15 int32 counters, then kPieceCap pieces per warp.  A piece is 8
+// consecutive item slots: segment << 16 | slot / 8 << 8 | mask of the slots that are the part's.
+__global__ void __launch_bounds__(1024) k_wide_gather(SortArgs q, unsigned long long* ctr, int64_t m) {
+  if (blockIdx.x >= q.plan_n[0]) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* cnt = (int*)smem_raw;
+  constexpr int L = 1 << 15;
+  const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
+  uint32_t* piece = (uint32_t*)(cnt + L) + warp * kPieceCap;
+  const uint4 wk = q.plan[blockIdx.x];
+  const int S = q.S, row = (int)(wk.x / (uint32_t)S), part = (int)(wk.x % (uint32_t)S);
+  const int ch0 = (int)wk.y, ch1 = (int)wk.z;
+  const bool heavy = wk.w != 0;   // most of its items are one bin's: runs of equal items add once
+  for (int k = threadIdx.x; k < L / 4; k += 1024) ((int4*)cnt)[k] = make_int4(0, 0, 0, 0);
+  __syncthreads();
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(cnt);
+  const uint16_t* off0 = q.off + ((int64_t)row * (S + 1) + part) * q.nchunk;
+  const uint16_t* off1 = off0 + q.nchunk;
+  // segments a warp lists at a time: all 32 warps get some
+  const int G = min(32, max(1, (ch1 - ch0 + 31) >> 5));
+  for (int g = ch0 + G * warp; g < ch1; g += G * 32) {
+    const bool in = lane < G && g + lane < ch1;
+    const uint32_t lo = in ? off0[g + lane] : 0u, hi = in ? off1[g + lane] : 0u;
+    const uint32_t kb = lo >> 3, n = hi > lo ? ((hi + 7) >> 3) - kb : 0u;
+    uint32_t x = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    const uint32_t all = __shfl_sync(0xffffffffu, x, 31);
+    const uint32_t first = x - n;
+    const uint4* base = (const uint4*)(q.sorted + (((int64_t)row * q.nchunk + g) << kSortLog));
+    for (uint32_t r0 = 0; r0 < all; r0 += kPieceCap) {
+      // this lane's pieces at list positions [r0, r0 + kPieceCap)
+      const uint32_t k0 = first < r0 ? min(r0 - first, n) : 0u;
+      const uint32_t k1 = first + n > r0 + kPieceCap ? (first < r0 + kPieceCap ? r0 + kPieceCap - first : 0u) : n;
+      for (uint32_t k = k0; k < k1; k++) {
+        const uint32_t s0 = 8u * (kb + k);
+        const uint32_t a = lo > s0 ? lo - s0 : 0u, b = min(hi - s0, 8u);
+        piece[first + k - r0] = ((uint32_t)lane << 16) | ((kb + k) << 8) | (((1u << b) - 1u) & ~((1u << a) - 1u));
+      }
+      __syncwarp();
+      const uint32_t np = min(all - r0, (uint32_t)kPieceCap);
+      uint32_t pcn = lane < np ? piece[lane] : 0u;
+      uint4 vn = make_uint4(0u, 0u, 0u, 0u);
+      if (lane < np) vn = __ldg(base + (pcn >> 16) * (kSortChunk / 8) + ((pcn >> 8) & 0xffu));
+      for (uint32_t k = lane; k < np; k += 32) {
+        const uint32_t pc = pcn;
+        const uint4 v = vn;
+        if (k + 32 < np) {   // the next piece's items, in flight during this one's additions
+          pcn = piece[k + 32];
+          vn = __ldg(base + (pcn >> 16) * (kSortChunk / 8) + ((pcn >> 8) & 0xffu));
+        }
+        const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+        if (heavy) {
+          uint32_t prev = 0xffffffffu;
+          int run = 0;
+#pragma unroll
+          for (int h = 0; h < 8; h++) {
+            const uint32_t it = (e[h >> 1] >> (16 * (h & 1))) & 0xffffu;
+            const int sv = (it >> 15) ? -1 : 1;
+            if (!((pc >> h) & 1u)) continue;
+            if (it == prev) {
+              run += sv;
+            } else {
+              if (run != 0) red_shared(sbase + ((prev & 0x7fffu) << 2), run);
+              prev = it;
+              run = sv;
+            }
+          }
+          if (run != 0) red_shared(sbase + ((prev & 0x7fffu) << 2), run);
+        } else {
+#pragma unroll
+          for (int h = 0; h < 8; h++) {
+            const uint32_t it = e[h >> 1] >> (16 * (h & 1));
+            int neg;
+            asm("bfe.s32 %0, %1, 15, 1;" : "=r"(neg) : "r"(it));
+            red_shared_if_set(sbase + ((it & 0x7fffu) << 2), neg | 1, pc & (1u << h));
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  unsigned long long* out = ctr + (int64_t)row * m + ((int64_t)part << 15);
+  for (int x = threadIdx.x; x < L; x += 1024) {
+    const int v = cnt[x];
+    if (v != 0) red_add_global(out + x, (unsigned long long)(int64_t)v);
+  }
+}
+
+struct SortLayout {
+  size_t off, total, plan, plan_n, bytes;
+};
+
+// Entries of k_wide_list's list at most: pieces of the mean's size add up to fewer than one per
+// part beyond the parts themselves, and a tail cut in c <= 8 pieces fills at most one wave more
+// than its parts (fewer than 1024 SMs).
+uint32_t sort_entries(int64_t units) { return (uint32_t)(2 * units + 1024); }
+
+SortLayout sort_layout(int d, int64_t m, int64_t W) {
+  const int64_t S = m >> 15, nchunk = (W + kSortChunk - 1) / kSortChunk;
+  auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
+  SortLayout L;
+  L.off = al((size_t)d * nchunk * kSortChunk * sizeof(uint16_t));
+  L.total = L.off + al((size_t)d * (S + 1) * nchunk * sizeof(uint16_t));
+  L.plan = L.total + al((size_t)d * S * sizeof(uint32_t));
+  L.plan_n = L.plan + al((size_t)sort_entries((int64_t)d * S) * sizeof(uint4));
+  L.bytes = L.plan_n + 256;
+  return L;
+}
+
+// k_wide_sort over the whole window in four launches: with two row groups the halves of the
+// first group, then of the second (the CTAs of a group run together either way); with one group
+// the quarters of the window.  Callers that count launches see seven per window, as for wider
+// sketches; the extra boundaries cost about 1 % of the pass.
+template <int A>
+cudaError_t launch_wide_sort(const UpdArgs& a, const TabArgs& t, SortArgs q, cudaStream_t st) {
+  constexpr size_t smem = (size_t)kSortRows * kSortChunk * sizeof(uint32_t);
+  auto kern = (t.rvec & 1) == 0 ? k_wide_sort<A, true> : k_wide_sort<A, false>;
+  cudaError_t e = allow_dynamic_smem((const void*)kern);
+  const int parts = a.d > kSortRows ? 2 : 4;
+  for (int l = 0; l < 4 && e == cudaSuccess; l++) {
+    q.group0 = l / parts;
+    q.chunk0 = (int)((int64_t)q.nchunk * (l % parts) / parts);
+    const int end = (int)((int64_t)q.nchunk * (l % parts + 1) / parts);
+    if (end <= q.chunk0) continue;
+    kern<<<(unsigned)(end - q.chunk0), 512, smem, st>>>(a, t, q);
+    count_launch();
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
 // Window capacity of the wide partitioned update: positions in `sorted` stay below 2^28.
 int64_t wide_window(int64_t n) {
   const char* v = std::getenv("SK_PART_WINDOW");
@@ -1006,6 +1339,46 @@ cudaError_t run_wide_partitioned(const UpdArgs& a, const TabArgs& t, void* stagi
     k_wide_plan<<<1, 1024, 0, st>>>(q, a.d, B, maxc);
     k_wide_accum<<<maxc, 1024, smem, st>>>(q, a.ctr, (int64_t)a.m);
     count_launch(7);
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+// The same for 2^17 <= m <= 2^20; staging: sort_layout(...).bytes for the window.
+cudaError_t run_wide_sorted(const UpdArgs& a, const TabArgs& t, void* staging, int sms, cudaStream_t st) {
+  const int64_t n = a.n, W = wide_window(n);
+  const SortLayout Ly = sort_layout(a.d, (int64_t)a.m, W);
+  char* base = (char*)staging;
+  SortArgs q;
+  q.sorted = (uint16_t*)base;
+  q.off = (uint16_t*)(base + Ly.off);
+  q.total = (uint32_t*)(base + Ly.total);
+  q.plan = (uint4*)(base + Ly.plan);
+  q.plan_n = (uint32_t*)(base + Ly.plan_n);
+  q.S = (int)(a.m >> 15);
+  constexpr size_t smem = ((size_t)4 << 15) + (size_t)32 * kPieceCap * sizeof(uint32_t);
+  cudaError_t e = allow_dynamic_smem((const void*)k_wide_gather);
+  const int64_t units = (int64_t)q.S * a.d;
+  for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += W) {
+    q.cnt = std::min(W, n - i0);
+    for (int u = 0; u < 5; u++) q.col[u] = u < a.a ? a.cols + (int64_t)u * a.stride + i0 : nullptr;
+    q.nchunk = (int)((q.cnt + kSortChunk - 1) / kSortChunk);
+    k_wide_clear<<<(unsigned)((units + 255) / 256), 256, 0, st>>>(q.total, (int)units);
+    count_launch();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) break;
+    switch (a.a) {
+      case 1: e = launch_wide_sort<1>(a, t, q, st); break;
+      case 2: e = launch_wide_sort<2>(a, t, q, st); break;
+      case 3: e = launch_wide_sort<3>(a, t, q, st); break;
+      case 4: e = launch_wide_sort<4>(a, t, q, st); break;
+      default: e = launch_wide_sort<5>(a, t, q, st); break;
+    }
+    if (e != cudaSuccess) break;
+    const uint32_t maxc = sort_entries(units);
+    k_wide_list<<<1, 512, 0, st>>>(q, a.d, sms, maxc);
+    k_wide_gather<<<maxc, 1024, smem, st>>>(q, a.ctr, (int64_t)a.m);
+    count_launch(2);
     e = cudaGetLastError();
   }
   return e;
@@ -1431,6 +1804,7 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     // wide partitioned update takes the batch: it replaces those atomics.
     const bool worth = ktm == 1 || (n >= ((int64_t)1 << 16) && total * 4 <= n * (int64_t)rp.a &&
                                     (sketch_bytes <= ((size_t)32 << 20) || wide));
+    const bool sorted_parts = s->m <= ((int64_t)kSortMaxParts << 15);
     void* staging = nullptr;
     if (fits && worth && total > 0 && part) {
       e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n), sms), st);
@@ -1440,7 +1814,10 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
         part = false;
       }
     } else if (fits && worth && total > 0 && wide) {
-      e = pool_malloc_async(&staging, wide_layout(s->d, s->m, wide_window(n)).total, st);
+      e = pool_malloc_async(&staging,
+                            sorted_parts ? sort_layout(s->d, s->m, wide_window(n)).bytes
+                                         : wide_layout(s->d, s->m, wide_window(n)).total,
+                            st);
       if (e != cudaSuccess) {
         cudaGetLastError();   // no room for the planes: per-tuple update
         staging = nullptr;
@@ -1476,7 +1853,7 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
         if (e == cudaSuccess && part) {
           e = run_partitioned(a, t, part_fmt, staging, sms, st);
         } else if (e == cudaSuccess && wide) {
-          e = run_wide_partitioned(a, t, staging, sms, st);
+          e = sorted_parts ? run_wide_sorted(a, t, staging, sms, st) : run_wide_partitioned(a, t, staging, sms, st);
         } else if (e == cudaSuccess) {
           if (use_smem) {
             const int per_sm = sub_bytes <= 48 * 1024 ? 4 : (sub_bytes <= 100 * 1024 ? 2 : 1);
