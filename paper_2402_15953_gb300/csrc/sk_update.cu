@@ -17,7 +17,9 @@
 //     L2 when d * m * 8 bytes is small against the 126 MiB L2).
 // Counters wrap like two's-complement int64 (additions are done on uint64).
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
+#include <type_traits>
 
 #include "sk_hash.cuh"
 #include "sk_internal.h"
@@ -101,8 +103,7 @@ __global__ void __launch_bounds__(256, (A > 0 && V8 && NARROW && POW2) ? 5 : 1) 
 }
 
 // ---------------------------------------------------------------------------
-// Partitioned update through the key tables (unit weights, power-of-two 1024 <= m <= 2^16,
-// d <= 14, at most 5 attributes: the star fact table).  k_update_tab adds each (tuple, row)
+// Partitioned update through the key tables (power-of-two 1024 <= m <= 2^16, d <= 14, at most 5 attributes: the star fact table).  k_update_tab adds each (tuple, row)
 // to the L2-resident int64 sketch with one 64-bit reduction, and the L2 lookup rate bounds it
 // (9 reductions per tuple at d = 9, about half of them forwarded between the two dies' L2
 // halves).  Shared-memory atomics run about ten times faster than L2 reductions on GB300,
@@ -125,6 +126,8 @@ __global__ void __launch_bounds__(256, (A > 0 && V8 && NARROW && POW2) ? 5 : 1) 
 //      into the int64 sketch with one 64-bit reduction.
 // Every counter receives the same sum as in k_update_tab (integer addition in any order);
 // a CTA's int32 counter holds at most its range's tuple count in magnitude, kept below 2^31.
+// Weighted batches take 32-bit items that carry Delta (2e7 turnstile tuples of five shuffled
+// columns, m = 2^16, d = 9: 0.93 ms; 1.24 ms through k_update_tab).
 //
 // Records for this path (32 bytes, built by k_key_table_l20 for d <= 9): row r's bin in bits
 // 20 (r mod 3) .. 20 (r mod 3) + 15 of 64-bit word r / 3 (words 0..2), the d sign bits in
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(256, (A > 0 && V8 && NARROW && POW2) ? 5 : 1) 
 constexpr int kPartMaxCtasPerSm = 8;   // phase-1 CTAs of 256 threads per SM, at most
 
 struct PartArgs {
-  uint16_t* items;               // phase-1 warp w, row j: region items + (w d + j) C
+  void* items;                   // phase-1 warp w, row j: region items + (w d + j) C, uint16_t each
   uint32_t* cnts;                // phase-1 warp w: [16 w + j] part-0 items of row j, [16 w + 15] valid tuples
   const int64_t* col[5];         // column u of the window's first tuple
   int64_t W;                     // window capacity, a multiple of 256
@@ -144,6 +147,8 @@ struct PartArgs {
   int nwarps;                    // warps of the phase-1 grid
   int logL;                      // part width 2^L
   const uint32_t* vbits;         // nullptr, or bit (i mod 32) of word i / 32: window tuple i is kept
+  const int64_t* wts;            // weighted: Delta of the window's first tuple (items are uint32_t)
+  int64_t wmax;                  // weighted: |Delta| <= wmax < 2^16 goes into an item
 };
 
 __device__ __forceinline__ uint64_t policy_evict_first() {
@@ -153,7 +158,11 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 }
 
 __device__ __forceinline__ void st_u16_hint(uint16_t* ptr, uint16_t v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(ptr), "h"(v), "l"(pol) : "memory");
+  asm volatile("st.global.L1::no_allocate.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(ptr), "h"(v), "l"(pol) : "memory");
+}
+
+__device__ __forceinline__ void st_u32_hint(uint32_t* ptr, uint32_t v, uint64_t pol) {
+  asm volatile("st.global.L1::no_allocate.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(ptr), "r"(v), "l"(pol) : "memory");
 }
 
 __device__ __forceinline__ int64_t ld_key_policy(const int64_t* ptr, uint64_t pol) {
@@ -257,25 +266,44 @@ __device__ __forceinline__ void ld_record24(const uint64_t* tbl, uint64_t k, uin
 // running counts five (48 registers) spilled and took the star's F update from 3.10 to 3.84 ms;
 // six for the instances of one or two attributes (40 registers, no spills) took a sub-query
 // family's update from 8.45 to 9.22 ms.
-template <int A, int FMT>
+//
+// A row costs one ballot, two population counts, a shuffle of its next slot and about 18
+// instructions.  What bounds F of the star (5 attributes; 480 us per 2e7 tuples) is the gathers:
+// alone, with nothing done to the records, they take 375 us (173 when every record hits L1; 32-byte
+// records 362 and 205, 16-byte ones 231), through the texture path 446.  So the registers go to
+// loads in flight: with every row's slot held in registers instead of shuffled the compiler
+// splits the gathers and the star step takes 3.70 ms instead of 3.45.  The weighted kernel holds
+// them all the same (HELD: 2e7 tuples 0.96 against 1.01 ms).  Item stores skip L1, which the
+// records need.
+//
+// WT (weighted batches): items are 32 bits, the bin's offset in bits 0..14 and Delta times the
+// sign above; a tuple with |Delta| > wmax goes to the int64 counters directly.
+template <int A, int FMT, bool WT>
 __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, PartArgs q) {
+  using Item = typename std::conditional<WT, uint32_t, uint16_t>::type;
+  constexpr bool HELD = WT && FMT != 1;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
   const uint32_t mask = (uint32_t)p.m - 1u;
   const uint32_t low = (1u << q.logL) - 1u;
+  const uint32_t half = mask & ~low;   // the bin bit that tells part 1 (0: one part)
   const unsigned lane = threadIdx.x & 31u;
   const uint32_t lt = (1u << lane) - 1u;
   const int d = p.d;
   const uint64_t pol = policy_evict_first();
   const uint4* tbl = (const uint4*)t.tbl;
   int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t rb = (uint32_t)(g >> 5) * (uint32_t)d;     // this warp's row-0 region index
   const uint32_t C = (uint32_t)q.C;
-  // counts so far: lane j < d holds row j's part-0 items, lane 15 the valid tuples
-  uint32_t cw = 0;
+  Item* const mine = (Item*)q.items + (g >> 5) * d * q.C;   // this warp's regions, row j's at j C
+  uint32_t nval = 0;    // valid tuples so far
+  uint32_t cw = lane * C;   // lane j < d: row j's next part-0 slot, j C + its part-0 items
+  uint32_t o0[9];           // HELD: the same for every row
+#pragma unroll
+  for (int j = 0; j < 9; j++) o0[j] = (uint32_t)j * C;
   // keys of the thread's next tuple, checked against their domains as they arrive: the
   // in-domain keys (< 2^31) as 32-bit values, bit u of okm set when key u is in its domain
   uint32_t kx[A], okm = 0;
+  int64_t wn = 0;
 #pragma unroll
   for (int u = 0; u < A; u++) {
     const int64_t k = g < q.cnt ? ld_key_policy(q.col[u] + g, pol) : -1;
@@ -283,13 +311,16 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
     okm |= (uint32_t)kin << u;
     kx[u] = kin ? (uint32_t)k : 0u;
   }
+  if (WT && g < q.cnt) wn = ld_key_policy(q.wts + g, pol);
   for (; g < gend; g += step) {
     const bool in = g < q.cnt;
-    const bool ok = in && okm == (1u << A) - 1u && (!q.vbits || ((q.vbits[g >> 5] >> lane) & 1u));
+    const bool whole = in && okm == (1u << A) - 1u && (!q.vbits || ((q.vbits[g >> 5] >> lane) & 1u));
+    const int64_t delta = wn;
+    const bool ok = whole && (!WT || (delta <= q.wmax && delta >= -q.wmax));
     uint32_t kg[A];   // global record indices (the host keeps this path's tables below 2^32 records)
 #pragma unroll
     for (int u = 0; u < A; u++) kg[u] = (uint32_t)t.base[u] + kx[u];
-    if (in && !ok) record(p.status, SK_ERR_KEY_OUT_OF_DOMAIN);   // left out of the tile below
+    if (in && !whole) record(p.status, SK_ERR_KEY_OUT_OF_DOMAIN);   // left out of the tile below
     const int64_t gn = g + step;
     okm = 0;
 #pragma unroll
@@ -299,70 +330,87 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
       okm |= (uint32_t)kin << u;
       kx[u] = kin ? (uint32_t)k : 0u;
     }
+    if (WT && gn < q.cnt) wn = ld_key_policy(q.wts + gn, pol);
     const uint32_t vb = __ballot_sync(0xffffffffu, ok);
     const uint32_t nv = __popc(vb), rv = __popc(vb & lt);   // valid tuples in the tile / before this lane
-    const uint32_t nval = __shfl_sync(0xffffffffu, cw, 15);  // valid tuples before the tile
-    uint32_t add = nv;   // this tile's part-0 items of row `lane` (lane < d), its valid tuples (lane 15)
-    // one row: with r1 the part-1 tuples before this lane, a part-0 tuple goes to slot
-    // (part-0 items so far) + rv - r1 and a part-1 one to C - 1 - (part-1 items so far) - r1
-    auto put = [&](int j, uint32_t bin, uint32_t neg) {
-      const bool hi = (bin >> q.logL) != 0;
-      const uint32_t hb = __ballot_sync(0xffffffffu, ok && hi);
-      const uint32_t n1 = __popc(hb), r1 = __popc(hb & lt);
-      const uint32_t c0 = __shfl_sync(0xffffffffu, cw, j);
-      const uint32_t pos = hi ? C - 1u - (nval - c0) - r1 : c0 + rv - r1;
-      // slot (rb + j) C + pos, formed here rather than kept as d row pointers across the
-      // loop (registers)
-      uint64_t slot;
-      asm volatile("{\n\t.reg .u32 r;\n\tadd.u32 r, %1, %2;\n\tmad.wide.u32 %0, r, %3, %4;\n\t}"
-                   : "=l"(slot) : "r"(rb), "r"((uint32_t)j), "r"(C), "l"((uint64_t)pos));
-      if (ok) st_u16_hint(q.items + slot, (uint16_t)((bin & low) | (neg << 15)), pol);
-      if (lane == (unsigned)j) add = nv - n1;
+    const uint32_t end1 = C - 1u - nval;   // a row's next part-1 slot is end1 past its next part-0 slot
+    uint32_t add = 0;   // this tile's part-0 items of row `lane`
+    // one row, x = its bin sum (bits above the bin arbitrary, 0 for a tuple left out): with r1
+    // the part-1 tuples before this lane, a part-0 tuple goes to slot (part-0 items so far) +
+    // rv - r1 and a part-1 one to C - 1 - (part-1 items so far) - r1
+    auto put = [&](int j, uint32_t x, uint32_t neg15) {
+      const bool hi = (x & half) != 0u;
+      const uint32_t hb = __ballot_sync(0xffffffffu, hi);
+      const uint32_t r1 = __popc(hb & lt);
+      const uint32_t at = (HELD ? o0[j] : __shfl_sync(0xffffffffu, cw, j)) + (hi ? end1 : rv) - r1;
+      if (WT) {
+        const int32_t v = neg15 ? -(int32_t)delta : (int32_t)delta;
+        if (ok) st_u32_hint((uint32_t*)mine + at, (x & low) | ((uint32_t)v << 15), pol);
+      } else if (ok) {
+        st_u16_hint((uint16_t*)mine + at, (uint16_t)((x & low) | neg15), pol);
+      }
+      if (HELD) o0[j] += nv - __popc(hb);
+      else if (lane == (unsigned)j) add = nv - __popc(hb);
+    };
+    // a weighted tuple beyond wmax: straight to the counters
+    auto far = [&](int j, uint32_t x, uint32_t neg15) {
+      red_add_global(p.ctr + (int64_t)j * p.m + (x & mask), (unsigned long long)(neg15 ? -delta : delta));
     };
     uint32_t sg = 0;
     if (FMT == 0) {
-      uint64_t acc0 = 0, acc1 = 0, acc2 = 0;
-      if (ok) {
+      uint64_t acc[3] = {0, 0, 0};
+      if (whole) {
 #pragma unroll
         for (int u = 0; u < A; u++) {
           uint32_t w[8];
           ld_record32(tbl + (uint64_t)kg[u] * 2, w);
-          acc0 += ((uint64_t)w[1] << 32) | w[0];
-          acc1 += ((uint64_t)w[3] << 32) | w[2];
-          acc2 += ((uint64_t)w[5] << 32) | w[4];
+          acc[0] += ((uint64_t)w[1] << 32) | w[0];
+          acc[1] += ((uint64_t)w[3] << 32) | w[2];
+          acc[2] += ((uint64_t)w[5] << 32) | w[4];
           sg ^= w[7];
         }
+      }
+      if (WT && whole && !ok) {
+        for (int j = 0; j < d; j++) far(j, (uint32_t)(acc[j / 3] >> (20 * (j % 3))), ((sg >> j) & 1u) << 15);
+        acc[0] = acc[1] = acc[2] = 0;
       }
 #pragma unroll
       for (int j = 0; j < 9; j++) {
         if (j >= d) break;
-        const uint64_t acc = j < 3 ? acc0 : (j < 6 ? acc1 : acc2);
-        put(j, (uint32_t)(acc >> (20 * (j % 3))) & mask, (sg >> j) & 1u);
+        put(j, (uint32_t)(acc[j / 3] >> (20 * (j % 3))), ((sg >> j) & 1u) << 15);
       }
     } else if (FMT == 2) {
-      uint64_t acc0 = 0, acc1 = 0, acc2 = 0;
-      if (ok) {
+      uint64_t acc[3] = {0, 0, 0};
+      if (whole) {
 #pragma unroll
         for (int u = 0; u < A; u++) {
           uint64_t w0, w1, w2;
           ld_record24((const uint64_t*)t.tbl, kg[u], w0, w1, w2);
-          acc0 += w0;
-          acc1 += w1;
-          acc2 += w2;
+          acc[0] += w0;
+          acc[1] += w1;
+          acc[2] += w2;
         }
+      }
+      if (WT && whole && !ok) {
+#pragma unroll
+        for (int j = 0; j < 9; j++) {
+          if (j >= d) break;
+          const uint32_t x = (uint32_t)(acc[j / 3] >> (22 * (j % 3)));
+          far(j, x, (x >> 4) & 0x8000u);
+        }
+        acc[0] = acc[1] = acc[2] = 0;
       }
 #pragma unroll
       for (int j = 0; j < 9; j++) {
         if (j >= d) break;
-        const uint64_t acc = j < 3 ? acc0 : (j < 6 ? acc1 : acc2);
-        const int sh = 22 * (j % 3);
-        put(j, (uint32_t)(acc >> sh) & mask, (uint32_t)(acc >> (sh + 19)) & 1u);
+        const uint32_t x = (uint32_t)(acc[j / 3] >> (22 * (j % 3)));
+        put(j, x, (x >> 4) & 0x8000u);   // the sign is lane bit 19
       }
     } else {
       uint32_t lo[7], all[7];
 #pragma unroll
       for (int j = 0; j < 7; j++) lo[j] = all[j] = 0;
-      if (ok) {
+      if (whole) {
 #pragma unroll
         for (int u = 0; u < A; u++) {
           uint32_t w[8];
@@ -378,15 +426,26 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
 #pragma unroll
       for (int j = 0; j < 14; j++) {
         if (j >= d) break;
-        const uint32_t sum = (j & 1) ? (all[j >> 1] - lo[j >> 1]) >> 16 : lo[j >> 1];
-        put(j, sum & mask, (sg >> j) & 1u);
+        uint32_t x = (j & 1) ? (all[j >> 1] - lo[j >> 1]) >> 16 : lo[j >> 1];
+        const uint32_t neg15 = ((sg >> j) & 1u) << 15;
+        if (WT && !ok) {
+          if (whole) far(j, x, neg15);
+          x = 0;
+        }
+        put(j, x, neg15);
       }
     }
-    cw += add;   // after the rows: their shuffles all read the counts before the tile
+    cw += add;   // after the rows: their shuffles all read the slots before the tile
+    nval += nv;
   }
   // the warp's counts: lane j < d row j's part-0 items, lane 15 the valid tuples
   const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (lane < (unsigned)d || lane == 15u) q.cnts[wg * 16 + lane] = cw;
+  if (HELD) {
+#pragma unroll
+    for (int j = 0; j < 9; j++)
+      if (lane == (unsigned)j) cw = o0[j];
+  }
+  if (lane < (unsigned)d || lane == 15u) q.cnts[wg * 16 + lane] = lane == 15u ? nval : cw - lane * C;
 }
 
 // shared counter at saddr += v when x < n (unsigned): one compare, one predicated reduction
@@ -430,12 +489,22 @@ __device__ __forceinline__ void add_chunk(uint32_t sbase, uint4 v, uint32_t b, u
   }
 }
 
+// The same for the 4 items of a weighted chunk (bin offset in bits 0..14, signed value above).
+__device__ __forceinline__ void add_chunk_weighted(uint32_t sbase, uint4 v, uint32_t b, uint32_t n) {
+  const uint32_t e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int k = 0; k < 4; k++)
+    red_shared_if_lt(sbase + ((e[k] & 0x7fffu) << 2), (int)e[k] >> 15, b + (uint32_t)k, n);
+}
+
 // blockIdx.x = h + S (row + d c), S = m >> logL: part h of row `row` over the regions of the
 // phase-1 warps [c R, min(c R + R, nwarps)), each region's part-h chunks (8 items, one 16-byte
 // load) split into 2^logP pieces.  Warp k of the CTA takes pieces k, k + 32, ...; lane l of a
 // warp takes the piece's chunks l, l + 32, ..., two per iteration, loads first.
+template <bool WT>
 __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long long* ctr, int64_t m, int d,
                                                      int logL, int R, int logP) {
+  constexpr int LI = WT ? 2 : 3, I = 1 << LI;   // items per 16-byte chunk
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int* cnt = (int*)smem_raw;
   const int S = (int)(m >> logL);
@@ -452,25 +521,32 @@ __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long l
   const int w1 = min(w0 + R, q.nwarps);
   const int npc = (w1 - w0) << logP;
   const uint32_t C = (uint32_t)q.C;
-  // slots b .. b + 7 counted from the part's first item: add the signs of those below n
-  auto unit = [&](uint4 v, uint32_t b, uint32_t n) { add_chunk(sbase, v, b, n); };
+  // slots b .. b + I - 1 counted from the part's first item: add those below n
+  auto unit = [&](uint4 v, uint32_t b, uint32_t n) {
+    if (WT) add_chunk_weighted(sbase, v, b, n);
+    else add_chunk(sbase, v, b, n);
+  };
   for (int pc = (int)(threadIdx.x >> 5); pc < npc; pc += (int)(blockDim.x >> 5)) {
     const int w = w0 + (pc >> logP);
     const uint32_t piece = (uint32_t)pc & ((1u << logP) - 1u);
     const uint32_t n0 = q.cnts[(int64_t)w * 16 + row], nv = q.cnts[(int64_t)w * 16 + 15];
     const uint32_t n = h ? nv - n0 : n0;         // part h's items in this region
     const uint32_t lo = h ? C - n : 0u;          // and the first of them
-    const uint32_t kb = lo >> 3, nk = ((lo + n + 7) >> 3) - kb;
+    const uint32_t kb = lo >> LI, nk = ((lo + n + I - 1) >> LI) - kb;
     const uint32_t ke = kb + (uint32_t)(((uint64_t)nk * (piece + 1)) >> logP);
     uint32_t k = kb + (uint32_t)(((uint64_t)nk * piece) >> logP) + lane;
-    const uint16_t* rg = q.items + ((int64_t)w * d + row) * q.C;
+    const uint4* rg = (const uint4*)q.items + (((int64_t)w * d + row) * q.C >> LI);
+    // two chunks per iteration, the next two in flight during their additions
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    uint4 v1 = k < ke ? rg[k] : none, v2 = k + 32 < ke ? rg[k + 32] : none;
     for (; k + 32 < ke; k += 64) {
-      const uint4 v1 = *(const uint4*)(rg + 8 * k);
-      const uint4 v2 = *(const uint4*)(rg + 8 * (k + 32));
-      unit(v1, 8 * k - lo, n);
-      unit(v2, 8 * (k + 32) - lo, n);
+      const uint4 c1 = v1, c2 = v2;
+      if (k + 64 < ke) v1 = rg[k + 64];
+      if (k + 96 < ke) v2 = rg[k + 96];
+      unit(c1, I * k - lo, n);
+      unit(c2, I * (k + 32) - lo, n);
     }
-    if (k < ke) unit(*(const uint4*)(rg + 8 * k), 8 * k - lo, n);
+    if (k < ke) unit(v1, I * k - lo, n);
   }
   __syncthreads();
   unsigned long long* out = ctr + (int64_t)row * m + ((int64_t)h << logL);
@@ -480,39 +556,165 @@ __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long l
   }
 }
 
-// CTAs of k_tab_items<A, FMT> per SM (no shared memory: the whole unified array is left to
-// L1, which caches the hot records).
-template <int A, int FMT>
-cudaError_t tab_items_per_sm(int* per_sm) {
-  auto kern = k_tab_items<A, FMT>;
+// Phase 1 for all views of a sub-query family's relation at once (24-byte records, unit weights):
+// the tuple's A records are gathered once and every view sums the records of its attributes, so
+// nv views cost one gather per attribute instead of one per (view, attribute).  A tuple with any
+// key outside its domain is left out of every view.
+// Regions are one CTA's here, [view][CTA][row][C]: 15 views of nine rows and two parts are 270
+// streams, and one set per warp left a million half-written lines, as much as L2 holds (4.3 ms
+// per 1e7 tuples, 5 GB read back and 5 GB written for 2.7 GB of items).  The CTA's warps take their
+// places from shared-memory counters, part-0 and part-1 items in the halves of one 64-bit word,
+// with one returning atomic per tile and view (lane j: row j).
+// 15 views of a 4-attribute relation, 1e7 tuples: 2.3 ms, 54 % issue (one view at a time: 2.7 ms).
+struct ViewMasks {
+  int nv;
+  uint8_t mask[SK_MAX_VIEWS];   // bit u: the view joins attribute u
+};
+
+template <int A, bool ALL9>
+__global__ void __launch_bounds__(256, 3) k_tab_items_views(UpdArgs p, TabArgs t, PartArgs q,
+                                                            const __grid_constant__ ViewMasks vm) {
+  __shared__ unsigned long long taken[SK_MAX_VIEWS * 9];   // items of row j of view v: part 0 | part 1 << 32
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
+  const uint32_t mask = (uint32_t)p.m - 1u;
+  const uint32_t low = (1u << q.logL) - 1u;
+  const uint32_t half = mask & ~low;
+  const unsigned lane = threadIdx.x & 31u;
+  const uint32_t lt = (1u << lane) - 1u;
+  const int d = ALL9 ? 9 : p.d, nv = vm.nv;
+  const uint64_t pol = policy_evict_first();
+  int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t C = (uint32_t)q.C;
+  const int64_t vstride = (int64_t)q.nwarps * d * q.C;
+  uint16_t* const mine = (uint16_t*)q.items + (int64_t)blockIdx.x * d * q.C;
+  for (int k = threadIdx.x; k < nv * 9; k += 256) taken[k] = 0ull;
+  __syncthreads();
+  uint32_t kx[A], okm = 0;
+#pragma unroll
+  for (int u = 0; u < A; u++) {
+    const int64_t k = g < q.cnt ? ld_key_policy(q.col[u] + g, pol) : -1;
+    const bool kin = (uint64_t)k < (uint64_t)p.dom[u];
+    okm |= (uint32_t)kin << u;
+    kx[u] = kin ? (uint32_t)k : 0u;
+  }
+  for (; g < gend; g += step) {
+    const bool in = g < q.cnt;
+    const bool ok = in && okm == (1u << A) - 1u;
+    if (in && !ok) record(p.status, SK_ERR_KEY_OUT_OF_DOMAIN);
+    uint64_t rec[A][3];
+#pragma unroll
+    for (int u = 0; u < A; u++) {
+      rec[u][0] = rec[u][1] = rec[u][2] = 0;
+      if (ok) ld_record24((const uint64_t*)t.tbl, (uint32_t)t.base[u] + kx[u], rec[u][0], rec[u][1], rec[u][2]);
+    }
+    const int64_t gn = g + step;
+    okm = 0;
+#pragma unroll
+    for (int u = 0; u < A; u++) {
+      const int64_t k = gn < q.cnt ? ld_key_policy(q.col[u] + gn, pol) : -1;
+      const bool kin = (uint64_t)k < (uint64_t)p.dom[u];
+      okm |= (uint32_t)kin << u;
+      kx[u] = kin ? (uint32_t)k : 0u;
+    }
+    const uint32_t vb = __ballot_sync(0xffffffffu, ok);
+    const uint32_t nt = __popc(vb), rv = __popc(vb & lt);
+    uint16_t* out = mine;
+    for (int v = 0; v < nv; v++, out += vstride) {
+      const uint32_t am = vm.mask[v];
+      uint64_t acc[3] = {0, 0, 0};
+#pragma unroll
+      for (int u = 0; u < A; u++)
+        if ((am >> u) & 1u) {
+          acc[0] += rec[u][0];
+          acc[1] += rec[u][1];
+          acc[2] += rec[u][2];
+        }
+      uint32_t hb[9], n1 = 0;   // each row's part-1 tuples; lane j: how many in row j
+#pragma unroll
+      for (int j = 0; j < 9; j++) {
+        if (!ALL9 && j >= d) break;
+        hb[j] = __ballot_sync(0xffffffffu, ((uint32_t)(acc[j / 3] >> (22 * (j % 3))) & half) != 0u);
+        if (lane == (unsigned)j) n1 = hb[j];
+      }
+      n1 = __popc(n1);
+      unsigned long long at0 = 0;
+      if (lane < (unsigned)d) {
+        at0 = atomicAdd(&taken[v * 9 + lane], (unsigned long long)(nt - n1) | ((unsigned long long)n1 << 32));
+        // this row's first free part-0 slot, last free part-1 slot, in the CTA's regions of the view
+        at0 = (unsigned long long)(lane * C + (uint32_t)at0) |
+              ((unsigned long long)(lane * C + C - 1u - (uint32_t)(at0 >> 32)) << 32);
+      }
+#pragma unroll
+      for (int j = 0; j < 9; j++) {
+        if (!ALL9 && j >= d) break;
+        const uint32_t x = (uint32_t)(acc[j / 3] >> (22 * (j % 3)));
+        const uint32_t b0 = __shfl_sync(0xffffffffu, (uint32_t)at0, j);
+        const uint32_t b1 = __shfl_sync(0xffffffffu, (uint32_t)(at0 >> 32), j);
+        const uint32_t r1 = __popc(hb[j] & lt);
+        const uint32_t at = (x & half) ? b1 - r1 : b0 + rv - r1;
+        if (ok) st_u16_hint(out + at, (uint16_t)((x & low) | ((x >> 4) & 0x8000u)), pol);
+      }
+    }
+  }
+  __syncthreads();
+  // the CTA's counts: word j < d row j's part-0 items, word 15 the valid tuples (any row's items)
+  for (int k = threadIdx.x; k < nv * 16; k += 256) {
+    const int v = k >> 4, j = k & 15;
+    if (j < d || j == 15) {
+      const unsigned long long n = taken[v * 9 + (j < d ? j : 0)];
+      q.cnts[((int64_t)v * q.nwarps + blockIdx.x) * 16 + j] = j < d ? (uint32_t)n : (uint32_t)n + (uint32_t)(n >> 32);
+    }
+  }
+}
+
+using TabItemsKernel = void (*)(UpdArgs, TabArgs, PartArgs);
+
+template <int FMT, bool WT>
+TabItemsKernel tab_items_of(int A) {
+  switch (A) {
+    case 1: return k_tab_items<1, FMT, WT>;
+    case 2: return k_tab_items<2, FMT, WT>;
+    case 3: return k_tab_items<3, FMT, WT>;
+    case 4: return k_tab_items<4, FMT, WT>;
+    default: return k_tab_items<5, FMT, WT>;
+  }
+}
+
+TabItemsKernel tab_items_kernel(int A, int fmt, bool weighted) {
+  if (weighted) return fmt == 0 ? tab_items_of<0, true>(A) : (fmt == 2 ? tab_items_of<2, true>(A) : tab_items_of<1, true>(A));
+  return fmt == 0 ? tab_items_of<0, false>(A) : (fmt == 2 ? tab_items_of<2, false>(A) : tab_items_of<1, false>(A));
+}
+
+// CTAs of a phase-1 kernel per SM (no shared memory: the whole unified array is left to L1,
+// which caches the hot records).
+cudaError_t tab_items_per_sm(TabItemsKernel kern, int* per_sm) {
   cudaError_t e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, 256, 0);
   *per_sm = std::max(1, std::min(*per_sm, kPartMaxCtasPerSm));
   return e;
 }
 
-template <int FMT>
-cudaError_t tab_items_occupancy(int A, int* per_sm) {
-  switch (A) {
-    case 1: return tab_items_per_sm<1, FMT>(per_sm);
-    case 2: return tab_items_per_sm<2, FMT>(per_sm);
-    case 3: return tab_items_per_sm<3, FMT>(per_sm);
-    case 4: return tab_items_per_sm<4, FMT>(per_sm);
-    default: return tab_items_per_sm<5, FMT>(per_sm);
+// Phase-2 split of nwarps regions (`units` (row, part) pairs, `slots` resident CTAs): the number
+// of ranges of regions per pair.  A wave of CTAs costs its share of the items plus a fixed
+// zeroing and flush of 2^15 counters (about 9 us on a GB300 SM, as long as 125 000 items take),
+// so few waves.
+int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps) {
+  double best = 0.0;
+  int64_t nr = 1;
+  // The star's 18 pairs take one wave of 144 CTAs (star step 3.41 ms, with at least two waves 3.43;
+  // 2e7 weighted tuples 0.931 and 0.944 ms); nine waves of 1368 CTAs flushed 45e6 counters (phase
+  // 2 162 us per 2e7 tuples, now about 110).
+  for (int64_t k = 1; k <= 16; k++) {
+    const int64_t r = std::max<int64_t>(1, k * slots / units);
+    const double waves = std::ceil((double)(r * units) / (double)slots);
+    const double cost = waves * ((double)items / (double)(r * units) + 125000.0);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      nr = r;
+    }
   }
-}
-
-template <int FMT>
-cudaError_t dispatch_tab_items(const UpdArgs& a, const TabArgs& t, const PartArgs& q, int grid, cudaStream_t st) {
-  switch (a.a) {
-    case 1: k_tab_items<1, FMT><<<grid, 256, 0, st>>>(a, t, q); break;
-    case 2: k_tab_items<2, FMT><<<grid, 256, 0, st>>>(a, t, q); break;
-    case 3: k_tab_items<3, FMT><<<grid, 256, 0, st>>>(a, t, q); break;
-    case 4: k_tab_items<4, FMT><<<grid, 256, 0, st>>>(a, t, q); break;
-    default: k_tab_items<5, FMT><<<grid, 256, 0, st>>>(a, t, q); break;
-  }
-  count_launch();
-  return cudaGetLastError();
+  return std::max<int64_t>(1, std::min<int64_t>(nr, nwarps));
 }
 
 // SK_PART_UPDATE=0 keeps the single-phase k_update_tab (and the per-tuple update) for batches
@@ -540,13 +742,36 @@ int64_t part_window(int64_t n) {
 
 // Regions of a window of W tuples: the phase-1 grid has at most sms x kPartMaxCtasPerSm CTAs
 // of 256 threads, so its warps' regions hold at most W + that many threads' tiles per row.
-size_t part_items_bytes(int d, int64_t W, int sms) {
+size_t part_items_bytes(int d, int64_t W, int sms, bool weighted) {
   const int64_t threads = (int64_t)sms * kPartMaxCtasPerSm * 256;
-  return ((size_t)d * (size_t)(W + threads) * sizeof(uint16_t) + 255) & ~(size_t)255;
+  return ((size_t)d * (size_t)(W + threads) * (weighted ? sizeof(uint32_t) : sizeof(uint16_t)) + 255) & ~(size_t)255;
 }
 
-size_t part_staging_bytes(int d, int64_t W, int sms) {
-  return part_items_bytes(d, W, sms) + (size_t)sms * kPartMaxCtasPerSm * 8 * 16 * sizeof(uint32_t);
+size_t part_staging_bytes(int d, int64_t W, int sms, bool weighted = false) {
+  return part_items_bytes(d, W, sms, weighted) + (size_t)sms * kPartMaxCtasPerSm * 8 * 16 * sizeof(uint32_t);
+}
+
+// Phase 2 over the regions of a window: R and the pieces per region follow from part_ranges.
+struct PartSplit {
+  int64_t nr;   // ranges per (row, part)
+  int R;        // regions per range
+  int logP;     // pieces per region, log2: a CTA's 32 warps get equal shares
+};
+
+PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps) {
+  PartSplit p;
+  p.nr = part_ranges(items, units, slots, nwarps);
+  p.R = (int)((nwarps + p.nr - 1) / p.nr);
+  p.nr = (nwarps + p.R - 1) / p.R;
+  p.logP = 5;
+  for (int lp = 0; lp < 5; lp++) {
+    const int64_t pcs = (int64_t)p.R << lp;
+    if ((pcs + 31) / 32 * 32 * 100 <= pcs * 105) {
+      p.logP = lp;
+      break;
+    }
+  }
+  return p;
 }
 
 // Both phases over every window of the batch; staging (part_staging_bytes) is caller-owned.
@@ -556,16 +781,17 @@ size_t part_staging_bytes(int d, int64_t W, int sms) {
 cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* staging, int sms, cudaStream_t st,
                             const int64_t* const* colp = nullptr, const uint32_t* vbits = nullptr) {
   const int64_t n = a.n;
+  const bool weighted = a.w != nullptr;
+  TabItemsKernel items = tab_items_kernel(a.a, fmt, weighted);
+  auto accum = weighted ? k_part_accum<true> : k_part_accum<false>;
   int tab_per_sm = 1;
-  cudaError_t e = fmt == 0   ? tab_items_occupancy<0>(a.a, &tab_per_sm)
-                  : fmt == 2 ? tab_items_occupancy<2>(a.a, &tab_per_sm)
-                             : tab_items_occupancy<1>(a.a, &tab_per_sm);
+  cudaError_t e = tab_items_per_sm(items, &tab_per_sm);
   if (e != cudaSuccess) return e;
   const int64_t full_grid = (int64_t)sms * tab_per_sm;
   const int64_t W = part_window(n);
   PartArgs q;
-  q.items = (uint16_t*)staging;
-  q.cnts = (uint32_t*)((char*)staging + part_items_bytes(a.d, W, sms));
+  q.items = staging;
+  q.cnts = (uint32_t*)((char*)staging + part_items_bytes(a.d, W, sms, weighted));
   q.W = W;
   int logm = 0;
   while (((int64_t)1 << logm) < (int64_t)a.m) logm++;
@@ -573,9 +799,9 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
   q.logL = logL;
   const int S = (int)(a.m >> logL);
   const size_t smem = (size_t)4 << logL;
-  e = allow_dynamic_smem((const void*)k_part_accum);
+  e = allow_dynamic_smem((const void*)accum);
   int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_part_accum, 1024, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accum, 1024, smem);
   const int64_t slots = (int64_t)sms * std::max(1, per_sm);
   const int64_t units = (int64_t)S * a.d;
   for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += W) {
@@ -587,28 +813,15 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
     const int64_t gend = (q.cnt + 31) / 32 * 32;
     q.C = 32 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
     q.nwarps = grid * 8;
-    e = fmt == 0   ? dispatch_tab_items<0>(a, t, q, grid, st)
-        : fmt == 2 ? dispatch_tab_items<2>(a, t, q, grid, st)
-                   : dispatch_tab_items<1>(a, t, q, grid, st);
+    const PartSplit sp = part_split(q.cnt * a.d, units, slots, q.nwarps);
+    // a phase-2 counter sums at most R C weighted items: below 2^31 in magnitude
+    q.wts = weighted ? a.w + i0 : nullptr;
+    q.wmax = std::min<int64_t>(65535, 0x7fffffff / ((int64_t)sp.R * q.C));
+    items<<<grid, 256, 0, st>>>(a, t, q);
+    count_launch();
+    e = cudaGetLastError();
     if (e != cudaSuccess) break;
-    // ranges of phase-1 warps per (row, part): the grid a whole number of waves when that
-    // takes 2..64 waves; pieces per region so that a CTA's 32 warps get equal shares
-    int64_t nr = 0;
-    for (int64_t k = 2; k <= 64 && !nr; k++)
-      if ((k * slots) % units == 0) nr = k * slots / units;
-    if (!nr) nr = (4 * slots + units - 1) / units;
-    nr = std::max<int64_t>(1, std::min<int64_t>(nr, q.nwarps));
-    const int R = (int)((q.nwarps + nr - 1) / nr);
-    nr = (q.nwarps + R - 1) / R;
-    int logP = 3;
-    for (int lp = 0; lp < 3; lp++) {
-      const int64_t pcs = (int64_t)R << lp;
-      if ((pcs + 31) / 32 * 32 * 100 <= pcs * 105) {
-        logP = lp;
-        break;
-      }
-    }
-    k_part_accum<<<(unsigned)(units * nr), 1024, smem, st>>>(q, a.ctr, (int64_t)a.m, a.d, logL, R, logP);
+    accum<<<(unsigned)(units * sp.nr), 1024, smem, st>>>(q, a.ctr, (int64_t)a.m, a.d, logL, sp.R, sp.logP);
     count_launch();
     e = cudaGetLastError();
   }
@@ -1780,12 +1993,12 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     t.base[rp.a] = total;
     t.narrow = s->m <= 65536 && s->d <= 32;
     t.rvec = key_record_vectors(s->d, t.narrow);
-    // The two-phase partitioned update (unit weights, power-of-two 1024 <= m <= 2^16, d <= 14,
+    // The two-phase partitioned update (power-of-two 1024 <= m <= 2^16, d <= 14,
     // at most 5 attributes, sketch too large for one CTA's shared memory, at least 16 tuples
     // per counter of a row, fewer than 2^32 table records) takes 24-byte records for d <= 9
     // (the 32-byte 20-bit lane ones with SK_PART_RECORD=32) and the narrow 32-byte format
     // otherwise.
-    bool part = part_update_mode() != 0 && pow2 && weights == nullptr && rp.a <= 5 && !use_smem && s->m >= 1024 &&
+    bool part = part_update_mode() != 0 && pow2 && rp.a <= 5 && !use_smem && s->m >= 1024 &&
                 s->m <= 65536 && s->d <= 14 && n >= (int64_t)s->m * 16 && total < ((int64_t)1 << 32);
     const int part_fmt = s->d <= 9 ? (part_record_bytes() == 32 ? 0 : 2) : 1;
     // The wide partitioned update (unit weights, power-of-two 2^17 <= m <= 2^24, d <= 16, at most
@@ -1807,7 +2020,7 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     const bool sorted_parts = s->m <= ((int64_t)kSortMaxParts << 15);
     void* staging = nullptr;
     if (fits && worth && total > 0 && part) {
-      e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n), sms), st);
+      e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n), sms, weights != nullptr), st);
       if (e != cudaSuccess) {
         cudaGetLastError();   // no room for the planes: single-phase update
         staging = nullptr;
@@ -1942,6 +2155,91 @@ sk_status launch_merge(int64_t* dst, const int64_t* src, int64_t count, cudaStre
   return set_status_from_cuda(cudaGetLastError());
 }
 
+namespace {
+
+using ViewItemsKernel = void (*)(UpdArgs, TabArgs, PartArgs, ViewMasks);
+
+template <bool ALL9>
+ViewItemsKernel view_items_kernel(int A) {
+  switch (A) {
+    case 1: return k_tab_items_views<1, ALL9>;
+    case 2: return k_tab_items_views<2, ALL9>;
+    case 3: return k_tab_items_views<3, ALL9>;
+    case 4: return k_tab_items_views<4, ALL9>;
+    default: return k_tab_items_views<5, ALL9>;
+  }
+}
+
+// Staging of the views' items for windows of W tuples, and the window that keeps it near 3 GiB
+// (the library's pool keeps 4 GiB between calls): a batch is cut into equal windows.
+size_t view_items_bytes(int nv, int d, int64_t W, int sms) { return nv * part_items_bytes(d, W, sms, false); }
+
+int64_t view_window(int nv, int d, int64_t n) {
+  const int64_t most = std::max<int64_t>(1 << 20, ((int64_t)3 << 30) / ((int64_t)nv * d * 2));
+  const int64_t wins = (n + most - 1) / most;
+  return part_window((n + wins - 1) / wins);
+}
+
+// The relation's 24-byte key records (every attribute in one join).
+cudaError_t family_table(const UpdArgs& a, const TabArgs& t, int64_t total, int sms, cudaStream_t st) {
+  const size_t coef_bytes = (size_t)a.d * a.row_len * sizeof(uint64_t);
+  const cudaError_t e = fit_dynamic_smem((const void*)k_key_table_l24<true>, coef_bytes);
+  if (e != cudaSuccess) return e;
+  const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
+  k_key_table_l24<true><<<bgrid, 256, coef_bytes, st>>>(a, t);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// Both phases of all nv views over every window; staging: view_items_bytes, then the counts.
+cudaError_t run_partitioned_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm,
+                                  unsigned long long* const* ctr, void* staging, int64_t W, int sms, cudaStream_t st) {
+  ViewItemsKernel items = a.d == 9 ? view_items_kernel<true>(a.a) : view_items_kernel<false>(a.a);
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, items, 256, 0);
+  if (e != cudaSuccess) return e;
+  const int64_t full_grid = (int64_t)sms * std::max(1, std::min(per_sm, kPartMaxCtasPerSm));
+  PartArgs q;
+  q.cnts = (uint32_t*)((char*)staging + view_items_bytes(vm.nv, a.d, W, sms));
+  q.W = W;
+  int logm = 0;
+  while (((int64_t)1 << logm) < (int64_t)a.m) logm++;
+  q.logL = std::min(logm, 15);
+  q.vbits = nullptr;
+  q.wts = nullptr;
+  q.wmax = 0;
+  const int S = (int)(a.m >> q.logL);
+  const size_t smem = (size_t)4 << q.logL;
+  e = allow_dynamic_smem((const void*)k_part_accum<false>);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_part_accum<false>, 1024, smem);
+  const int64_t slots = (int64_t)sms * std::max(1, per_sm), units = (int64_t)S * a.d;
+  for (int64_t i0 = 0; i0 < a.n && e == cudaSuccess; i0 += W) {
+    q.items = staging;
+    q.cnt = std::min(W, a.n - i0);
+    for (int u = 0; u < 5; u++) q.col[u] = u < a.a ? a.cols + (int64_t)u * a.stride + i0 : nullptr;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((q.cnt + 255) / 256, full_grid));
+    const int64_t gend = (q.cnt + 31) / 32 * 32;
+    q.C = 256 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
+    q.nwarps = grid;   // regions are the CTAs'
+    items<<<grid, 256, 0, st>>>(a, t, q, vm);
+    count_launch();
+    e = cudaGetLastError();
+    const PartSplit sp = part_split(q.cnt * a.d, units, slots, q.nwarps);
+    for (int v = 0; v < vm.nv && e == cudaSuccess; v++) {
+      PartArgs qv = q;
+      qv.items = (uint16_t*)q.items + (int64_t)v * q.nwarps * a.d * q.C;
+      qv.cnts = q.cnts + (int64_t)v * q.nwarps * 16;
+      k_part_accum<false><<<(unsigned)(units * sp.nr), 1024, smem, st>>>(qv, ctr[v], (int64_t)a.m, a.d, q.logL, sp.R,
+                                                                         sp.logP);
+      count_launch();
+      e = cudaGetLastError();
+    }
+  }
+  return e;
+}
+
+}  // namespace
+
 // One bit per tuple: all of the relation's keys inside their declared domains (a tuple with a
 // key outside is reported and left out of every view).
 __global__ void __launch_bounds__(256) k_valid_bits(UpdArgs p, uint32_t* bits) {
@@ -2003,6 +2301,35 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
     cudaGetLastError();
     return SK_OK;
   }
+  // All views in one first phase: for two views or more of a relation of at most five attributes,
+  // from 2^21 tuples (a 4-attribute relation's 15 views, m = 2^16, d = 9, against one view at a
+  // time: 0.80 and 0.82 ms at 2^20 tuples, where the second phases are most of either form, 1.10
+  // and 1.17 at 2^21, 3.00 and 3.59 at 2^23).
+  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)1 << 21)) {
+    ViewMasks vm;
+    vm.nv = 0;
+    unsigned long long* vctr[SK_MAX_VIEWS];
+    for (int v = 0; v < nv; v++)
+      if (amask[v]) {
+        vctr[vm.nv] = ctr[v];
+        vm.mask[vm.nv++] = (uint8_t)amask[v];
+      }
+    const int64_t W = view_window(vm.nv, a.d, n);
+    const size_t vbytes = view_items_bytes(vm.nv, a.d, W, sms) +
+                          (size_t)vm.nv * sms * kPartMaxCtasPerSm * 16 * sizeof(uint32_t);
+    if (pool_malloc_async(&staging, vbytes, st) == cudaSuccess) {
+      *done = true;
+      t.tbl = (uint32_t*)tbl;
+      cudaError_t e = family_table(a, t, total, sms, st);
+      if (e == cudaSuccess) e = run_partitioned_views(a, t, vm, vctr, staging, W, sms, st);
+      cudaError_t ef = cudaFreeAsync(tbl, st);
+      const cudaError_t es = cudaFreeAsync(staging, st);
+      if (ef == cudaSuccess) ef = es;
+      return set_status_from_cuda(e != cudaSuccess ? e : ef);
+    }
+    cudaGetLastError();   // no room for the views' items: one view at a time
+    staging = nullptr;
+  }
   const size_t sbytes = part_staging_bytes(a.d, part_window(n), sms);
   const size_t vbytes = (size_t)(n + 31) / 32 * sizeof(uint32_t);
   if (pool_malloc_async(&staging, sbytes + ((vbytes + 255) & ~(size_t)255), st) != cudaSuccess) {
@@ -2013,14 +2340,7 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
   *done = true;
   uint32_t* vbits = (uint32_t*)((char*)staging + sbytes);
   t.tbl = (uint32_t*)tbl;
-  const size_t coef_bytes = (size_t)a.d * a.row_len * sizeof(uint64_t);
-  cudaError_t e = fit_dynamic_smem((const void*)k_key_table_l24<true>, coef_bytes);
-  if (e == cudaSuccess) {
-    const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
-    k_key_table_l24<true><<<bgrid, 256, coef_bytes, st>>>(a, t);
-    count_launch();
-    e = cudaGetLastError();
-  }
+  cudaError_t e = family_table(a, t, total, sms, st);
   if (e == cudaSuccess) {
     k_valid_bits<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, vbits);
     count_launch();
