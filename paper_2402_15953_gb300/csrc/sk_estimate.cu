@@ -328,7 +328,6 @@ __host__ __device__ __forceinline__ uint64_t gl_pow(uint64_t b, uint64_t e) {
 struct CplxOps {
   using T = double2;
   static constexpr bool kExact = false;   // rounding: twiddles always come from the table
-  static constexpr bool kReg = false;     // transforms through smem_dif_il
   static __device__ __forceinline__ T mul(T a, T b) { return cmul(a, b); }
   static __device__ __forceinline__ T add(T a, T b) { return make_double2(a.x + b.x, a.y + b.y); }
   static __device__ __forceinline__ T sub(T a, T b) { return make_double2(a.x - b.x, a.y - b.y); }
@@ -347,7 +346,6 @@ struct CplxOps {
 struct GlOps {
   using T = uint64_t;
   static constexpr bool kExact = true;
-  static constexpr bool kReg = false;   // transforms through smem_dif_il
   static __device__ __forceinline__ T mul(T a, T b) { return gl_mul(a, b); }
   static __device__ __forceinline__ T add(T a, T b) { return gl_add(a, b); }
   static __device__ __forceinline__ T sub(T a, T b) { return gl_sub(a, b); }
@@ -500,122 +498,6 @@ __device__ void smem_dif_il(typename Ops::T* s, int cnt, int S, int logL, const 
   }
 }
 
-// ---------------------------------------------------------------------------
-// Register transforms (exact arithmetics only, lengths L = 2^6..2^10).  A length-L DFT in
-// natural order is taken as A x B (L = A B): with x_i at i = B a + b and X_k at k = c + A e,
-//   X[c + A e] = sum_b w_B^(b e) (w_L^(b c) sum_a x[B a + b] w_A^(a c)),
-// so step 1 gives each thread one b: the A-point DFT over a of its stride-B elements, held in
-// registers, times w_L^(b c), written back to the same positions B c + b; step 2 gives each
-// thread one c: the B-point DFT over b of the contiguous block B c .. B c + B - 1, written
-// to the positions c + A e.  Every twiddle is a power of w_L, read from an L-entry table in
-// shared memory (the same entry across the threads of one vector: broadcast reads).
-// ---------------------------------------------------------------------------
-template <int LOG>
-__host__ __device__ constexpr int bitrev_const(int k) {
-  int r = 0;
-  for (int i = 0; i < LOG; i++) r |= ((k >> i) & 1) << (LOG - 1 - i);
-  return r;
-}
-
-// 2^LOG-point DFT of x (natural order in and out); wt[j] = w_N^j for j < N / 2.  Radix-2
-// decimation in frequency (stage s pairs j and j + N / 2^(s+1) with the twiddle
-// w_N^(j 2^s)), then the bit reversal as a renaming of registers.
-template <class Ops, int LOG>
-__device__ __forceinline__ void reg_dft(typename Ops::T (&x)[1 << LOG], const typename Ops::T (&wt)[(1 << LOG) / 2]) {
-  using T = typename Ops::T;
-  constexpr int N = 1 << LOG;
-#pragma unroll
-  for (int st = 0; st < LOG; st++) {
-    const int h = N >> (st + 1);
-#pragma unroll
-    for (int blk = 0; blk < N; blk += 2 * h) {
-#pragma unroll
-      for (int j = 0; j < h; j++) {
-        const T u = x[blk + j], v = x[blk + j + h];
-        x[blk + j] = Ops::add(u, v);
-        const T dl = Ops::sub(u, v);
-        x[blk + j + h] = j == 0 ? dl : Ops::mul(dl, wt[j << st]);
-      }
-    }
-  }
-  T y[N];
-#pragma unroll
-  for (int k = 0; k < N; k++) y[k] = x[bitrev_const<LOG>(k)];
-#pragma unroll
-  for (int k = 0; k < N; k++) x[k] = y[k];
-}
-
-// In-place natural-order DFTs of `cnt` (a power of two) vectors of length L = 2^(LA + LB),
-// element i of vector v at s[i S + v]; stw[e] = w_L^e for e < L.  Needs cnt 2^max(LA, LB)
-// <= blockDim.x (one A- or B-point DFT per thread and step).  Ends with a barrier.
-template <class Ops, int LA, int LB>
-__device__ void smem_ntt_2lvl(typename Ops::T* s, int cnt, int S, const typename Ops::T* stw) {
-  using T = typename Ops::T;
-  constexpr int A = 1 << LA, B = 1 << LB;
-  const int lc = __ffs(cnt) - 1;
-  const int t = threadIdx.x;
-  {
-    T w[A / 2];
-#pragma unroll
-    for (int j = 0; j < A / 2; j++) w[j] = stw[B * j];   // w_A^j
-    if (t < cnt * B) {
-      const int v = t & (cnt - 1), b = t >> lc;
-      T x[A];
-#pragma unroll
-      for (int a = 0; a < A; a++) x[a] = s[(B * a + b) * S + v];
-      reg_dft<Ops, LA>(x, w);
-#pragma unroll
-      for (int c = 1; c < A; c++) x[c] = Ops::mul(x[c], stw[b * c]);
-#pragma unroll
-      for (int c = 0; c < A; c++) s[(B * c + b) * S + v] = x[c];
-    }
-  }
-  __syncthreads();
-  {
-    T w[B / 2];
-#pragma unroll
-    for (int j = 0; j < B / 2; j++) w[j] = stw[A * j];   // w_B^j
-    const bool act = t < cnt * A;
-    const int v = t & (cnt - 1), c = t >> lc;
-    T x[B];
-    if (act) {
-#pragma unroll
-      for (int b = 0; b < B; b++) x[b] = s[(B * c + b) * S + v];
-    }
-    __syncthreads();   // every block read before any position c + A e is written
-    if (act) {
-      reg_dft<Ops, LB>(x, w);
-#pragma unroll
-      for (int e = 0; e < B; e++) s[(c + A * e) * S + v] = x[e];
-    }
-  }
-  __syncthreads();
-}
-
-// The register transform for length 2^logL when this arithmetic has one (kReg) and the tile
-// of cnt vectors fits it; fills stw (L entries) from the length-N half table first.  false:
-// nothing done (the caller takes smem_dif_il, bit-reversed output).
-template <class Ops>
-__device__ bool smem_ntt_reg(typename Ops::T* s, int cnt, int S, int logL, const typename Ops::T* __restrict__ tw,
-                             int64_t twstride, int64_t N, bool inv, typename Ops::T* stw) {
-  if constexpr (Ops::kReg) {
-    if (logL < 6 || logL > 10 || (cnt << (logL - logL / 2)) > (int)blockDim.x) return false;
-    const int L = 1 << logL;
-    for (int e = threadIdx.x; e < L; e += blockDim.x) stw[e] = twid<Ops>(tw, ((int64_t)e * twstride) & (N - 1), N >> 1, inv);
-    __syncthreads();
-    switch (logL) {
-      case 6: smem_ntt_2lvl<Ops, 3, 3>(s, cnt, S, stw); break;
-      case 7: smem_ntt_2lvl<Ops, 3, 4>(s, cnt, S, stw); break;
-      case 8: smem_ntt_2lvl<Ops, 4, 4>(s, cnt, S, stw); break;
-      case 9: smem_ntt_2lvl<Ops, 4, 5>(s, cnt, S, stw); break;
-      default: smem_ntt_2lvl<Ops, 5, 5>(s, cnt, S, stw); break;
-    }
-    return true;
-  } else {
-    return false;
-  }
-}
-
 // loads each thread of the four-step passes keeps in flight while filling its tile (16
 // measured no faster than 8 for 32-bit residues)
 template <class T>
@@ -653,10 +535,7 @@ __global__ void __launch_bounds__(512, 2) k_xf_cols(typename Ops::T* __restrict_
     }
   }
   __syncthreads();
-  // natural-order register transform where it applies (its twiddle table after the tile),
-  // else the radix-2 one with bit-reversed output
-  const bool nat = smem_ntt_reg<Ops>(sm, cb, S, logR, tw, C, N, inv, sm + (int64_t)R * S);
-  if (!nat) smem_dif_il<Ops>(sm, cb, S, logR, tw, C, inv, r4);
+  smem_dif_il<Ops>(sm, cb, S, logR, tw, C, inv, r4);
   const int64_t half = N >> 1;
   if (Ops::kExact && (blockDim.x & (cb - 1)) == 0) {
     // each thread keeps one column n2 and walks rows k1 = k1_0 + j kstep: the twiddle
@@ -667,7 +546,7 @@ __global__ void __launch_bounds__(512, 2) k_xf_cols(typename Ops::T* __restrict_
     T w = twid<Ops>(tw, (n2 * (threadIdx.x >> lcb)) & (N - 1), half, inv);
     const T ws = twid<Ops>(tw, (n2 * kstep) & (N - 1), half, inv);
     for (int k1 = threadIdx.x >> lcb; k1 < R; k1 += kstep) {
-      v[(int64_t)k1 * C + n2] = Ops::mul(sm[(nat ? k1 : bitrev(k1, logR)) * S + c], w);
+      v[(int64_t)k1 * C + n2] = Ops::mul(sm[bitrev(k1, logR) * S + c], w);
       w = Ops::mul(w, ws);
     }
   } else {
@@ -675,7 +554,7 @@ __global__ void __launch_bounds__(512, 2) k_xf_cols(typename Ops::T* __restrict_
       const int c = idx & (cb - 1), k1 = idx >> lcb;
       const int64_t n2 = c0 + c;
       const T w = twid<Ops>(tw, (n2 * k1) & (N - 1), half, inv);
-      v[(int64_t)k1 * C + n2] = Ops::mul(sm[(nat ? k1 : bitrev(k1, logR)) * S + c], w);
+      v[(int64_t)k1 * C + n2] = Ops::mul(sm[bitrev(k1, logR) * S + c], w);
     }
   }
 }
@@ -712,11 +591,10 @@ __global__ void __launch_bounds__(512, 2) k_xf_rows(const typename Ops::T* __res
     }
   }
   __syncthreads();
-  const bool nat = smem_ntt_reg<Ops>(sm, rb, S, logC, tw, R, N, inv, sm + (int64_t)C * S);
-  if (!nat) smem_dif_il<Ops>(sm, rb, S, logC, tw, R, inv, r4);
+  smem_dif_il<Ops>(sm, rb, S, logC, tw, R, inv, r4);
   for (int idx = threadIdx.x; idx < C * rb; idx += blockDim.x) {
     const int rr = idx & (rb - 1), k2 = idx >> lrb;
-    vo[(int64_t)(r0 + rr) + (int64_t)R * k2] = sm[(nat ? k2 : bitrev(k2, logC)) * S + rr];
+    vo[(int64_t)(r0 + rr) + (int64_t)R * k2] = sm[bitrev(k2, logC) * S + rr];
   }
 }
 
@@ -1216,6 +1094,20 @@ cudaError_t ensure(Scratch& s, size_t bytes, cudaStream_t st) {
     if (_s != SK_OK) return _s;    \
   } while (0)
 
+// xform for lengths up to 2^12: whole transforms in shared memory.
+template <class Ops>
+sk_status xform_small(typename Ops::T* src, typename Ops::T* dst, int64_t batch, int64_t m, const typename Ops::T* tw,
+                      bool inv, typename Ops::T r4, cudaStream_t st) {
+  const int L = (int)m;
+  const int vpc = (int)std::max<int64_t>(1, std::min<int64_t>(4096 / L, batch));
+  const int64_t grid = (batch + vpc - 1) / vpc;
+  const size_t smem = (size_t)vpc * L * sizeof(typename Ops::T);
+  SK_CK(allow_dynamic_smem((const void*)k_xf_small<Ops>));
+  k_xf_small<Ops><<<(unsigned)grid, 256, smem, st>>>(src, dst, batch, ilog2(m), vpc, tw, 1, inv, r4);
+  count_launch();
+  return set_status_from_cuda(cudaGetLastError());
+}
+
 // Forward (inv = false) or inverse (unnormalised) transform of `batch` vectors of
 // length m held in src; the result is written to dst, src is clobbered.  Complex FP64
 // with the W table (conjugated for the inverse), or GF(q) with the w^t / w^-t table.
@@ -1225,16 +1117,7 @@ sk_status xform(typename Ops::T* src, typename Ops::T* dst, int64_t batch, int64
   using T = typename Ops::T;
   const int logm = ilog2(m);
   const int esz = (int)sizeof(T);
-  if (logm <= 12) {
-    const int L = (int)m;
-    const int vpc = (int)std::max<int64_t>(1, std::min<int64_t>(4096 / L, batch));
-    const int64_t grid = (batch + vpc - 1) / vpc;
-    const size_t smem = (size_t)vpc * L * esz;
-    SK_CK(allow_dynamic_smem((const void*)k_xf_small<Ops>));
-    k_xf_small<Ops><<<(unsigned)grid, 256, smem, st>>>(src, dst, batch, logm, vpc, tw, 1, inv, r4);
-    count_launch();
-    return set_status_from_cuda(cudaGetLastError());
-  }
+  if (logm <= 12) return xform_small<Ops>(src, dst, batch, m, tw, inv, r4, st);
   const int logR = logm / 2, logC = logm - logR;
   const int R = 1 << logR, C = 1 << logC;
   // 64 KB tiles: two or three CTAs per SM (measured against 128 KB at m = 2^20, one CTA per SM:
@@ -1248,20 +1131,7 @@ sk_status xform(typename Ops::T* src, typename Ops::T* dst, int64_t batch, int64
   while (cb > 4 && batch * (C / cb) < want) cb >>= 1;
   while (rb > 1 && batch * (R / rb) < want) rb >>= 1;
   if ((cb & (cb - 1)) || (rb & (rb - 1))) return SK_ERR_INVALID_ARG;   // the kernels index by shifts
-  // the register transform (exact arithmetics, lengths 2^6..2^10) takes one A- or B-point DFT
-  // per thread: at most 512 >> max(log A, log B) vectors per tile; plus its twiddle table
-  size_t smc_tw = 0, smr_tw = 0;
-  if (Ops::kReg) {
-    if (logR >= 6 && logR <= 10) {
-      cb = std::min(cb, 512 >> (logR - logR / 2));
-      smc_tw = (size_t)R * esz;
-    }
-    if (logC >= 6 && logC <= 10) {
-      rb = std::min(rb, 512 >> (logC - logC / 2));
-      smr_tw = (size_t)C * esz;
-    }
-  }
-  const size_t smc = (size_t)(cb + 1) * R * esz + smc_tw, smr = (size_t)(rb + 1) * C * esz + smr_tw;   // padded tiles
+  const size_t smc = (size_t)(cb + 1) * R * esz, smr = (size_t)(rb + 1) * C * esz;   // padded tiles
   SK_CK(allow_dynamic_smem((const void*)k_xf_cols<Ops>));
   SK_CK(allow_dynamic_smem((const void*)k_xf_rows<Ops>));
   k_xf_cols<Ops><<<(unsigned)(batch * (C / cb)), 512, smc, st>>>(src, logR, logC, cb, tw, inv, r4);
@@ -1474,7 +1344,6 @@ template <int PI>
 struct MontOps {
   using T = uint32_t;
   static constexpr bool kExact = true;
-  static constexpr bool kReg = true;    // lengths 2^6..2^10 through smem_ntt_2lvl
   static __device__ __forceinline__ T mul(T a, T b) { return mont32(a, b, c_fu_p[PI], c_fu_pinv[PI]); }
   static __device__ __forceinline__ T add(T a, T b) {
     const uint32_t p = c_fu_p[PI], s = a + b;
@@ -1739,7 +1608,7 @@ sk_status fu_prime_pass(sk_set* s, const FuPrime& fp, int64_t M, uint32_t* V, ui
       s->d_fu_rel, r, d, M, fp.r2, fp.r3, V);
   count_launch();
   SK_CK(cudaGetLastError());
-  sk_status fs = xform<MontOps<PI>>(V, W, (int64_t)r * d, M, tw, false, r4, st);
+  sk_status fs = xform_small<MontOps<PI>>(V, W, (int64_t)r * d, M, tw, false, r4, st);
   if (fs != SK_OK) return fs;
   k_fu_reduce<PI><<<d * nchunk, 256, 0, st>>>(W, r, d, M, negmask, nchunk, part);
   k_fu_final<PI><<<(d + 63) / 64, 64, 0, st>>>(part, d, nchunk, fw.minv, res, np);
@@ -2323,164 +2192,151 @@ sk_status run_estimate_pairwise(sk_set* s, sk_estimate* out, cudaStream_t st, bo
 }
 
 // ---------------------------------------------------------------------------
-// Algorithm 3 step by step modulo each CRT prime, for every query shape (components of
-// three or more attributes, Figure 3) and every width.  The schedule is the one the
-// stepwise estimate runs; the row estimate is a polynomial in the counters, so running it
-// in Z/p for each prime and reconstructing by CRT (np from the l1 bound above) gives it
-// exactly, with one transform per operand of a correlation and no limbs.  Slots hold d
-// rows of M residues (Montgomery form), zero beyond m.
+// Algorithm 3 step by step modulo the CRT primes, for every query shape (components of three
+// or more attributes, Figure 3) and every width.  The schedule is the one the stepwise estimate
+// runs; the row estimate is a polynomial in the counters, so running it in Z/p for each prime
+// and reconstructing by CRT (np from the l1 bound above) gives it exactly, with no limbs.  All
+// primes that fit the scratch run in each launch.  A leaf is its relation's counters themselves; a
+// correlation is two column passes, one row pass (k_ntt_corr) and a column pass back, and for
+// widths that are not a power of two at least 1024 (zero-padded to M >= 2m - 1) its circular fold
+// happens where the result is read; a Hadamard product that only feeds the sum is not stored.
+// Every entry of a slot carries the same known factor 2^(-32 e) M^f, taken out of the sums here.
+// Zeroing, three updates of 10^6 tuples and this estimate for a chain of three, m = 10^6, d = 5 (3
+// primes, M = 2^21): 1.49 ms; 2.82 ms with a kernel per leaf, product, fold and transform pass and prime.
 // ---------------------------------------------------------------------------
-template <int PI>
-__global__ void k_crt_leaf(const int64_t* __restrict__ c, int d, int64_t m, int64_t M, uint32_t r2, uint32_t r3,
-                           uint32_t* __restrict__ out) {
-  using O = MontOps<PI>;
-  const uint32_t p = c_fu_p[PI];
-  const int64_t total = (int64_t)d * M, step = (int64_t)gridDim.x * blockDim.x;
-  const int lM = __ffsll((unsigned long long)M) - 1;   // M is a power of two
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
-    const int64_t row = g >> lM, j = g - row * M;
-    uint32_t v = 0;
-    if (j < m) {
-      const int64_t x = c[row * m + j];
-      const uint64_t mag = x < 0 ? 0ull - (uint64_t)x : (uint64_t)x;
-      uint32_t h = (uint32_t)(mag >> 32);
-      if (h >= p) h -= p;
-      v = O::add(O::mul(h, r3), O::mul((uint32_t)mag, r2));
-      if (x < 0) v = O::neg(v);
-    }
-    out[g] = v;
-  }
-}
-
-template <int PI>
-__global__ void k_crt_had(uint32_t* __restrict__ x, const uint32_t* __restrict__ y, int64_t n) {
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += step)
-    x[g] = MontOps<PI>::mul(x[g], y[g]);
-}
-
-// X[row][k] <- A[row][-k mod M] X[row][k] / M: the spectrum of z = a (star) x, since
-// sum_j z_j w^jk = sum_i a_i w^-ik sum_t x_t w^tk (Definition 3.1, t = i + j mod M)
-template <int PI>
-__global__ void k_crt_product(const uint32_t* __restrict__ A, uint32_t* __restrict__ X, int d, int64_t M,
-                              uint32_t minv) {
-  using O = MontOps<PI>;
-  const int64_t total = (int64_t)d * M, step = (int64_t)gridDim.x * blockDim.x;
-  const int lM = __ffsll((unsigned long long)M) - 1;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
-    const int64_t row = g >> lM, k = g - row * M;
-    X[g] = O::mul(O::mul(A[row * M + ((M - k) & (M - 1))], X[g]), minv);
-  }
-}
-
-// x[row][j] = L[row][j] + L[row][j - m mod M] for j < m, 0 beyond: the circular correlation
-// mod m from the length-M one of the zero-padded rows (M >= 2m - 1)
-template <int PI>
-__global__ void k_crt_fold(const uint32_t* __restrict__ L, uint32_t* __restrict__ x, int d, int64_t m, int64_t M) {
-  const int64_t total = (int64_t)d * M, step = (int64_t)gridDim.x * blockDim.x;
-  const int lM = __ffsll((unsigned long long)M) - 1;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
-    const int64_t row = g >> lM, j = g - row * M;
-    x[g] = j < m ? MontOps<PI>::add(L[g], L[row * M + M - m + j]) : 0u;
-  }
-}
-
-// part[row * nchunk + c] = sum of the c-th chunk of row `row` (mod p)
-template <int PI>
-__global__ void __launch_bounds__(256) k_crt_rowsum(const uint32_t* __restrict__ x, int64_t M, int nchunk,
-                                                    uint32_t* part) {
-  using O = MontOps<PI>;
-  __shared__ uint32_t red[256];
-  const int row = blockIdx.x / nchunk, c = blockIdx.x % nchunk;
-  const int64_t clen = M / nchunk;
-  const uint32_t* v = x + (int64_t)row * M + (int64_t)c * clen;
-  uint32_t s = 0;
-  for (int64_t j = threadIdx.x; j < clen; j += blockDim.x) s = O::add(s, v[j]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int h = blockDim.x >> 1; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) red[threadIdx.x] = O::add(red[threadIdx.x], red[threadIdx.x + h]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-// One prime's run of the schedule; the row sums' residues go to f.d_res[row][PI].
-template <int PI>
-sk_status crt_prime_pass(sk_set* s, const FuPrime& fp, int64_t M, uint32_t* slots, uint32_t* T1, uint32_t* T2,
-                         const FuSetup& f, cudaStream_t st) {
-  using O = MontOps<PI>;
-  const int d = s->d;
-  const int64_t m = s->m, dM = (int64_t)d * M;
-  const FuWidth& fw = fu_width(PI, M);
-  const uint32_t one = fw.one, r4 = fw.r4, r4i = fw.r4i, minv = fw.minv;
-  const uint32_t* tw = s->d_fu_tw + (size_t)PI * M;
-  auto slot = [&](int i) { return slots + (size_t)i * dM; };
-  const int eg = grid_for(dM);
-  for (const EstOp& op : s->plan) {
-    if (op.kind == OP_LEAF) {
-      k_crt_leaf<PI><<<eg, 256, 0, st>>>(s->rel_ctr[op.rel], d, m, M, fp.r2, fp.r3, slot(op.dst));
-      count_launch();
-    } else if (op.kind == OP_HAD) {
-      k_crt_had<PI><<<eg, 256, 0, st>>>(slot(op.dst), slot(op.src), dM);
-      count_launch();
-    } else if (op.kind == OP_CORR) {
-      // src (a) is not read after its correlation, so its slot may be clobbered
-      sk_status e = xform<O>(slot(op.src), T1, d, M, tw, false, r4, st);
-      if (e == SK_OK) e = xform<O>(slot(op.dst), T2, d, M, tw, false, r4, st);
-      if (e != SK_OK) return e;
-      k_crt_product<PI><<<eg, 256, 0, st>>>(T1, T2, d, M, minv);
-      count_launch();
-      SK_CK(cudaGetLastError());
-      if (M == m) {
-        e = xform<O>(T2, slot(op.dst), d, M, tw + M / 2, true, r4i, st);
-        if (e != SK_OK) return e;
-      } else {
-        e = xform<O>(T2, T1, d, M, tw + M / 2, true, r4i, st);
-        if (e != SK_OK) return e;
-        k_crt_fold<PI><<<eg, 256, 0, st>>>(T1, slot(op.dst), d, m, M);
-        count_launch();
-      }
-    } else {   // OP_SUM
-      k_crt_rowsum<PI><<<d * f.nchunk, 256, 0, st>>>(slot(op.dst), M, f.nchunk, f.d_part);
-      k_fu_final<PI><<<(d + 63) / 64, 64, 0, st>>>(f.d_part, d, f.nchunk, one, f.d_res, kFuMaxPrimes);
-      count_launch(2);
-    }
-    SK_CK(cudaGetLastError());
-  }
-  return SK_OK;
-}
-
-// The stepwise CRT estimate; *done false when nine primes do not cover the bound.
 sk_status run_estimate_crt(sk_set* s, sk_estimate* out, cudaStream_t st, bool* done) {
   *done = false;
   const int64_t m = s->m;
-  const int64_t M = (m & (m - 1)) == 0 ? m : (int64_t)1 << ilog2(2 * m - 1);
-  if (M < 2 || M > (1ll << 22) || s->n_slots + 1 > 64) return SK_OK;
+  const int d = s->d;
+  const bool whole = (m & (m - 1)) == 0 && m >= (1ll << ntt::kMinLog);
+  const int64_t M = whole ? m : std::max<int64_t>((int64_t)1 << ntt::kMinLog, (int64_t)1 << ilog2(2 * m - 1));
+  if (m < 2 || M > (1ll << ntt::kMaxLog) || s->n_slots + 1 > 64) return SK_OK;
   FuSetup f;
-  SK_CK_ST(fu_setup(s, M, false, true, st, &f));
+  SK_CK_ST(fu_setup(s, M, false, false, st, &f));
   if (!f.np) return SK_OK;
-  const std::vector<FuPrime>& pr = fu_primes();
-  const size_t dM = (size_t)s->d * M;
-  SK_CK(ensure(s->fft_scratch, (size_t)(s->n_slots + 2) * dM * sizeof(uint32_t), st));
-  uint32_t* slots = (uint32_t*)s->fft_scratch.ptr;
-  uint32_t* T1 = slots + (size_t)s->n_slots * dM;
-  uint32_t* T2 = T1 + dM;
-  for (int i = 0; i < f.np; i++) {
-    sk_status ps;
-    switch (i) {
-#define SK_CRT_CASE(I)                                                   \
-  case I:                                                                \
-    ps = fu_twiddles<I>(s, pr[I], M, st);                                \
-    if (ps == SK_OK) ps = crt_prime_pass<I>(s, pr[I], M, slots, T1, T2, f, st); \
-    break;
-      SK_CRT_CASE(0) SK_CRT_CASE(1) SK_CRT_CASE(2) SK_CRT_CASE(3) SK_CRT_CASE(4) SK_CRT_CASE(5) SK_CRT_CASE(6)
-      SK_CRT_CASE(7) default: SK_CRT_CASE(8)
-#undef SK_CRT_CASE
+  const size_t dM = (size_t)d * M;
+  // buffers: one per slot that a step writes, and two for a correlation's transformed operands
+  std::vector<int> buf(s->n_slots, -1);
+  int nbuf = 2;
+  for (const EstOp& op : s->plan)
+    if ((op.kind == OP_CORR || op.kind == OP_HAD) && buf[op.dst] < 0) buf[op.dst] = nbuf++;
+  const size_t per_prime = (size_t)nbuf * dM * sizeof(uint32_t);
+  const int at_once = (int)std::min<size_t>(f.np, std::max<size_t>(1, ((size_t)1 << 30) / per_prime));
+  const size_t nsum = (size_t)d * kFuMaxPrimes;
+  unsigned long long* d_sums = (unsigned long long*)f.d_res;
+  SK_CK(cudaMemsetAsync(d_sums, 0, nsum * 8, st));
+  uint32_t* pool = nullptr;
+  SK_CK(pool_malloc_async((void**)&pool, (size_t)at_once * per_prime, st));
+  int e_r = 0, e_m = 0;   // the sums' factor: 2^(-32 e_r) M^e_m
+  auto run = [&]() -> sk_status {
+    const int logM = ilog2(M), logR = logM - ntt::kLogRow;
+    for (int i = 0; i < f.np; i += at_once) {
+      const int np = std::min(at_once, f.np - i);
+      auto buffer = [&](int b) { return pool + (size_t)b * np * dM; };
+      struct Slot {
+        int rel = -1;      // >= 0: this relation's counters
+        bool fold = false;
+        int e_r = 0, e_m = 0;
+      };
+      std::vector<Slot> slot(s->n_slots);
+      auto operand = [&](int k) {
+        ntt::Operand o = {nullptr, nullptr, 0};
+        if (slot[k].rel >= 0) o.c = s->rel_ctr[slot[k].rel];
+        else o.u = buffer(buf[k]);
+        if (slot[k].fold) o.fold = M - m;
+        return o;
+      };
+      auto forward = [&](int k, int dir, uint32_t* to) {
+        ntt::ColArgs c;
+        c.base = s->d_fu_rel + std::max(0, slot[k].rel);
+        c.per = d;
+        c.m = m;
+        c.negmask = (unsigned long long)dir;
+        c.dirs = nullptr;
+        c.logR = logR;
+        c.V = to;
+        c.stride = d;
+        c.prime0 = i;
+        for (int t = 0; t < kFuMaxPrimes; t++) c.nvec[t] = d;
+        if (slot[k].rel < 0) {
+          c.words = buffer(buf[k]);
+          c.fold = slot[k].fold ? M - m : 0;
+        }
+        return ntt::cols(c, d, np, st);
+      };
+      for (size_t t = 0; t < s->plan.size(); t++) {
+        const EstOp& op = s->plan[t];
+        if (op.kind == OP_LEAF) {
+          slot[op.dst] = Slot();
+          slot[op.dst].rel = op.rel;
+        } else if (op.kind == OP_CORR) {
+          SK_CK(forward(op.src, 1, buffer(0)));
+          SK_CK(forward(op.dst, 0, buffer(1)));
+          ntt::CorrRowArgs r = {buffer(0), buffer(1), buffer(buf[op.dst]), d, logR, i, d};
+          SK_CK(ntt::corr_rows(r, np, st));
+          ntt::ColArgs c;
+          c.base = nullptr;
+          c.per = d;
+          c.m = M;
+          c.negmask = 1;
+          c.dirs = nullptr;
+          c.logR = logR;
+          c.V = buffer(buf[op.dst]);
+          c.stride = d;
+          c.prime0 = i;
+          for (int k = 0; k < kFuMaxPrimes; k++) c.nvec[k] = d;
+          c.words = c.V;
+          SK_CK(ntt::cols_back(c, d, np, st));
+          Slot z;
+          z.fold = M != m;
+          z.e_r = slot[op.dst].e_r + slot[op.src].e_r + 1;
+          z.e_m = slot[op.dst].e_m + slot[op.src].e_m + 1;
+          slot[op.dst] = z;
+        } else {
+          // a product whose only reader is the sum right after it is summed as it is formed
+          const bool had = op.kind == OP_HAD;
+          const EstOp* next = t + 1 < s->plan.size() ? &s->plan[t + 1] : nullptr;
+          const bool sum = !had || (next && next->kind == OP_SUM && next->dst == op.dst);
+          ntt::HadArgs h;
+          h.x = operand(op.dst);
+          h.y = had ? operand(op.src) : ntt::Operand{nullptr, nullptr, 0};
+          h.out = sum ? nullptr : buffer(buf[op.dst]);
+          h.sums = d_sums;
+          h.stride = d;
+          h.m = m;
+          h.logN = logM;
+          h.prime0 = i;
+          SK_CK(ntt::had(h, d, np, num_sms(), st));
+          Slot z;
+          z.e_r = slot[op.dst].e_r + (had ? slot[op.src].e_r + 1 : 0);
+          z.e_m = slot[op.dst].e_m + (had ? slot[op.src].e_m : 0);
+          if (sum) {
+            e_r = z.e_r;
+            e_m = z.e_m;
+            break;   // the sum is the schedule's last step
+          }
+          slot[op.dst] = z;
+        }
+      }
     }
-    if (ps != SK_OK) return ps;
+    return SK_OK;
+  };
+  const sk_status status = run();
+  const cudaError_t ef = cudaFreeAsync(pool, st);
+  if (status != SK_OK) return status;
+  SK_CK(ef);
+  std::vector<unsigned long long> sums(nsum);
+  SK_CK(cudaMemcpyAsync(sums.data(), d_sums, nsum * 8, cudaMemcpyDeviceToHost, st));
+  SK_CK(cudaStreamSynchronize(st));
+  std::vector<uint32_t> res(nsum, 0u);
+  for (int i = 0; i < f.np; i++) {
+    const uint64_t p = fu_primes()[i].p;
+    const uint64_t fac = fu_powmod((1ull << 32) % p, (uint64_t)e_r, p) *
+                         fu_powmod(fu_width(i, M).minv_p, (uint64_t)e_m, p) % p;
+    for (int row = 0; row < d; row++)
+      res[(size_t)row * kFuMaxPrimes + i] = (uint32_t)(sums[(size_t)row * kFuMaxPrimes + i] % p * fac % p);
   }
-  SK_CK_ST(fu_finish(s, f, out, st));
+  SK_CK_ST(fu_fill(s, res.data(), f.np, out));
   *done = true;
   return SK_OK;
 }
@@ -2833,7 +2689,7 @@ sk_status fu_group_pass(const FuPrime& fp, int64_t M, const int64_t* const* d_ro
   k_fu_load_rows<PI><<<grid_for(nvec * M), 256, 0, st>>>(d_rows, nvec, ilog2(M), fp.r2, fp.r3, V);
   count_launch(2);
   SK_CK(cudaGetLastError());
-  sk_status fs = xform<MontOps<PI>>(V, W, nvec, M, tw, false, fw.r4, st);
+  sk_status fs = xform_small<MontOps<PI>>(V, W, nvec, M, tw, false, fw.r4, st);
   if (fs != SK_OK) return fs;
   k_fu_reduce_many<PI><<<nout * nchunk, 256, 0, st>>>(W, d_outs, M, nchunk, part);
   k_fu_final<PI><<<(nout + 63) / 64, 64, 0, st>>>(part, nout, nchunk, fw.minv, res, kFuMaxPrimes);

@@ -131,8 +131,26 @@ __device__ __forceinline__ void dft(uint32_t (&x)[1 << LOG], const uint32_t* w64
   for (int k = 0; k < N; k++) x[k] = y[k];
 }
 
-// Vectors of one launch: vector v is base[v / per] + (v % per) m (m int64 counters, taken as
-// zero from m to N); its direction (1: inverse root) is dirs[v] or bit v / per of negmask.
+// x[i] = L[i stride] for i < K, zero where i stride >= left; with fold, the circular value
+// L[i stride] + L[i stride + fold].
+template <int K>
+__device__ __forceinline__ void load_words(uint32_t (&x)[K], const uint32_t* L, int64_t stride, int64_t left,
+                                           int64_t fold, Mod q) {
+#pragma unroll
+  for (int i = 0; i < K; i++) x[i] = i * stride < left ? L[i * stride] : 0u;
+  if (fold) {
+    uint32_t y[K];
+#pragma unroll
+    for (int i = 0; i < K; i++) y[i] = i * stride < left ? L[i * stride + fold] : 0u;
+#pragma unroll
+    for (int i = 0; i < K; i++) x[i] = add(x[i], y[i], q);
+  }
+}
+
+// Vectors of one launch.  Counters: vector v is base[v / per] + (v % per) m, its direction (1:
+// inverse root) dirs[v] or bit v / per of negmask.  Words: vector v of the prime is the residues
+// at words + (prime stride + v) N, direction bit 0 of negmask.  Either is taken as zero from m on,
+// and words with fold != 0 as the circular sum of two of them (see load_words).
 struct ColArgs {
   const int64_t* const* base;
   int per;
@@ -144,6 +162,8 @@ struct ColArgs {
   int64_t stride;           // vectors per prime in V
   int prime0;               // prime of grid y = 0
   int nvec[kMaxPrimes];     // vectors of each prime (leading ones)
+  const uint32_t* words = nullptr;   // may be V: a CTA reads its columns before it writes them
+  int64_t fold = 0;
 };
 
 __device__ __forceinline__ int dir_of(const ColArgs& a, int64_t v) {
@@ -161,7 +181,10 @@ __device__ __forceinline__ uint32_t root_pow(int prime, int dir, int logR, uint3
 // exchange between the two levels and back to global memory.  LA = 0: R = B points per thread,
 // no exchange.  64-byte column segments are read and 32-byte ones written at least, so tiles
 // wider than eight columns would not save sectors.
-template <int LA, int LB>
+//
+// WORDS: residues instead of counters.  BACK: the inverse transform's column pass, on residues
+// that k_ntt_corr has multiplied by the inverse twiddle already.
+template <int LA, int LB, bool WORDS, bool BACK>
 __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __grid_constant__ ColArgs a) {
   constexpr int A = 1 << LA, B = 1 << LB, LR = LA + LB;
   constexpr int LCB = LA ? 8 - LA : 8, CB = 1 << LCB;
@@ -171,10 +194,11 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __gri
   const int n2 = (int)(blockIdx.x & ((1u << (kLogRow - LCB)) - 1u)) * CB + (int)(threadIdx.x & (CB - 1));
   const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
   const uint32_t r2 = c_prime[prime].r2;
-  const int dir = dir_of(a, vec);
+  const int dir = WORDS ? (int)(a.negmask & 1ull) : dir_of(a, vec);
   const uint32_t* w64 = c_prime[prime].w64[dir];
-  const int64_t* src = a.base[vec / a.per] + (vec % a.per) * a.m + n2;
-  uint32_t* dst = a.V + (((int64_t)blockIdx.y * a.stride + vec) << (LR + kLogRow)) + n2;
+  const int64_t at0 = (((int64_t)blockIdx.y * a.stride + vec) << (LR + kLogRow)) + n2;
+  const int64_t* src = WORDS ? nullptr : a.base[vec / a.per] + (vec % a.per) * a.m + n2;
+  uint32_t* dst = a.V + at0;
   const int64_t left = a.m - n2;   // counters of this column: rows n1 with 1024 n1 < left
   extern __shared__ uint32_t s_col[];
   const int c = (int)(threadIdx.x >> LCB);   // this thread's k1 residue at the second level
@@ -193,7 +217,8 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __gri
       const int b = (int)(threadIdx.x >> LCB) + A * s;
       uint32_t y[A];
       const int64_t at = (int64_t)b << kLogRow;
-      load_residues<A>(y, src + at, (int64_t)B << kLogRow, left - at, q, r2);
+      if (WORDS) load_words<A>(y, a.words + at0 + at, (int64_t)B << kLogRow, left - at, a.fold, q);
+      else load_residues<A>(y, src + at, (int64_t)B << kLogRow, left - at, q, r2);
       dft<LA>(y, w64, q);
 #pragma unroll
       for (int i = 0; i < A; i++) ex[(i * (B + 1) + b) * CB + v] = i ? mul(y[i], tw[i * B + b], q) : y[i];
@@ -202,12 +227,16 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __gri
 #pragma unroll
     for (int b = 0; b < B; b++) x[b] = ex[(c * (B + 1) + b) * CB + v];
   } else {
-    load_residues<B>(x, src, 1 << kLogRow, left, q, r2);
+    if (WORDS) load_words<B>(x, a.words + at0, 1 << kLogRow, left, a.fold, q);
+    else load_residues<B>(x, src, 1 << kLogRow, left, q, r2);
   }
   dft<LB>(x, w64, q);
   // x[e] is row k1 = c + A e: times w_N^(n2 k1), advanced in two chains of step w_N^(2 A n2)
-  if constexpr (LR > 0) {
-    const uint32_t k0 = LA ? (uint32_t)c : 0u;
+  const uint32_t k0 = LA ? (uint32_t)c : 0u;
+  if constexpr (BACK) {
+#pragma unroll
+    for (int e = 0; e < B; e++) dst[(int64_t)(k0 + A * e) << kLogRow] = x[e];
+  } else if constexpr (LR > 0) {
     uint32_t w0 = root_pow(prime, dir, LR, (uint32_t)n2 * k0, q);
     const uint32_t st = root_pow(prime, dir, LR, (uint32_t)n2 * A, q);
     uint32_t w1 = mul(w0, st, q);
@@ -318,33 +347,188 @@ __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ Row
   }
 }
 
-template <int LA, int LB>
-cudaError_t launch_cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
-  constexpr int LCB = LA ? 8 - LA : 8;
-  const size_t smem = LA ? ((size_t)(1 << (LA + LB)) + ((size_t)(1 << LA) * ((1 << LB) + 1) << LCB)) * 4 : 0;
-  const cudaError_t e = fit_dynamic_smem((const void*)k_ntt_cols<LA, LB>, smem);
+// One correlation of the step-by-step schedule, between the column passes: rows k1 of A (columns
+// transformed with the inverse root, so its entries are A(-nu)) and X, both transformed, multiplied
+// and transformed back in one warp's registers -- entry k2 = c + 32 e of a product is where the
+// inverse transform's first level wants it -- then times w_N^(-n2 k1) for k_ntt_cols<.., BACK>.
+// The result carries 2^-32 from the product and M from the missing 1 / M; the caller keeps track.
+struct CorrRowArgs {
+  const uint32_t *A, *X;   // [prime][stride][N]
+  uint32_t* Z;
+  int64_t stride;
+  int logR, prime0, nvec;
+};
+
+__global__ void __launch_bounds__(256, 2) k_ntt_corr(const __grid_constant__ CorrRowArgs a) {
+  __shared__ uint32_t s_tw[2][1024];
+  __shared__ uint32_t s_ex[8][32 * 33];
+  extern __shared__ uint32_t s_prod[];   // 8 x 1024
+  const int prime = a.prime0 + (int)blockIdx.y;
+  const int R = 1 << a.logR;
+  const int lcta = a.logR > 3 ? a.logR - 3 : 0;
+  const int64_t v = blockIdx.x >> lcta;
+  const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
+  const int k1 = (int)(blockIdx.x & ((1u << lcta) - 1u)) * 8 + warp;
+  const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
+  for (int i = threadIdx.x; i < 2048; i += 256) ((uint32_t*)s_tw)[i] = ((const uint32_t*)g_row[prime])[i];
+  __syncthreads();
+  if (k1 >= R) return;
+  const int64_t at = (((int64_t)blockIdx.y * a.stride + v) << (a.logR + kLogRow)) + ((int64_t)k1 << kLogRow) + lane;
+  uint32_t* ex = s_ex[warp];
+  uint32_t* prod = s_prod + warp * 1024 + lane;
+  uint32_t x[32], y[32];
+#pragma unroll
+  for (int i = 0; i < 32; i++) x[i] = __ldcs(a.A + at + 32 * i);
+  // A with the inverse root, X, then the product with the inverse root
+#pragma unroll 1
+  for (int step = 0; step < 3; step++) {
+    const int dir = step == 1 ? 0 : 1;
+    const uint32_t* w64 = c_prime[prime].w64[dir];
+    const uint32_t* tw = s_tw[dir];
+    dft<5>(x, w64, q);
+#pragma unroll
+    for (int i = 0; i < 32; i++) ex[i * 33 + lane] = i ? mul(x[i], tw[i * 32 + lane], q) : x[i];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 32; i++) y[i] = ex[lane * 33 + i];
+    __syncwarp();
+    if (step == 0) {
+#pragma unroll
+      for (int i = 0; i < 32; i++) x[i] = __ldcs(a.X + at + 32 * i);
+    }
+    dft<5>(y, w64, q);
+    if (step == 0) {
+#pragma unroll
+      for (int i = 0; i < 32; i++) prod[32 * i] = y[i];
+    } else if (step == 1) {
+#pragma unroll
+      for (int i = 0; i < 32; i++) x[i] = mul(prod[32 * i], y[i], q);
+    }
+  }
+  // y[e] is column n2 = lane + 32 e
+  uint32_t w0 = root_pow(prime, 1, a.logR, (uint32_t)k1 * (uint32_t)lane, q);
+  const uint32_t st = root_pow(prime, 1, a.logR, (uint32_t)k1 * 32u, q);
+  uint32_t w1 = mul(w0, st, q);
+  const uint32_t st2 = mul(st, st, q);
+#pragma unroll
+  for (int e = 0; e < 32; e += 2) {
+    a.Z[at + 32 * e] = mul(y[e], w0, q);
+    a.Z[at + 32 * (e + 1)] = mul(y[e + 1], w1, q);
+    w0 = mul(w0, st2, q);
+    w1 = mul(w1, st2, q);
+  }
+}
+
+// A vector operand of the schedule's elementwise steps: row v's counters c + v m, or its residues
+// u + (prime stride + v) N, circular (fold) or not; m entries either way.
+struct Operand {
+  const int64_t* c;
+  const uint32_t* u;
+  int64_t fold;
+};
+
+struct HadArgs {
+  Operand x, y;               // y.c and y.u null: x alone (the plain sum)
+  uint32_t* out;              // [prime][stride][N] products x y 2^-32; nullptr: only their sums
+  unsigned long long* sums;   // [row][kMaxPrimes]
+  int64_t stride, m;
+  int logN, prime0;
+};
+
+__device__ __forceinline__ uint32_t operand_at(const Operand& o, int64_t at, int64_t row, int64_t m, int64_t j, Mod q,
+                                               uint32_t r2) {
+  if (o.c) {
+    const int64_t c = __ldg(o.c + row * m + j);
+    if ((uint64_t)(c + (1ll << 30)) < (1ull << 31)) return min((uint32_t)c, (uint32_t)c + q.p);
+    return residue(c, q, r2);
+  }
+  const uint32_t v = o.u[at + j];
+  return o.fold ? add(v, o.u[at + j + o.fold], q) : v;
+}
+
+// grid (chunks, rows, primes), 256 threads
+__global__ void __launch_bounds__(256) k_ntt_had(const __grid_constant__ HadArgs a) {
+  __shared__ unsigned long long s_sum[8];
+  const int prime = a.prime0 + (int)blockIdx.z;
+  const int64_t row = blockIdx.y;
+  const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
+  const uint32_t r2 = c_prime[prime].r2;
+  const int64_t at = ((int64_t)blockIdx.z * a.stride + row) << a.logN;
+  const bool two = a.y.c || a.y.u;
+  unsigned long long sum = 0;
+  for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < a.m; j += (int64_t)gridDim.x * 256) {
+    uint32_t v = operand_at(a.x, at, row, a.m, j, q, r2);
+    if (two) v = mul(v, operand_at(a.y, at, row, a.m, j, q, r2), q);
+    if (a.out) a.out[at + j] = v;
+    else sum += v;
+  }
+  if (a.out) return;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, s);
+  if ((threadIdx.x & 31u) == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) sum += s_sum[w];
+    atomicAdd(a.sums + row * kMaxPrimes + prime, sum);
+  }
+}
+
+inline cudaError_t corr_rows(const CorrRowArgs& a, int primes, cudaStream_t st) {
+  const int lcta = a.logR > 3 ? a.logR - 3 : 0;
+  constexpr size_t smem = 8 * 1024 * sizeof(uint32_t);
+  const cudaError_t e = allow_dynamic_smem((const void*)k_ntt_corr);
   if (e != cudaSuccess) return e;
-  k_ntt_cols<LA, LB><<<dim3((unsigned)(nvec << (kLogRow - LCB)), (unsigned)primes), 256, smem, st>>>(a);
+  k_ntt_corr<<<dim3((unsigned)((int64_t)a.nvec << lcta), (unsigned)primes), 256, smem, st>>>(a);
   count_launch();
   return cudaGetLastError();
 }
 
-inline cudaError_t cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+inline cudaError_t had(const HadArgs& a, int rows, int primes, int sms, cudaStream_t st) {
+  // about four waves of CTAs of at least 1024 entries
+  const int64_t want = (4ll * 8 * sms + (int64_t)rows * primes - 1) / ((int64_t)rows * primes);
+  const int64_t most = (a.m + 1023) / 1024;
+  k_ntt_had<<<dim3((unsigned)(want < most ? want : most), (unsigned)rows, (unsigned)primes), 256, 0, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <int LA, int LB, bool WORDS, bool BACK>
+cudaError_t launch_cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+  constexpr int LCB = LA ? 8 - LA : 8;
+  const size_t smem = LA ? ((size_t)(1 << (LA + LB)) + ((size_t)(1 << LA) * ((1 << LB) + 1) << LCB)) * 4 : 0;
+  const cudaError_t e = fit_dynamic_smem((const void*)k_ntt_cols<LA, LB, WORDS, BACK>, smem);
+  if (e != cudaSuccess) return e;
+  k_ntt_cols<LA, LB, WORDS, BACK>
+      <<<dim3((unsigned)(nvec << (kLogRow - LCB)), (unsigned)primes), 256, smem, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <bool WORDS, bool BACK>
+cudaError_t cols_of(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
   switch (a.logR) {
-    case 0: return launch_cols<0, 0>(a, nvec, primes, st);
-    case 1: return launch_cols<0, 1>(a, nvec, primes, st);
-    case 2: return launch_cols<0, 2>(a, nvec, primes, st);
-    case 3: return launch_cols<0, 3>(a, nvec, primes, st);
-    case 4: return launch_cols<0, 4>(a, nvec, primes, st);
-    case 5: return launch_cols<0, 5>(a, nvec, primes, st);
-    case 6: return launch_cols<3, 3>(a, nvec, primes, st);
-    case 7: return launch_cols<3, 4>(a, nvec, primes, st);
-    case 8: return launch_cols<4, 4>(a, nvec, primes, st);
-    case 9: return launch_cols<4, 5>(a, nvec, primes, st);
-    case 10: return launch_cols<5, 5>(a, nvec, primes, st);
-    case 11: return launch_cols<5, 6>(a, nvec, primes, st);
-    default: return launch_cols<6, 6>(a, nvec, primes, st);
+    case 0: return launch_cols<0, 0, WORDS, BACK>(a, nvec, primes, st);
+    case 1: return launch_cols<0, 1, WORDS, BACK>(a, nvec, primes, st);
+    case 2: return launch_cols<0, 2, WORDS, BACK>(a, nvec, primes, st);
+    case 3: return launch_cols<0, 3, WORDS, BACK>(a, nvec, primes, st);
+    case 4: return launch_cols<0, 4, WORDS, BACK>(a, nvec, primes, st);
+    case 5: return launch_cols<0, 5, WORDS, BACK>(a, nvec, primes, st);
+    case 6: return launch_cols<3, 3, WORDS, BACK>(a, nvec, primes, st);
+    case 7: return launch_cols<3, 4, WORDS, BACK>(a, nvec, primes, st);
+    case 8: return launch_cols<4, 4, WORDS, BACK>(a, nvec, primes, st);
+    case 9: return launch_cols<4, 5, WORDS, BACK>(a, nvec, primes, st);
+    case 10: return launch_cols<5, 5, WORDS, BACK>(a, nvec, primes, st);
+    case 11: return launch_cols<5, 6, WORDS, BACK>(a, nvec, primes, st);
+    default: return launch_cols<6, 6, WORDS, BACK>(a, nvec, primes, st);
   }
+}
+
+inline cudaError_t cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+  return a.words ? cols_of<true, false>(a, nvec, primes, st) : cols_of<false, false>(a, nvec, primes, st);
+}
+
+inline cudaError_t cols_back(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+  return cols_of<true, true>(a, nvec, primes, st);
 }
 
 inline cudaError_t rows(const RowArgs& a, int64_t nout, int primes, cudaStream_t st) {

@@ -64,3 +64,23 @@ def test_many_sets_equal_single(logms):
         s.set_estimator("ntt")
         assert s.estimate()["rows"] == e["rows"]
     assert np.all([e["retries"] == 0 for e in many])
+
+
+_SHARED = ([1, 2, 1, 1], [(0, 0, 1, 0), (2, 0, 1, 0), (3, 0, 1, 1)])   # three relations share an attribute
+
+
+@pytest.mark.parametrize("m", [2, 3, 127, 512, 513, 1000, 1024, 1025, 2048, 5000, 16384, 20_001, 65_536, 100_000,
+                               131_073, 524_288, 1_000_000, 1 << 22])
+@pytest.mark.parametrize("query", [_SHARED, _chain(2), _chain(3), _chain(5), _star(4)])
+def test_schedule_equals_stepwise(m, query, monkeypatch):
+    """Widths that are no power of two and shared attributes: the schedule modulo the primes."""
+    if query is not _SHARED and (m & (m - 1)) == 0:
+        pytest.skip("a product of spectra")
+    d = 5 if m < 100_000 else 2
+    s = sk.SketchSet(*query, m, d, 7)
+    _fill(s, m % 1000 + len(query[0]), 20)
+    got = s.estimate()
+    assert got["max_limbs"] < 9 and got["limb_bits"] == 0   # CRT primes, not limbs
+    s.set_estimator("ntt")
+    assert s.estimate()["rows"] == got["rows"]
+    s.close()
