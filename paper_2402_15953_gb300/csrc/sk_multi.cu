@@ -32,6 +32,7 @@ constexpr int kMaxMultiAttrs = 5;   // joined attributes per relation in a batch
 struct MultiItem {
   UpdArgs args;
   int64_t chunk0;   // first global chunk of this item
+  int64_t chunk;    // tuples per chunk
   int pow2;
   int use_smem;     // 0 global counters, 1 int32 shared sub-sketch, 2 packed 16-bit one
   int deg1;         // every attribute in exactly one join
@@ -66,6 +67,10 @@ __device__ __forceinline__ void multi_chunk(const UpdArgs& p, int use_smem, cons
       if (lo != 0) red_add_global(p.ctr + 2 * k, (unsigned long long)(int64_t)lo);
       if (hi != 0 && 2 * k + 1 < dm) red_add_global(p.ctr + 2 * k + 1, (unsigned long long)(int64_t)hi);
     }
+  } else if constexpr (A == 1) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = t0 + (threadIdx.x - lane); b < t1; b += blockDim.x)
+      update_warp_key<POW2, DEG1>(p, s_coef, b + lane, b + lane < t1);
   } else {
     for (int64_t i = t0 + threadIdx.x; i < t1; i += blockDim.x)
       update_tuple<A, POW2, false, false, DEG1>(p, s_coef, s_sub, i);
@@ -85,7 +90,7 @@ __device__ __forceinline__ void multi_dispatch(const UpdArgs& p, int use_smem, c
 }
 
 __global__ void __launch_bounds__(256, 4) k_update_multi(const MultiItem* __restrict__ items, int n_items, int64_t total_chunks,
-                               int64_t chunk, int coef_words, unsigned long long* queue) {
+                               int coef_words, unsigned long long* queue) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int64_t s_c;
   __shared__ int s_item;
@@ -127,8 +132,8 @@ __global__ void __launch_bounds__(256, 4) k_update_multi(const MultiItem* __rest
       __syncthreads();
     }
     const UpdArgs& p = s_args;
-    const int64_t t0 = (c - items[it].chunk0) * chunk;
-    const int64_t t1 = min(p.n, t0 + chunk);
+    const int64_t t0 = (c - items[it].chunk0) * items[it].chunk;
+    const int64_t t1 = min(p.n, t0 + items[it].chunk);
     if (s_pow2) {
       if (s_deg1) multi_dispatch<true, true>(p, s_smem, s_coef, s_sub, t0, t1);
       else multi_dispatch<true, false>(p, s_smem, s_coef, s_sub, t0, t1);
@@ -171,6 +176,17 @@ int sms() {
   return n;
 }
 
+// Tuples per chunk of an item, at most cfg's: about 32 chunks per SM over all items, so that the
+// last chunks do not leave most SMs idle (at 32768 tuples 96 relations of 2.2e7 tuples made 714
+// chunks for 456 resident CTAs) and a small batch spreads over the GPU; at least 2048 tuples (a
+// chunk's start costs about as much as 200), and for shared sub-sketches four tuples per counter
+// of a row, so that flushing d m counters stays below the d updates of each tuple.
+int64_t multi_chunk_tuples(int64_t tuples, int64_t m, bool smem, int64_t most) {
+  const int64_t want = (tuples / (32 * (int64_t)sms()) + 255) / 256 * 256;
+  const int64_t least = smem ? std::max<int64_t>(2048, 4 * m) : 2048;
+  return std::max<int64_t>(1, std::min<int64_t>(most, std::max<int64_t>(least, want)));
+}
+
 }  // namespace
 
 size_t multi_item_size() { return sizeof(MultiItem); }
@@ -181,6 +197,8 @@ sk_status multi_describe(const sk_update_item* items, int n, const sk_update_pla
   int64_t chunk0 = 0;
   int coef_words = 0;
   int64_t sub_words = 0;
+  int64_t tuples = 0;
+  for (int i = 0; i < n; i++) tuples += items[i].n_rows;
   for (int i = 0; i < n; i++) {
     const sk_update_item& it = items[i];
     sk_set* s = it.set;
@@ -214,11 +232,12 @@ sk_status multi_describe(const sk_update_item* items, int n, const sk_update_pla
                         dm * 2 <= 160 * 1024;
     mi.use_smem = fits32 ? 1 : (fits16 ? 2 : 0);
     a.s16 = mi.use_smem == 2 ? 1 : 0;
+    mi.chunk = multi_chunk_tuples(tuples, s->m, mi.use_smem != 0, cfg.chunk_tuples);
     // |Delta| below which a tuple goes to the sub-sketch: a chunk's sum per counter then
     // stays within int32 (1) or within +-32767 (2, the 16-bit halves never carry)
-    a.smem_wmax = (int64_t)(mi.use_smem == 2 ? 0x7fff : 0x7fffffff) / std::max<int64_t>(cfg.chunk_tuples, 1);
+    a.smem_wmax = (int64_t)(mi.use_smem == 2 ? 0x7fff : 0x7fffffff) / mi.chunk;
     mi.chunk0 = chunk0;
-    chunk0 += (it.n_rows + cfg.chunk_tuples - 1) / cfg.chunk_tuples;
+    chunk0 += (it.n_rows + mi.chunk - 1) / mi.chunk;
     coef_words = std::max(coef_words, s->d * rp.coef_row_len);
     if (mi.use_smem) sub_words = std::max(sub_words, mi.use_smem == 1 ? dm : (dm + 1) / 2);
     out[i] = mi;
@@ -238,8 +257,8 @@ sk_status multi_launch(const void* d_desc, int n, int64_t total_chunks, const sk
   e = allow_dynamic_smem((const void*)k_update_multi);
   if (e != cudaSuccess) return set_status_from_cuda(e);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(total_chunks, (int64_t)sms() * cfg.ctas_per_sm));
-  k_update_multi<<<grid, cfg.threads, smem_bytes, st>>>((const MultiItem*)d_desc, n, total_chunks, cfg.chunk_tuples,
-                                                        coef_words, d_queue);
+  k_update_multi<<<grid, cfg.threads, smem_bytes, st>>>((const MultiItem*)d_desc, n, total_chunks, coef_words,
+                                                        d_queue);
   count_launch();
   return set_status_from_cuda(cudaGetLastError());
 }

@@ -31,7 +31,8 @@ using namespace dev;
 
 
 template <int A, bool POW2, bool SMEM, bool DEG1>
-__global__ void __launch_bounds__(256) k_update(UpdArgs p) {
+__global__ void __launch_bounds__(256) k_update(UpdArgs p, const int* unless) {
+  if (unless && *unless) return;   // another path has the batch (see update_undeclared)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* s_coef = (uint64_t*)smem_raw;
   const int ncoef = p.d * p.row_len;
@@ -43,6 +44,12 @@ __global__ void __launch_bounds__(256) k_update(UpdArgs p) {
   __syncthreads();
 
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  if constexpr (A == 1 && !SMEM) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x - lane); b < p.n; b += step)
+      update_warp_key<POW2, DEG1>(p, s_coef, b + lane, b + lane < p.n);
+    return;
+  }
   if (SMEM && p.agg) {
     // warp-uniform loop: every lane of a warp runs the same iterations (collectives inside)
     const int lane = threadIdx.x & 31;
@@ -149,6 +156,7 @@ struct PartArgs {
   const uint32_t* vbits;         // nullptr, or bit (i mod 32) of word i / 32: window tuple i is kept
   const int64_t* wts;            // weighted: Delta of the window's first tuple (items are uint32_t)
   int64_t wmax;                  // weighted: |Delta| <= wmax < 2^16 goes into an item
+  const int* go;                 // nullptr, or both phases return at once when it reads 0
 };
 
 __device__ __forceinline__ uint64_t policy_evict_first() {
@@ -202,6 +210,13 @@ __global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t) {
   }
 }
 
+// The largest key of each attribute of a batch whose domains were not declared.
+struct FoundDomains {
+  unsigned long long top[5];
+  int go;        // every key is dense enough for the tables
+  int blocks;    // CTAs of the scan that are done
+};
+
 // Key-table records of 24 bytes (d <= 9, one thread per domain key): rows 3w .. 3w + 2 in
 // 64-bit word w (w = 0, 1, 2), row r's lane at bit 22 (r mod 3): its bin (below 2^16) in the
 // lane's bits 0..15 and its sign bit at lane bit 19.  Summing A <= 5 records word by word in
@@ -215,18 +230,30 @@ __global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t) {
 // the first 8 bytes hold word 2 and the aligned pair after it words 0 and 1, so a reader
 // always takes words 0 and 1 with one 16-byte load and word 2 with one 8-byte load.
 template <bool DEG1>
-__global__ void __launch_bounds__(256) k_key_table_l24(UpdArgs p, TabArgs t) {
+__global__ void __launch_bounds__(256) k_key_table_l24(UpdArgs p, TabArgs t, const FoundDomains* found) {
+  if (found && !found->go) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* s_coef = (uint64_t*)smem_raw;
   const int ncoef = p.d * p.row_len;
   for (int i = threadIdx.x; i < ncoef; i += blockDim.x) s_coef[i] = p.coef[i];
   __syncthreads();
-  const int64_t total = t.base[p.a];
+  // keys to hash: every declared domain, or [0, largest key] of each attribute as found
+  int64_t total = t.base[p.a];
+  if (found) {
+    total = 0;
+    for (int u = 0; u < p.a; u++) total += (int64_t)found->top[u] + 1;
+  }
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   uint64_t* tbl = (uint64_t*)t.tbl;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
     int u = 0;
-    while (u + 1 < p.a && g >= t.base[u + 1]) u++;
+    int64_t g = i;
+    if (found) {
+      while (g > (int64_t)found->top[u]) g -= (int64_t)found->top[u++] + 1;
+      g += t.base[u];
+    } else {
+      while (u + 1 < p.a && g >= t.base[u + 1]) u++;
+    }
     const uint32_t x = (uint32_t)(g - t.base[u]);
     const uint64_t* cr = s_coef + t.off[u];
     uint64_t lane[3] = {0, 0, 0};
@@ -280,6 +307,7 @@ __device__ __forceinline__ void ld_record24(const uint64_t* tbl, uint64_t k, uin
 // sign above; a tuple with |Delta| > wmax goes to the int64 counters directly.
 template <int A, int FMT, bool WT>
 __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, PartArgs q) {
+  if (q.go && !*q.go) return;
   using Item = typename std::conditional<WT, uint32_t, uint16_t>::type;
   constexpr bool HELD = WT && FMT != 1;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
@@ -505,6 +533,7 @@ template <bool WT>
 __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long long* ctr, int64_t m, int d,
                                                      int logL, int R, int logP) {
   constexpr int LI = WT ? 2 : 3, I = 1 << LI;   // items per 16-byte chunk
+  if (q.go && !*q.go) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int* cnt = (int*)smem_raw;
   const int S = (int)(m >> logL);
@@ -722,6 +751,13 @@ int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps)
 // width, rows, arity and weights it accepts, whatever the sketch's size and the batch length.
 // SK_PART_WINDOW caps the tuples per window (default and largest: 2^30, which keeps every
 // shared-memory counter of k_part_accum below 2^31 in magnitude; 2^24 for the wide update).
+// SK_UNDECLARED_LEAST: the fewest tuples for which update_undeclared looks for dense keys.
+int64_t undeclared_least() {
+  const char* v = std::getenv("SK_UNDECLARED_LEAST");
+  const long long x = v ? std::atoll(v) : 0;
+  return x > 0 ? (int64_t)x : (int64_t)1 << 22;
+}
+
 int part_update_mode() {
   const char* v = std::getenv("SK_PART_UPDATE");
   return (v && v[0] == '0') ? 0 : ((v && v[0] == '2') ? 2 : 1);
@@ -733,12 +769,16 @@ int part_record_bytes() {
   return (v && std::atoi(v) == 32) ? 32 : 24;
 }
 
-int64_t part_window(int64_t n) {
+int64_t part_window(int64_t n, int64_t most = (int64_t)1 << 30) {
   const char* v = std::getenv("SK_PART_WINDOW");
   const long long x = v ? std::atoll(v) : 0;
-  const int64_t cap = (x > 0 && x < (1ll << 30)) ? (int64_t)x : ((int64_t)1 << 30);
+  const int64_t cap = (x > 0 && x < most) ? (int64_t)x : most;
   return std::min<int64_t>((n + 255) / 256 * 256, (cap + 255) / 256 * 256);
 }
+
+// Tuples per window: weighted items take twice the bytes, and staging beyond what the library's
+// pool keeps (4 GiB) would be mapped again for every call.
+int64_t part_most(const int64_t* weights) { return (int64_t)1 << (weights ? 26 : 30); }
 
 // Regions of a window of W tuples: the phase-1 grid has at most sms x kPartMaxCtasPerSm CTAs
 // of 256 threads, so its warps' regions hold at most W + that many threads' tiles per row.
@@ -777,9 +817,10 @@ PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps) {
 // Both phases over every window of the batch; staging (part_staging_bytes) is caller-owned.
 // colp: the first tuple's key of each of the a.a attributes (nullptr: a.cols + u a.stride).
 // vbits: nullptr, or one bit per batch tuple (bit i mod 32 of word i / 32) that must be set
-// for the tuple to be added.
+// for the tuple to be added.  most: tuples per window at most.  go: see PartArgs.
 cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* staging, int sms, cudaStream_t st,
-                            const int64_t* const* colp = nullptr, const uint32_t* vbits = nullptr) {
+                            const int64_t* const* colp = nullptr, const uint32_t* vbits = nullptr,
+                            int64_t most = (int64_t)1 << 30, const int* go = nullptr) {
   const int64_t n = a.n;
   const bool weighted = a.w != nullptr;
   TabItemsKernel items = tab_items_kernel(a.a, fmt, weighted);
@@ -788,8 +829,9 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
   cudaError_t e = tab_items_per_sm(items, &tab_per_sm);
   if (e != cudaSuccess) return e;
   const int64_t full_grid = (int64_t)sms * tab_per_sm;
-  const int64_t W = part_window(n);
+  const int64_t W = part_window(n, most);
   PartArgs q;
+  q.go = go;
   q.items = staging;
   q.cnts = (uint32_t*)((char*)staging + part_items_bytes(a.d, W, sms, weighted));
   q.W = W;
@@ -1627,12 +1669,21 @@ cudaError_t dispatch_tab(const UpdArgs& a, const TabArgs& t, int grid, size_t sm
   }
 }
 
+int sm_count() {
+  static const int n = [] {   // thread-safe one-time initialisation
+    int dev = 0, x = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&x, cudaDevAttrMultiProcessorCount, dev);
+    return x > 0 ? x : 1;
+  }();
+  return n;
+}
+
 // CTAs per SM of the global-atomic update grid.  Default: one tuple per thread (a grid of
 // n / 256 CTAs), which measured fastest on the 1e8-row star fact table (12.18 ms, against
 // 13.01 / 12.80 / 12.45 / 12.28 ms for 6 / 8 / 16 / 32 grid-stride CTAs per SM);
 // SK_UPDATE_GRID=<n> caps the grid at n CTAs per SM instead.
-int update_grid_per_sm(int resident) {
-  (void)resident;
+int update_grid_per_sm() {
   const char* v = std::getenv("SK_UPDATE_GRID");
   const int x = v ? std::atoi(v) : 0;
   return x <= 0 ? (1 << 30) / 64 : x;
@@ -1648,36 +1699,29 @@ bool all_deg1(const UpdArgs& a) {
 
 // grid <= 0 sizes the grid with update_grid_per_sm.
 template <int A, bool POW2, bool SMEM>
-cudaError_t launch_one(const UpdArgs& a, int grid, size_t smem, cudaStream_t st) {
+cudaError_t launch_one(const UpdArgs& a, int grid, size_t smem, cudaStream_t st, const int* unless) {
   auto kern = (A > 0 && all_deg1(a)) ? k_update<A, POW2, SMEM, (A > 0)> : k_update<A, POW2, SMEM, false>;
-  cudaError_t e = allow_dynamic_smem((const void*)kern);
+  cudaError_t e = fit_dynamic_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   if (grid <= 0) {
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t want = (a.n + 255) / 256;
-    const int mult = update_grid_per_sm(std::max(1, per_sm));
-    const int64_t cap = std::min<int64_t>((int64_t)mult * std::max(1, sms), 0x7fffffff);
+    const int64_t cap = std::min<int64_t>((int64_t)update_grid_per_sm() * sm_count(), 0x7fffffff);
     grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
   }
-  kern<<<grid, 256, smem, st>>>(a);
+  kern<<<grid, 256, smem, st>>>(a, unless);
   count_launch();
   return cudaGetLastError();
 }
 
 template <bool POW2, bool SMEM>
-cudaError_t dispatch_a(const UpdArgs& a, int grid, size_t smem, cudaStream_t st) {
+cudaError_t dispatch_a(const UpdArgs& a, int grid, size_t smem, cudaStream_t st, const int* unless = nullptr) {
   switch (a.a) {
-    case 1: return launch_one<1, POW2, SMEM>(a, grid, smem, st);
-    case 2: return launch_one<2, POW2, SMEM>(a, grid, smem, st);
-    case 3: return launch_one<3, POW2, SMEM>(a, grid, smem, st);
-    case 4: return launch_one<4, POW2, SMEM>(a, grid, smem, st);
-    case 5: return launch_one<5, POW2, SMEM>(a, grid, smem, st);
-    default: return launch_one<0, POW2, SMEM>(a, grid, smem, st);
+    case 1: return launch_one<1, POW2, SMEM>(a, grid, smem, st, unless);
+    case 2: return launch_one<2, POW2, SMEM>(a, grid, smem, st, unless);
+    case 3: return launch_one<3, POW2, SMEM>(a, grid, smem, st, unless);
+    case 4: return launch_one<4, POW2, SMEM>(a, grid, smem, st, unless);
+    case 5: return launch_one<5, POW2, SMEM>(a, grid, smem, st, unless);
+    default: return launch_one<0, POW2, SMEM>(a, grid, smem, st, unless);
   }
 }
 
@@ -1928,14 +1972,144 @@ size_t key_table_max_bytes() {
   return (size_t)(x < 0 ? 0 : x) << 20;
 }
 
-int sm_count() {
-  static const int n = [] {   // thread-safe one-time initialisation
-    int dev = 0, x = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&x, cudaDevAttrMultiProcessorCount, dev);
-    return x > 0 ? x : 1;
-  }();
-  return n;
+// 24-byte key records of the declared domains, or of the found ones.
+cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDomains* found, int grid, cudaStream_t st) {
+  auto kern = all_deg1(a) ? k_key_table_l24<true> : k_key_table_l24<false>;
+  const size_t smem = (size_t)a.d * a.row_len * sizeof(uint64_t);
+  const cudaError_t e = fit_dynamic_smem((const void*)kern, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, 256, smem, st>>>(a, t, found);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Batches whose domains were not declared.  Hashing every tuple costs 36 a Horner steps for nine
+// rows; most key columns are dense codes, for which the tables serve as well as declared
+// domains do, but only the data tells.  So, without the host waiting for it: k_dom_probe looks at
+// 1024 tuples (sparse keys are seen there, and the scan is spared); k_dom_scan finds each column's
+// largest key; and either the tables and both phases of the partitioned update run, when every
+// key is below cap records per attribute, or the per-tuple update does: the kernels of the other
+// way return at once on the flag.  Counters are the same either way.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, uint64_t cap) {
+  const int64_t i = p.n / 1024 * threadIdx.x;
+  bool dense = true;
+  for (int u = 0; u < p.a; u++) dense = dense && (uint64_t)p.cols[(int64_t)u * p.stride + i] < cap;
+  dense = __syncthreads_and(dense);
+  if (threadIdx.x < 5) f->top[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    f->go = dense ? 1 : 0;
+    f->blocks = 0;
+  }
+}
+
+template <int A>
+__global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, uint64_t cap) {
+  __shared__ unsigned long long s_top[A];
+  if (!f->go) return;
+  if (threadIdx.x < A) s_top[threadIdx.x] = 0;
+  __syncthreads();
+  uint64_t top[A];
+#pragma unroll
+  for (int u = 0; u < A; u++) top[u] = 0;
+  const int64_t step = (int64_t)gridDim.x * 256;
+  constexpr int U = 4;   // tuples in flight per thread
+  for (int64_t i0 = (int64_t)blockIdx.x * 256 + threadIdx.x; i0 < p.n; i0 += U * step) {
+    uint64_t k[U][A];
+#pragma unroll
+    for (int t = 0; t < U; t++)
+#pragma unroll
+      for (int u = 0; u < A; u++)
+        k[t][u] = i0 + t * step < p.n ? (uint64_t)ld_key_stream(p.cols + (int64_t)u * p.stride + i0 + t * step) : 0ull;
+#pragma unroll
+    for (int t = 0; t < U; t++)
+#pragma unroll
+      for (int u = 0; u < A; u++) top[u] = k[t][u] > top[u] ? k[t][u] : top[u];
+  }
+#pragma unroll
+  for (int u = 0; u < A; u++) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint64_t v = __shfl_xor_sync(0xffffffffu, top[u], o);
+      top[u] = v > top[u] ? v : top[u];
+    }
+    if ((threadIdx.x & 31u) == 0) atomicMax(&s_top[u], (unsigned long long)top[u]);
+  }
+  __syncthreads();
+  if (threadIdx.x < A) {
+    atomicMax(&f->top[threadIdx.x], s_top[threadIdx.x]);
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(&f->blocks, 1) == (int)gridDim.x - 1) {   // the last CTA decides
+    __threadfence();
+    bool dense = true;
+    for (int u = 0; u < A; u++) dense = dense && *(volatile unsigned long long*)&f->top[u] < cap;
+    f->go = dense ? 1 : 0;
+  }
+}
+
+// *done = false (nothing launched) unless the batch is one the partitioned update would take with
+// declared domains, of two attributes or more and at least 2^22 tuples.  Five columns, m = 2^16,
+// d = 9: dense keys 254 against 458 us at 2^22 tuples and 670 against 1810 at 2^24 (1e7
+// tuples 1080 -> 538 us); sparse keys, which pay for the kernels that
+// return, 961 against 938 and 3745 against 3730.  One attribute is left to update_warp_key.
+// Captured streams keep the per-tuple update, which allocates nothing.
+cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int sms, cudaStream_t st, bool* done) {
+  *done = false;
+  const int64_t n = a0.n;
+  if (part_update_mode() == 0 || key_table_mode() == 0 || a0.has_dom || !pow2 || use_smem || a0.a < 2 || a0.a > 5 ||
+      a0.d > 9 || a0.m < 1024 || a0.m > 65536 || n < std::max<int64_t>((int64_t)a0.m * 16, undeclared_least()))
+    return cudaSuccess;
+  cudaStreamCaptureStatus cap_st = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap_st);
+  if (e != cudaSuccess || cap_st != cudaStreamCaptureStatusNone) return e;
+  // records per attribute: a quarter of the tuples (the rule for declared domains), within the
+  // tables' limit
+  const int64_t cap = std::min<int64_t>(n / 4, (int64_t)(key_table_max_bytes() / 24) / a0.a);
+  if (cap < 1) return cudaSuccess;
+  const int64_t W = part_window(n, (int64_t)1 << 26);
+  const size_t b_part = part_staging_bytes(a0.d, W, sms, a0.w != nullptr), b_tab = ((size_t)a0.a * cap * 24 + 255) & ~(size_t)255;
+  char* buf = nullptr;
+  if (pool_malloc_async((void**)&buf, b_part + b_tab + 256, st) != cudaSuccess) {
+    cudaGetLastError();   // no room: hash per tuple
+    return cudaSuccess;
+  }
+  *done = true;
+  FoundDomains* f = (FoundDomains*)(buf + b_part + b_tab);
+  UpdArgs a = a0;
+  TabArgs t;
+  int off = 0;
+  for (int u = 0; u < a.a; u++) {
+    a.dom[u] = cap;
+    t.base[u] = u * cap;
+    t.off[u] = off;
+    off += 2 + 4 * a.deg[u];
+  }
+  t.base[a.a] = a.a * cap;
+  t.rvec = 2;
+  t.narrow = 1;
+  t.tbl = (uint32_t*)(buf + b_part);
+  k_dom_probe<<<1, 1024, 0, st>>>(a, f, (uint64_t)cap);
+  const int grid = sms * 8;
+  switch (a.a) {
+    case 2: k_dom_scan<2><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
+    case 3: k_dom_scan<3><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
+    case 4: k_dom_scan<4><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
+    default: k_dom_scan<5><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
+  }
+  count_launch(2);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_table_l24(a, t, f, sms * 32, st);
+  if (e == cudaSuccess) e = run_partitioned(a, t, 2, buf, sms, st, nullptr, nullptr, (int64_t)1 << 26, &f->go);
+  // a fixed grid, whose CTAs return at once in the dense case: 1e7 dense tuples 538 us in all with
+  // 32 CTAs per SM, 552 with a tuple per thread; sparse ones measured the same
+  const size_t cb = (size_t)a0.d * a0.row_len * sizeof(uint64_t);
+  if (e == cudaSuccess)
+    e = dispatch_a<true, false>(a0, (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 32), cb, st, &f->go);
+  const cudaError_t ef = cudaFreeAsync(buf, st);
+  return e != cudaSuccess ? e : ef;
 }
 
 }  // namespace
@@ -2020,7 +2194,8 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     const bool sorted_parts = s->m <= ((int64_t)kSortMaxParts << 15);
     void* staging = nullptr;
     if (fits && worth && total > 0 && part) {
-      e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n), sms, weights != nullptr), st);
+      e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n, part_most(weights)), sms, weights != nullptr),
+                            st);
       if (e != cudaSuccess) {
         cudaGetLastError();   // no room for the planes: single-phase update
         staging = nullptr;
@@ -2051,20 +2226,22 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
         t.tbl = (uint32_t*)buf;
         a.smem_wmax = 0;
         const bool d1 = all_deg1(a);
-        auto kb = (part && part_fmt == 2)   ? (d1 ? k_key_table_l24<true> : k_key_table_l24<false>)
-                  : (part && part_fmt == 0) ? (d1 ? k_key_table_l20<true> : k_key_table_l20<false>)
-                  : pow2 ? (d1 ? k_key_table<true, true> : k_key_table<true, false>)
-                         : (d1 ? k_key_table<false, true> : k_key_table<false, false>);
-        e = cudaSuccess;
-        e = fit_dynamic_smem((const void*)kb, coef_bytes);
-        if (e == cudaSuccess) {
-          const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
-          kb<<<bgrid, 256, coef_bytes, st>>>(a, t);
-          count_launch();
-          e = cudaGetLastError();
+        const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
+        if (part && part_fmt == 2) {
+          e = launch_table_l24(a, t, nullptr, bgrid, st);
+        } else {
+          auto kb = (part && part_fmt == 0) ? (d1 ? k_key_table_l20<true> : k_key_table_l20<false>)
+                    : pow2 ? (d1 ? k_key_table<true, true> : k_key_table<true, false>)
+                           : (d1 ? k_key_table<false, true> : k_key_table<false, false>);
+          e = fit_dynamic_smem((const void*)kb, coef_bytes);
+          if (e == cudaSuccess) {
+            kb<<<bgrid, 256, coef_bytes, st>>>(a, t);
+            count_launch();
+            e = cudaGetLastError();
+          }
         }
         if (e == cudaSuccess && part) {
-          e = run_partitioned(a, t, part_fmt, staging, sms, st);
+          e = run_partitioned(a, t, part_fmt, staging, sms, st, nullptr, nullptr, part_most(weights));
         } else if (e == cudaSuccess && wide) {
           e = sorted_parts ? run_wide_sorted(a, t, staging, sms, st) : run_wide_partitioned(a, t, staging, sms, st);
         } else if (e == cudaSuccess) {
@@ -2091,6 +2268,11 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     } else if (staging) {
       cudaFreeAsync(staging, st);
     }
+  }
+  if (!domain) {
+    bool done = false;
+    e = update_undeclared(a, pow2, use_smem, sms, st, &done);
+    if (done || e != cudaSuccess) return set_status_from_cuda(e);
   }
   const bool cache_ok = !use_smem && pow2 && s->d <= 32 && rp.a >= 1 && rp.a <= 5 && s->m <= (1ll << 30) &&
                         n >= (int64_t)1 << 17 && !cache_disabled();
@@ -2180,17 +2362,6 @@ int64_t view_window(int nv, int d, int64_t n) {
   return part_window((n + wins - 1) / wins);
 }
 
-// The relation's 24-byte key records (every attribute in one join).
-cudaError_t family_table(const UpdArgs& a, const TabArgs& t, int64_t total, int sms, cudaStream_t st) {
-  const size_t coef_bytes = (size_t)a.d * a.row_len * sizeof(uint64_t);
-  const cudaError_t e = fit_dynamic_smem((const void*)k_key_table_l24<true>, coef_bytes);
-  if (e != cudaSuccess) return e;
-  const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
-  k_key_table_l24<true><<<bgrid, 256, coef_bytes, st>>>(a, t);
-  count_launch();
-  return cudaGetLastError();
-}
-
 // Both phases of all nv views over every window; staging: view_items_bytes, then the counts.
 cudaError_t run_partitioned_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm,
                                   unsigned long long* const* ctr, void* staging, int64_t W, int sms, cudaStream_t st) {
@@ -2208,6 +2379,7 @@ cudaError_t run_partitioned_views(const UpdArgs& a, const TabArgs& t, const View
   q.vbits = nullptr;
   q.wts = nullptr;
   q.wmax = 0;
+  q.go = nullptr;
   const int S = (int)(a.m >> q.logL);
   const size_t smem = (size_t)4 << q.logL;
   e = allow_dynamic_smem((const void*)k_part_accum<false>);
@@ -2320,7 +2492,7 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
     if (pool_malloc_async(&staging, vbytes, st) == cudaSuccess) {
       *done = true;
       t.tbl = (uint32_t*)tbl;
-      cudaError_t e = family_table(a, t, total, sms, st);
+      cudaError_t e = launch_table_l24(a, t, nullptr, (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32), st);
       if (e == cudaSuccess) e = run_partitioned_views(a, t, vm, vctr, staging, W, sms, st);
       cudaError_t ef = cudaFreeAsync(tbl, st);
       const cudaError_t es = cudaFreeAsync(staging, st);
@@ -2340,7 +2512,7 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
   *done = true;
   uint32_t* vbits = (uint32_t*)((char*)staging + sbytes);
   t.tbl = (uint32_t*)tbl;
-  cudaError_t e = family_table(a, t, total, sms, st);
+  cudaError_t e = launch_table_l24(a, t, nullptr, (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32), st);
   if (e == cudaSuccess) {
     k_valid_bits<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, vbits);
     count_launch();
