@@ -873,7 +873,8 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
 // ---------------------------------------------------------------------------
 // Partitioned update for the widest sketches (unit weights, power-of-two 2^21 <= m <= 2^24,
 // d <= 16, at most 5 attributes, declared domains; 2^17 <= m <= 2^20 takes k_wide_sort below,
-// whose one-word items have no room for more bins).  A d x m int64 sketch of 128 MB does not
+// whose one-word items have no room for more bins, unless its two reads of the keys would
+// cross the host link).  A d x m int64 sketch of 128 MB does not
 // stay in L2, and one 64-bit reduction per (tuple, row) then
 // waits on DRAM.  Each row's bins are split into S = m / 2^15 parts of 2^15 bins (the int32
 // counters of one part fill 128 KB of one SM's shared memory); the items of a window are
@@ -1972,6 +1973,17 @@ size_t key_table_max_bytes() {
   return (size_t)(x < 0 ? 0 : x) << 20;
 }
 
+// The two paths below read a batch's keys twice.  Columns in host memory (mapped or managed), whose
+// every read crosses the link, stay with the ones that read them once.
+bool in_device_memory(const int64_t* cols) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, cols) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice;
+}
+
 // 24-byte key records of the declared domains, or of the found ones.
 cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDomains* found, int grid, cudaStream_t st) {
   auto kern = all_deg1(a) ? k_key_table_l24<true> : k_key_table_l24<false>;
@@ -2064,7 +2076,7 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
     return cudaSuccess;
   cudaStreamCaptureStatus cap_st = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(st, &cap_st);
-  if (e != cudaSuccess || cap_st != cudaStreamCaptureStatusNone) return e;
+  if (e != cudaSuccess || cap_st != cudaStreamCaptureStatusNone || !in_device_memory(a0.cols)) return e;
   // records per attribute: a quarter of the tuples (the rule for declared domains), within the
   // tables' limit
   const int64_t cap = std::min<int64_t>(n / 4, (int64_t)(key_table_max_bytes() / 24) / a0.a);
@@ -2191,7 +2203,9 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
     // wide partitioned update takes the batch: it replaces those atomics.
     const bool worth = ktm == 1 || (n >= ((int64_t)1 << 16) && total * 4 <= n * (int64_t)rp.a &&
                                     (sketch_bytes <= ((size_t)32 << 20) || wide));
-    const bool sorted_parts = s->m <= ((int64_t)kSortMaxParts << 15);
+    // k_wide_sort reads the keys once per group of eight rows
+    const bool sorted_parts = wide && s->m <= ((int64_t)kSortMaxParts << 15) &&
+                              (s->d <= kSortRows || in_device_memory(cols));
     void* staging = nullptr;
     if (fits && worth && total > 0 && part) {
       e = pool_malloc_async(&staging, part_staging_bytes(s->d, part_window(n, part_most(weights)), sms, weights != nullptr),
@@ -2486,10 +2500,10 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
         vctr[vm.nv] = ctr[v];
         vm.mask[vm.nv++] = (uint8_t)amask[v];
       }
-    const int64_t W = view_window(vm.nv, a.d, n);
+    const int64_t W = view_window(std::max(1, vm.nv), a.d, n);
     const size_t vbytes = view_items_bytes(vm.nv, a.d, W, sms) +
                           (size_t)vm.nv * sms * kPartMaxCtasPerSm * 16 * sizeof(uint32_t);
-    if (pool_malloc_async(&staging, vbytes, st) == cudaSuccess) {
+    if (vm.nv > 0 && pool_malloc_async(&staging, vbytes, st) == cudaSuccess) {
       *done = true;
       t.tbl = (uint32_t*)tbl;
       cudaError_t e = launch_table_l24(a, t, nullptr, (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32), st);
