@@ -2127,8 +2127,14 @@ sk_status run_estimate_pairwise(sk_set* s, sk_estimate* out, cudaStream_t st, bo
   const std::vector<FuPrime>& pr = fu_primes();
   const size_t words = (size_t)s->r * s->d * m;
   if (wide) {
-    const int at_once = ntt_primes_at_once(words, f.np);
-    SK_CK(ensure(s->fft_scratch, (size_t)at_once * words * sizeof(uint32_t), st));
+    int at_once = ntt_primes_at_once(words, f.np);
+    cudaError_t ea = ensure(s->fft_scratch, (size_t)at_once * words * sizeof(uint32_t), st);
+    if (ea == cudaErrorMemoryAllocation && at_once > 1) {   // little room: one prime at a time
+      cudaGetLastError();
+      at_once = 1;
+      ea = ensure(s->fft_scratch, words * sizeof(uint32_t), st);
+    }
+    SK_CK(ea);
     unsigned long long* d_sums = (unsigned long long*)f.d_res;   // [d][kFuMaxPrimes]
     const size_t nsum = (size_t)s->d * kFuMaxPrimes;
     SK_CK(cudaMemsetAsync(d_sums, 0, nsum * 8, st));
@@ -2222,12 +2228,18 @@ sk_status run_estimate_crt(sk_set* s, sk_estimate* out, cudaStream_t st, bool* d
   for (const EstOp& op : s->plan)
     if ((op.kind == OP_CORR || op.kind == OP_HAD) && buf[op.dst] < 0) buf[op.dst] = nbuf++;
   const size_t per_prime = (size_t)nbuf * dM * sizeof(uint32_t);
-  const int at_once = (int)std::min<size_t>(f.np, std::max<size_t>(1, ((size_t)1 << 30) / per_prime));
+  int at_once = (int)std::min<size_t>(f.np, std::max<size_t>(1, ((size_t)1 << 30) / per_prime));
   const size_t nsum = (size_t)d * kFuMaxPrimes;
   unsigned long long* d_sums = (unsigned long long*)f.d_res;
   SK_CK(cudaMemsetAsync(d_sums, 0, nsum * 8, st));
   uint32_t* pool = nullptr;
-  SK_CK(pool_malloc_async((void**)&pool, (size_t)at_once * per_prime, st));
+  cudaError_t ea = pool_malloc_async((void**)&pool, (size_t)at_once * per_prime, st);
+  if (ea == cudaErrorMemoryAllocation && at_once > 1) {   // little room: one prime at a time
+    cudaGetLastError();
+    at_once = 1;
+    ea = pool_malloc_async((void**)&pool, per_prime, st);
+  }
+  SK_CK(ea);
   int e_r = 0, e_m = 0;   // the sums' factor: 2^(-32 e_r) M^e_m
   auto run = [&]() -> sk_status {
     const int logM = ilog2(M), logR = logM - ntt::kLogRow;
