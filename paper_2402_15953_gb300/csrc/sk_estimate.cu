@@ -1869,7 +1869,8 @@ cudaError_t ntt_constants() {
   const std::vector<FuPrime>& pr = fu_primes();
   constexpr int NP = ntt::kMaxPrimes, NL = ntt::kMaxLog - ntt::kMinLog + 1;
   static_assert(NP == kFuMaxPrimes, "one table per CRT prime");
-  std::vector<uint32_t> root((size_t)NP * 2 * 4096), low((size_t)NP * 2 * NL * 1024), row((size_t)NP * 2 * 1024);
+  std::vector<uint32_t> root((size_t)NP * 2 * 4096), low((size_t)NP * 2 * NL * 1024);
+  std::vector<ntt::Factor> row((size_t)NP * 2 * 1024);
   std::vector<ntt::PrimeConst> pc(NP);
   for (int i = 0; i < NP; i++) {
     const uint64_t p = pr[i].p;
@@ -1888,13 +1889,19 @@ cudaError_t ntt_constants() {
       powers(4096, 4096, r);
       for (int k = 0; k < NL; k++)
         powers((int64_t)1 << (ntt::kMinLog + k), 1024, &low[(((size_t)i * 2 + dir) * NL + k) * 1024]);
-      for (int e = 0; e < 1024; e++) row[((size_t)i * 2 + dir) * 1024 + e] = r[4 * ((e >> 5) * (e & 31))];
-      for (int j = 0; j < 32; j++) pc[i].w64[dir][j] = r[64 * j];
+      // root e of order 4096, plain, with its quotient
+      const uint64_t plain = fu_powmod((1ull << 32) % p, p - 2, p);   // 2^-32
+      auto factor = [&](int e) {
+        const uint64_t w = r[e] * plain % p;
+        return ntt::Factor{(uint32_t)w, (uint32_t)((w << 32) / p)};
+      };
+      for (int e = 0; e < 1024; e++) row[((size_t)i * 2 + dir) * 1024 + e] = factor(4 * ((e >> 5) * (e & 31)));
+      for (int j = 0; j < 32; j++) pc[i].w64[dir][j] = factor(64 * j);
     }
   }
   cudaError_t e = cudaMemcpyToSymbol(ntt::g_root, root.data(), root.size() * 4);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_low, low.data(), low.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_row, row.data(), row.size() * 4);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_row, row.data(), row.size() * sizeof(ntt::Factor));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::c_prime, pc.data(), pc.size() * sizeof(ntt::PrimeConst));
   return e;
 }

@@ -13,14 +13,17 @@
 // that all factors of a product sit in the same lane and register.  All primes of an estimate
 // run in one launch (grid y).
 //
-// Bound: the integer multiplier (a modular product is two 32 x 32 -> 64-bit multiplies and one
-// 32-bit one; ncu: 64 % of the pipe in the row pass, 50 % issue).  m = 2^20 and 2^16: 3.1 ns per
-// 1024 elements and prime in the column pass, 2.3 ns in the row pass, against 1.8 and 0.6 ns for
-// their bytes at the measured copy rate.  The chain of eight at m = 2^20, d = 16 (6 primes): 4.17 ms,
-// 11.4 ms with residues, spectra and products each in their own pass over memory.
+// Bound: the integer multiplier, about five modular products per element and pass (a Montgomery
+// product is two 32 x 32 -> 64-bit multiplies and one 32-bit one: 64 % of the pipe in the row pass,
+// 50 % issue), and in the column pass the bytes.  m = 2^20 and 2^16 with Montgomery products
+// throughout: 3.1 ns per 1024 elements and prime in the column pass, 2.3 ns in the row pass,
+// against 1.8 and 0.6 ns for their bytes at the measured copy rate.  The chain of eight at m = 2^20,
+// d = 16 (6 primes): 3.85 ms; 4.18 ms with Montgomery products throughout, 11.4 ms with residues,
+// spectra and products each in their own pass over memory.
 //
-// Residues are plain (not in Montgomery form); the twiddles are in Montgomery form with
-// R = 2^32, so x (*) w is again a plain residue.  The r - 1 products of spectra each bring a
+// Residues are plain (not in Montgomery form).  The fixed twiddles of the DFTs and of the row
+// exchange come with their quotients (Factor), the others in Montgomery form with R = 2^32, so
+// x (*) w is again a plain residue either way.  The r - 1 products of spectra each bring a
 // factor 2^-32, which the host takes out of the final sums.
 #pragma once
 
@@ -34,17 +37,23 @@ constexpr int kMaxPrimes = 9;
 constexpr int kLogRow = 10;                 // row length 1024
 constexpr int kMinLog = 10, kMaxLog = 22;   // transform lengths
 
+// A fixed factor w with its quotient floor(w 2^32 / p) (Shoup's modular product).
+struct alignas(8) Factor {
+  uint32_t w, s;
+};
+
 struct PrimeConst {
-  uint32_t p, pinv;       // pinv = -p^-1 mod 2^32
-  uint32_t r2;            // 2^64 mod p
-  uint32_t w64[2][32];    // w_64^j, j < 32 (Montgomery form): [0] forward, [1] inverse root
+  uint32_t p, pinv;     // pinv = -p^-1 mod 2^32
+  uint32_t r2;          // 2^64 mod p
+  Factor w64[2][32];    // w_64^j, j < 32: [0] forward, [1] inverse root
 };
 __constant__ PrimeConst c_prime[kMaxPrimes];
+
+__device__ __align__(16) Factor g_row[kMaxPrimes][2][1024];   // w_1024^(c b) at 32 c + b, [prime][direction]
 
 // Powers of the roots of unity, Montgomery form, [prime][direction]:
 __device__ uint32_t g_root[kMaxPrimes][2][4096];                           // w_4096^e
 __device__ uint32_t g_low[kMaxPrimes][2][kMaxLog - kMinLog + 1][1024];     // w_N^e, e < 1024
-__device__ uint32_t g_row[kMaxPrimes][2][1024];                            // w_1024^(c b) at 32 c + b
 
 struct Mod {
   uint32_t p, pinv;
@@ -64,6 +73,14 @@ __device__ __forceinline__ uint32_t mul(uint32_t a, uint32_t b, Mod q) {
   const uint64_t t = (uint64_t)a * b;
   const uint32_t m = (uint32_t)t * q.pinv;
   const uint32_t u = (uint32_t)((t + (uint64_t)m * q.p) >> 32);
+  return min(u, u - q.p);
+}
+
+// a w mod p for any a: with q = floor(a s / 2^32), a w - q p < 2p.  One 64-bit product and two
+// 32-bit ones; a Montgomery product takes two and one (32-point DFTs alone: 0.61 -> 0.48 ns
+// per 1024 elements).
+__device__ __forceinline__ uint32_t mul(uint32_t a, Factor f, Mod q) {
+  const uint32_t u = a * f.w - __umulhi(a, f.s) * q.p;
   return min(u, u - q.p);
 }
 
@@ -109,7 +126,7 @@ constexpr int rev_bits(int k, int bits) {
 // 2^LOG-point DFT in registers, natural order in and out; w64[j] = w_64^j.  Radix-2 decimation
 // in frequency; the difference of a butterfly with a twiddle is left in (0, 2p) for mul.
 template <int LOG>
-__device__ __forceinline__ void dft(uint32_t (&x)[1 << LOG], const uint32_t* w64, Mod q) {
+__device__ __forceinline__ void dft(uint32_t (&x)[1 << LOG], const Factor* w64, Mod q) {
   constexpr int N = 1 << LOG;
 #pragma unroll
   for (int st = 0; st < LOG; st++) {
@@ -195,7 +212,7 @@ __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __gri
   const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
   const uint32_t r2 = c_prime[prime].r2;
   const int dir = WORDS ? (int)(a.negmask & 1ull) : dir_of(a, vec);
-  const uint32_t* w64 = c_prime[prime].w64[dir];
+  const Factor* w64 = c_prime[prime].w64[dir];
   const int64_t at0 = (((int64_t)blockIdx.y * a.stride + vec) << (LR + kLogRow)) + n2;
   const int64_t* src = WORDS ? nullptr : a.base[vec / a.per] + (vec % a.per) * a.m + n2;
   uint32_t* dst = a.V + at0;
@@ -277,7 +294,7 @@ struct RowArgs {
 // (2.40 against 2.24 ns per 1024 elements), and more warps per SM (80 registers) only spilled
 // more (2.6): the multiplier pipe, not the number of warps, sets the rate.
 __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ RowArgs a) {
-  __shared__ uint32_t s_tw[2][1024];
+  __shared__ __align__(16) Factor s_tw[2][1024];
   __shared__ uint32_t s_ex[8][32 * 33];
   __shared__ unsigned long long s_sum[8];
   extern __shared__ uint32_t s_prod[];   // 8 x 1024
@@ -289,7 +306,7 @@ __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ Row
   const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
   const int k1 = (int)(blockIdx.x & ((1u << lcta) - 1u)) * 8 + warp;
   const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
-  for (int i = threadIdx.x; i < 2048; i += 256) ((uint32_t*)s_tw)[i] = ((const uint32_t*)g_row[prime])[i];
+  for (int i = threadIdx.x; i < 1024; i += 256) ((uint4*)s_tw)[i] = ((const uint4*)g_row[prime])[i];
   __syncthreads();
   unsigned long long sum = 0;
   if (k1 < R) {
@@ -310,8 +327,8 @@ __global__ void __launch_bounds__(256, 2) k_ntt_rows(const __grid_constant__ Row
     for (int i = 0; i < 32; i++) x[i] = __ldcs(row + 32 * i);
     for (int k = 0; k < f.r; k++) {
       const int dir = (int)((f.negmask >> k) & 1ull);
-      const uint32_t* w64 = c_prime[prime].w64[dir];
-      const uint32_t* tw = s_tw[dir];
+      const Factor* w64 = c_prime[prime].w64[dir];
+      const Factor* tw = s_tw[dir];
       dft<5>(x, w64, q);
 #pragma unroll
       for (int i = 0; i < 32; i++) ex[i * 33 + lane] = i ? mul(x[i], tw[i * 32 + lane], q) : x[i];
@@ -360,7 +377,7 @@ struct CorrRowArgs {
 };
 
 __global__ void __launch_bounds__(256, 2) k_ntt_corr(const __grid_constant__ CorrRowArgs a) {
-  __shared__ uint32_t s_tw[2][1024];
+  __shared__ __align__(16) Factor s_tw[2][1024];
   __shared__ uint32_t s_ex[8][32 * 33];
   extern __shared__ uint32_t s_prod[];   // 8 x 1024
   const int prime = a.prime0 + (int)blockIdx.y;
@@ -370,7 +387,7 @@ __global__ void __launch_bounds__(256, 2) k_ntt_corr(const __grid_constant__ Cor
   const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
   const int k1 = (int)(blockIdx.x & ((1u << lcta) - 1u)) * 8 + warp;
   const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
-  for (int i = threadIdx.x; i < 2048; i += 256) ((uint32_t*)s_tw)[i] = ((const uint32_t*)g_row[prime])[i];
+  for (int i = threadIdx.x; i < 1024; i += 256) ((uint4*)s_tw)[i] = ((const uint4*)g_row[prime])[i];
   __syncthreads();
   if (k1 >= R) return;
   const int64_t at = (((int64_t)blockIdx.y * a.stride + v) << (a.logR + kLogRow)) + ((int64_t)k1 << kLogRow) + lane;
@@ -383,8 +400,8 @@ __global__ void __launch_bounds__(256, 2) k_ntt_corr(const __grid_constant__ Cor
 #pragma unroll 1
   for (int step = 0; step < 3; step++) {
     const int dir = step == 1 ? 0 : 1;
-    const uint32_t* w64 = c_prime[prime].w64[dir];
-    const uint32_t* tw = s_tw[dir];
+    const Factor* w64 = c_prime[prime].w64[dir];
+    const Factor* tw = s_tw[dir];
     dft<5>(x, w64, q);
 #pragma unroll
     for (int i = 0; i < 32; i++) ex[i * 33 + lane] = i ? mul(x[i], tw[i * 32 + lane], q) : x[i];
@@ -534,7 +551,7 @@ inline cudaError_t cols_back(const ColArgs& a, int64_t nvec, int primes, cudaStr
 inline cudaError_t rows(const RowArgs& a, int64_t nout, int primes, cudaStream_t st) {
   const int lcta = a.logR > 3 ? a.logR - 3 : 0;
   constexpr size_t smem = 8 * 1024 * sizeof(uint32_t);
-  const cudaError_t e = allow_dynamic_smem((const void*)k_ntt_rows);   // 74 KB with its static arrays
+  const cudaError_t e = allow_dynamic_smem((const void*)k_ntt_rows);   // 82 KB with its static arrays
   if (e != cudaSuccess) return e;
   k_ntt_rows<<<dim3((unsigned)(nout << lcta), (unsigned)primes), 256, smem, st>>>(a);
   count_launch();
