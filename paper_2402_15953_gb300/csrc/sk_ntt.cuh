@@ -177,8 +177,9 @@ struct ColArgs {
   int logR;
   uint32_t* V;              // [prime][stride vectors][N]
   int64_t stride;           // vectors per prime in V
-  int prime0;               // prime of grid y = 0
+  int prime0;               // first prime of the launch
   int nvec[kMaxPrimes];     // vectors of each prime (leading ones)
+  int primes = 1;           // of the launch
   const uint32_t* words = nullptr;   // may be V: a CTA reads its columns before it writes them
   int64_t fold = 0;
 };
@@ -205,15 +206,17 @@ template <int LA, int LB, bool WORDS, bool BACK>
 __global__ void __launch_bounds__(256, (LB <= 5 ? 4 : 2)) k_ntt_cols(const __grid_constant__ ColArgs a) {
   constexpr int A = 1 << LA, B = 1 << LB, LR = LA + LB;
   constexpr int LCB = LA ? 8 - LA : 8, CB = 1 << LCB;
-  const int prime = a.prime0 + (int)blockIdx.y;
-  const int64_t vec = blockIdx.x >> (kLogRow - LCB);
+  // the primes of one tile run next to each other: its counters come from memory once
+  const unsigned pi = blockIdx.x % (unsigned)a.primes, tile = blockIdx.x / (unsigned)a.primes;
+  const int prime = a.prime0 + (int)pi;
+  const int64_t vec = tile >> (kLogRow - LCB);
   if (vec >= a.nvec[prime]) return;
-  const int n2 = (int)(blockIdx.x & ((1u << (kLogRow - LCB)) - 1u)) * CB + (int)(threadIdx.x & (CB - 1));
+  const int n2 = (int)(tile & ((1u << (kLogRow - LCB)) - 1u)) * CB + (int)(threadIdx.x & (CB - 1));
   const Mod q = {c_prime[prime].p, c_prime[prime].pinv};
   const uint32_t r2 = c_prime[prime].r2;
   const int dir = WORDS ? (int)(a.negmask & 1ull) : dir_of(a, vec);
   const Factor* w64 = c_prime[prime].w64[dir];
-  const int64_t at0 = (((int64_t)blockIdx.y * a.stride + vec) << (LR + kLogRow)) + n2;
+  const int64_t at0 = (((int64_t)pi * a.stride + vec) << (LR + kLogRow)) + n2;
   const int64_t* src = WORDS ? nullptr : a.base[vec / a.per] + (vec % a.per) * a.m + n2;
   uint32_t* dst = a.V + at0;
   const int64_t left = a.m - n2;   // counters of this column: rows n1 with 1024 n1 < left
@@ -510,13 +513,13 @@ inline cudaError_t had(const HadArgs& a, int rows, int primes, int sms, cudaStre
 }
 
 template <int LA, int LB, bool WORDS, bool BACK>
-cudaError_t launch_cols(const ColArgs& a, int64_t nvec, int primes, cudaStream_t st) {
+cudaError_t launch_cols(ColArgs a, int64_t nvec, int primes, cudaStream_t st) {
   constexpr int LCB = LA ? 8 - LA : 8;
   const size_t smem = LA ? ((size_t)(1 << (LA + LB)) + ((size_t)(1 << LA) * ((1 << LB) + 1) << LCB)) * 4 : 0;
   const cudaError_t e = fit_dynamic_smem((const void*)k_ntt_cols<LA, LB, WORDS, BACK>, smem);
   if (e != cudaSuccess) return e;
-  k_ntt_cols<LA, LB, WORDS, BACK>
-      <<<dim3((unsigned)(nvec << (kLogRow - LCB)), (unsigned)primes), 256, smem, st>>>(a);
+  a.primes = primes;
+  k_ntt_cols<LA, LB, WORDS, BACK><<<(unsigned)((nvec << (kLogRow - LCB)) * primes), 256, smem, st>>>(a);
   count_launch();
   return cudaGetLastError();
 }
