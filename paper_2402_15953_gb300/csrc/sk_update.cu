@@ -585,41 +585,49 @@ __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long l
   }
 }
 
-// Phase 1 for all views of a sub-query family's relation at once (24-byte records, unit weights):
-// the tuple's A records are gathered once and every view sums the records of its attributes, so
-// nv views cost one gather per attribute instead of one per (view, attribute).  A tuple with any
-// key outside its domain is left out of every view.
-// Regions are one CTA's here, [view][CTA][row][C]: 15 views of nine rows and two parts are 270
-// streams, and one set per warp left a million half-written lines, as much as L2 holds (4.3 ms
-// per 1e7 tuples, 5 GB read back and 5 GB written for 2.7 GB of items).  The CTA's warps take their
-// places from shared-memory counters, part-0 and part-1 items in the halves of one 64-bit word,
-// with one returning atomic per tile and view (lane j: row j).
-// 15 views of a 4-attribute relation, 1e7 tuples: 2.3 ms, 54 % issue (one view at a time: 2.7 ms).
+// All views of a sub-query family's relation (24-byte records, unit weights).  A view's bin is the
+// sum of its attributes' bins, so the views need no items of their own:
+//   1. k_view_planes gathers a tuple's A records once and leaves, for every row and attribute, the
+//      16-bit bins and one sign bit per tuple in planes over the window's tuples, and one bit per
+//      tuple that all its keys are inside their domains (others are left out of every view);
+//   2. k_view_accum: a CTA owns a part (at most 2^15 bins) of one view's row as int32 counters in
+//      shared memory; a thread loads the same eight tuples of each of the view's attributes (16
+//      bytes and one of signs), adds the bins two to a word and adds the eight signs of those
+//      whose bin is in the part.
+// Nine rows of 15 views of a 4-attribute relation, 2e7 tuples, m = 2^16: k_view_planes 0.64 ms (70 % of
+// the L1 data pipe: four gathers and 36 stores per tuple), k_view_accum 3.14 ms (issue 86 %, about 18
+// instructions per tuple, view, row and part; 1.5 GB of planes against 5.4 GB of items).  With items
+// written per view (k_tab_items' partition for every view at once) the two phases took 7.1 ms.
 struct ViewMasks {
   int nv;
   uint8_t mask[SK_MAX_VIEWS];   // bit u: the view joins attribute u
 };
 
+// The planes of a window are cut into tiles of kViewTile tuples, [tile][bins d a | signs d a | kept]:
+// a CTA's stores stay within one tile (with planes over the whole window they went to 76 pages
+// at a time and k_view_planes took 1.30 ms instead of 0.64).
+constexpr int kViewTile = 8192;   // a chunk of eight tuples for each of k_view_accum's threads
+
+struct ViewPlanes {
+  uint8_t* tiles;
+  int64_t stride;          // bytes per tile
+  const int64_t* col[5];   // column u of the window's first tuple
+  int64_t cnt;             // tuples in this window
+};
+
+struct ViewCounters {
+  unsigned long long* ctr[SK_MAX_VIEWS];   // [d][m] each
+};
+
 template <int A, bool ALL9>
-__global__ void __launch_bounds__(256, 3) k_tab_items_views(UpdArgs p, TabArgs t, PartArgs q,
-                                                            const __grid_constant__ ViewMasks vm) {
-  __shared__ unsigned long long taken[SK_MAX_VIEWS * 9];   // items of row j of view v: part 0 | part 1 << 32
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+__global__ void __launch_bounds__(256, A <= 4 ? 4 : 3) k_view_planes(UpdArgs p, TabArgs t, ViewPlanes q) {
+  const int64_t step = (int64_t)gridDim.x * 256;
   const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
-  const uint32_t mask = (uint32_t)p.m - 1u;
-  const uint32_t low = (1u << q.logL) - 1u;
-  const uint32_t half = mask & ~low;
   const unsigned lane = threadIdx.x & 31u;
-  const uint32_t lt = (1u << lane) - 1u;
-  const int d = ALL9 ? 9 : p.d, nv = vm.nv;
+  const int d = ALL9 ? 9 : p.d;
   const uint64_t pol = policy_evict_first();
-  int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t C = (uint32_t)q.C;
-  const int64_t vstride = (int64_t)q.nwarps * d * q.C;
-  uint16_t* const mine = (uint16_t*)q.items + (int64_t)blockIdx.x * d * q.C;
-  for (int k = threadIdx.x; k < nv * 9; k += 256) taken[k] = 0ull;
-  __syncthreads();
-  uint32_t kx[A], okm = 0;
+  int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  uint32_t kx[A], okm = 0;   // the thread's next tuple, see k_tab_items
 #pragma unroll
   for (int u = 0; u < A; u++) {
     const int64_t k = g < q.cnt ? ld_key_policy(q.col[u] + g, pol) : -1;
@@ -646,54 +654,150 @@ __global__ void __launch_bounds__(256, 3) k_tab_items_views(UpdArgs p, TabArgs t
       okm |= (uint32_t)kin << u;
       kx[u] = kin ? (uint32_t)k : 0u;
     }
-    const uint32_t vb = __ballot_sync(0xffffffffu, ok);
-    const uint32_t nt = __popc(vb), rv = __popc(vb & lt);
-    uint16_t* out = mine;
-    for (int v = 0; v < nv; v++, out += vstride) {
-      const uint32_t am = vm.mask[v];
-      uint64_t acc[3] = {0, 0, 0};
+    const uint32_t kept = __ballot_sync(0xffffffffu, ok);
+    const uint32_t at = (uint32_t)g & (kViewTile - 1u);
+    uint8_t* const tile = q.tiles + (g / kViewTile) * q.stride;
+    uint16_t* const bins = (uint16_t*)tile + at;
+    uint32_t* const bits = (uint32_t*)(tile + (size_t)d * A * kViewTile * 2) + (at >> 5);
+    if (lane == 0) bits[d * A * (kViewTile / 32)] = kept;
+    uint32_t sb[2] = {0, 0};   // lane l: the sign bits of plane l, of plane 32 + l
 #pragma unroll
-      for (int u = 0; u < A; u++)
-        if ((am >> u) & 1u) {
-          acc[0] += rec[u][0];
-          acc[1] += rec[u][1];
-          acc[2] += rec[u][2];
-        }
-      uint32_t hb[9], n1 = 0;   // each row's part-1 tuples; lane j: how many in row j
+    for (int j = 0; j < 9; j++) {
+      if (!ALL9 && j >= d) break;
 #pragma unroll
-      for (int j = 0; j < 9; j++) {
-        if (!ALL9 && j >= d) break;
-        hb[j] = __ballot_sync(0xffffffffu, ((uint32_t)(acc[j / 3] >> (22 * (j % 3))) & half) != 0u);
-        if (lane == (unsigned)j) n1 = hb[j];
-      }
-      n1 = __popc(n1);
-      unsigned long long at0 = 0;
-      if (lane < (unsigned)d) {
-        at0 = atomicAdd(&taken[v * 9 + lane], (unsigned long long)(nt - n1) | ((unsigned long long)n1 << 32));
-        // this row's first free part-0 slot, last free part-1 slot, in the CTA's regions of the view
-        at0 = (unsigned long long)(lane * C + (uint32_t)at0) |
-              ((unsigned long long)(lane * C + C - 1u - (uint32_t)(at0 >> 32)) << 32);
-      }
-#pragma unroll
-      for (int j = 0; j < 9; j++) {
-        if (!ALL9 && j >= d) break;
-        const uint32_t x = (uint32_t)(acc[j / 3] >> (22 * (j % 3)));
-        const uint32_t b0 = __shfl_sync(0xffffffffu, (uint32_t)at0, j);
-        const uint32_t b1 = __shfl_sync(0xffffffffu, (uint32_t)(at0 >> 32), j);
-        const uint32_t r1 = __popc(hb[j] & lt);
-        const uint32_t at = (x & half) ? b1 - r1 : b0 + rv - r1;
-        if (ok) st_u16_hint(out + at, (uint16_t)((x & low) | ((x >> 4) & 0x8000u)), pol);
+      for (int u = 0; u < A; u++) {
+        const uint32_t x = (uint32_t)(rec[u][j / 3] >> (22 * (j % 3)));   // sign: bit 19
+        st_u16_hint(bins + (j * A + u) * kViewTile, (uint16_t)x, pol);
+        const uint32_t b = __ballot_sync(0xffffffffu, (x & 0x80000u) != 0u);
+        if (lane == (unsigned)((j * A + u) & 31)) sb[(j * A + u) >> 5] = b;
       }
     }
+    if (lane < (unsigned)(d * A)) bits[lane * (kViewTile / 32)] = sb[0];
+    if (A * 9 > 32 && lane + 32u < (unsigned)(d * A)) bits[(lane + 32u) * (kViewTile / 32)] = sb[1];
+  }
+}
+
+// The top bit of byte k of w over a whole word: 0 or -1.
+__device__ __forceinline__ int byte_sign(uint32_t w, int k) {
+  int r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(w), "r"(0x1111u * (8u + (uint32_t)k)));
+  return r;
+}
+
+// shared counter at saddr += v unless (w ^ flip) has the bit
+__device__ __forceinline__ void red_shared_unless(uint32_t saddr, int v, uint32_t w, uint32_t flip, uint32_t bit) {
+  asm volatile("{\n\t.reg .pred q;\n\t.reg .b32 t;\n\txor.b32 t, %2, %3;\n\tand.b32 t, t, %4;\n\t"
+               "setp.eq.u32 q, t, 0;\n\t@q red.shared.add.s32 [%0], %1;\n\t}"
+               ::"r"(saddr), "r"(v), "r"(w), "r"(flip), "r"(bit) : "memory");
+}
+
+// Eight tuples: bins in the low halves of lo and the high halves of hi, sign bits sg; of two parts
+// (TWO) those whose top bin bit is the part's; !ALL: bits of keep clear are left out.  The reductions
+// are predicated: with every lane adding, zero or to a spare word of its own where the bin is the
+// other part's, a tuple takes a quarter fewer instructions, but hot counters queue in both parts'
+// CTAs (4-attribute relation, 2e7 tuples: 3.40 ms, predicated 3.14).
+template <bool TWO, bool ALL>
+__device__ __forceinline__ void add_view_chunk(uint32_t sbase, const uint32_t (&lo)[4], const uint32_t (&hi)[4],
+                                               uint32_t sg, uint32_t keep, uint32_t low, uint32_t flip) {
+  // bits 0..3 and 4..7 of the signs at the tops of four bytes (the four products do not overlap)
+  constexpr uint32_t kSpread = (1u << 7) | (1u << 14) | (1u << 21) | (1u << 28);
+  const uint32_t s0 = (sg & 15u) * kSpread, s1 = (sg >> 4) * kSpread;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    const uint32_t w = (k & 1) ? hi[k >> 1] : lo[k >> 1];
+    const uint32_t at = sbase + ((k & 1) ? (w & (low << 16)) >> 14 : (w & low) << 2);
+    int v = byte_sign(k < 4 ? s0 : s1, k & 3) | 1;
+    if (!ALL && !(keep & (1u << k))) v = 0;
+    if (TWO) red_shared_unless(at, v, w, flip, (k & 1) ? 0x80000000u : 0x8000u);
+    else red_shared(at, v);
+  }
+}
+
+template <int C, bool TWO>
+__device__ __forceinline__ void view_accum_tiles(const ViewPlanes& q, uint32_t am, int A, int d, int row, uint32_t sbase,
+                                                 uint32_t low, uint32_t flip, int t0, int t1) {
+  // this thread's chunk in the tile: bins at 16 bytes per chunk, signs and kept at one
+  const uint8_t* tile = q.tiles + t0 * q.stride;
+  uint32_t plane[C];
+#pragma unroll
+  for (int i = 0; i < C; i++) {
+    plane[i] = (uint32_t)(row * A + __ffs(am) - 1);
+    am &= am - 1u;
+  }
+  const uint32_t signs0 = (uint32_t)(d * A) * (kViewTile * 2) + threadIdx.x;
+  uint4 nb[C];
+  uint32_t ns[C], nk = 0;
+  auto load = [&](const uint8_t* at) {
+#pragma unroll
+    for (int i = 0; i < C; i++) {
+      nb[i] = __ldg((const uint4*)(at + plane[i] * (kViewTile * 2)) + threadIdx.x);
+      ns[i] = __ldg(at + signs0 + plane[i] * (kViewTile / 8));
+    }
+    nk = __ldg(at + signs0 + (uint32_t)(d * A) * (kViewTile / 8));
+  };
+  // chunks of the last tile that hold tuples
+  const int last = (int)((q.cnt - (int64_t)(t1 - 1) * kViewTile + 7) >> 3);
+  if (t1 - 1 > t0 || (int)threadIdx.x < last) load(tile);
+  for (int t = t0; t < t1; t++) {
+    if (t + 1 == t1 && (int)threadIdx.x >= last) break;
+    uint32_t lo[4] = {nb[0].x, nb[0].y, nb[0].z, nb[0].w};
+    uint32_t hi[4] = {nb[0].x, nb[0].y, nb[0].z, nb[0].w};
+    uint32_t sg = ns[0];
+    const uint32_t keep = nk;
+    // low halves: a plain sum; high halves: no carry comes up from masked words
+#pragma unroll
+    for (int i = 1; i < C; i++) {
+      const uint32_t w[4] = {nb[i].x, nb[i].y, nb[i].z, nb[i].w};
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        lo[k] += w[k];
+        hi[k] += w[k] & 0xffff0000u;
+      }
+      sg ^= ns[i];
+    }
+    tile += q.stride;
+    if (t + 2 < t1 || (t + 2 == t1 && (int)threadIdx.x < last)) load(tile);   // in flight during the additions
+    if (keep == 0xffu) add_view_chunk<TWO, true>(sbase, lo, hi, sg, keep, low, flip);
+    else add_view_chunk<TWO, false>(sbase, lo, hi, sg, keep, low, flip);
+  }
+}
+
+// blockIdx.x = part + S (view + nv (row + d range)): the CTAs that run together read the planes
+// of a few rows.
+template <bool TWO>
+__global__ void __launch_bounds__(1024) k_view_accum(ViewPlanes q, const __grid_constant__ ViewMasks vm,
+                                                     const __grid_constant__ ViewCounters vc, int A, int d, int64_t m,
+                                                     int logL, int nr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int* cnt = (int*)smem_raw;
+  constexpr int S = TWO ? 2 : 1;
+  const int L = 1 << logL;
+  unsigned b = blockIdx.x;
+  const int part = (int)(b % (unsigned)S);
+  b /= (unsigned)S;
+  const int v = (int)(b % (unsigned)vm.nv);
+  b /= (unsigned)vm.nv;
+  const int row = (int)(b % (unsigned)d), range = (int)(b / (unsigned)d);
+  for (int k = threadIdx.x; k < L / 4; k += 1024) ((int4*)cnt)[k] = make_int4(0, 0, 0, 0);
+  __syncthreads();
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(cnt);
+  const int64_t nt = (q.cnt + kViewTile - 1) / kViewTile;
+  const int t0 = (int)(nt * range / nr), t1 = (int)(nt * (range + 1) / nr);
+  const uint32_t low = (uint32_t)(L - 1);
+  const uint32_t flip = part ? 0x80008000u : 0u;
+  const uint32_t am = vm.mask[v];
+  switch (__popc(am)) {
+    case 1: view_accum_tiles<1, TWO>(q, am, A, d, row, sbase, low, flip, t0, t1); break;
+    case 2: view_accum_tiles<2, TWO>(q, am, A, d, row, sbase, low, flip, t0, t1); break;
+    case 3: view_accum_tiles<3, TWO>(q, am, A, d, row, sbase, low, flip, t0, t1); break;
+    case 4: view_accum_tiles<4, TWO>(q, am, A, d, row, sbase, low, flip, t0, t1); break;
+    default: view_accum_tiles<5, TWO>(q, am, A, d, row, sbase, low, flip, t0, t1); break;
   }
   __syncthreads();
-  // the CTA's counts: word j < d row j's part-0 items, word 15 the valid tuples (any row's items)
-  for (int k = threadIdx.x; k < nv * 16; k += 256) {
-    const int v = k >> 4, j = k & 15;
-    if (j < d || j == 15) {
-      const unsigned long long n = taken[v * 9 + (j < d ? j : 0)];
-      q.cnts[((int64_t)v * q.nwarps + blockIdx.x) * 16 + j] = j < d ? (uint32_t)n : (uint32_t)n + (uint32_t)(n >> 32);
-    }
+  unsigned long long* out = vc.ctr[v] + (int64_t)row * m + ((int64_t)part << logL);
+  for (int x = threadIdx.x; x < L; x += 1024) {
+    const int s = cnt[x];
+    if (s != 0) red_add_global(out + x, (unsigned long long)(int64_t)s);
   }
 }
 
@@ -2353,73 +2457,65 @@ sk_status launch_merge(int64_t* dst, const int64_t* src, int64_t count, cudaStre
 
 namespace {
 
-using ViewItemsKernel = void (*)(UpdArgs, TabArgs, PartArgs, ViewMasks);
+using ViewPlanesKernel = void (*)(UpdArgs, TabArgs, ViewPlanes);
 
 template <bool ALL9>
-ViewItemsKernel view_items_kernel(int A) {
+ViewPlanesKernel view_planes_kernel(int A) {
   switch (A) {
-    case 1: return k_tab_items_views<1, ALL9>;
-    case 2: return k_tab_items_views<2, ALL9>;
-    case 3: return k_tab_items_views<3, ALL9>;
-    case 4: return k_tab_items_views<4, ALL9>;
-    default: return k_tab_items_views<5, ALL9>;
+    case 1: return k_view_planes<1, ALL9>;
+    case 2: return k_view_planes<2, ALL9>;
+    case 3: return k_view_planes<3, ALL9>;
+    case 4: return k_view_planes<4, ALL9>;
+    default: return k_view_planes<5, ALL9>;
   }
 }
 
-// Staging of the views' items for windows of W tuples, and the window that keeps it near 3 GiB
-// (the library's pool keeps 4 GiB between calls): a batch is cut into equal windows.
-size_t view_items_bytes(int nv, int d, int64_t W, int sms) { return nv * part_items_bytes(d, W, sms, false); }
+// Bytes of a tile, and of the planes of a window of W tuples.
+int64_t view_tile_bytes(int A, int d) { return (int64_t)kViewTile * 2 * A * d + kViewTile / 8 * (A * d + 1); }
 
-int64_t view_window(int nv, int d, int64_t n) {
-  const int64_t most = std::max<int64_t>(1 << 20, ((int64_t)3 << 30) / ((int64_t)nv * d * 2));
+size_t view_plane_bytes(int A, int d, int64_t W) {
+  return (size_t)((W + kViewTile - 1) / kViewTile) * (size_t)view_tile_bytes(A, d);
+}
+
+// Tuples per window: planes near 3 GiB at most (the library's pool keeps 4 GiB between calls), a
+// batch cut into equal windows.
+int64_t view_window(int A, int d, int64_t n) {
+  const int64_t most = ((int64_t)3 << 30) / view_tile_bytes(A, d) * kViewTile;
   const int64_t wins = (n + most - 1) / most;
   return part_window((n + wins - 1) / wins);
 }
 
-// Both phases of all nv views over every window; staging: view_items_bytes, then the counts.
-cudaError_t run_partitioned_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm,
-                                  unsigned long long* const* ctr, void* staging, int64_t W, int sms, cudaStream_t st) {
-  ViewItemsKernel items = a.d == 9 ? view_items_kernel<true>(a.a) : view_items_kernel<false>(a.a);
+// Both kernels over every window; planes: view_plane_bytes.
+cudaError_t run_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm, const ViewCounters& vc, void* planes,
+                      int64_t W, int sms, cudaStream_t st) {
+  ViewPlanesKernel make = a.d == 9 ? view_planes_kernel<true>(a.a) : view_planes_kernel<false>(a.a);
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, items, 256, 0);
+  cudaError_t e = cudaFuncSetAttribute((const void*)make, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, make, 256, 0);
   if (e != cudaSuccess) return e;
-  const int64_t full_grid = (int64_t)sms * std::max(1, std::min(per_sm, kPartMaxCtasPerSm));
-  PartArgs q;
-  q.cnts = (uint32_t*)((char*)staging + view_items_bytes(vm.nv, a.d, W, sms));
-  q.W = W;
-  int logm = 0;
-  while (((int64_t)1 << logm) < (int64_t)a.m) logm++;
-  q.logL = std::min(logm, 15);
-  q.vbits = nullptr;
-  q.wts = nullptr;
-  q.wmax = 0;
-  q.go = nullptr;
-  const int S = (int)(a.m >> q.logL);
-  const size_t smem = (size_t)4 << q.logL;
-  e = allow_dynamic_smem((const void*)k_part_accum<false>);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_part_accum<false>, 1024, smem);
-  const int64_t slots = (int64_t)sms * std::max(1, per_sm), units = (int64_t)S * a.d;
+  const int64_t full_grid = (int64_t)sms * std::max(1, per_sm);
+  int logL = 0;
+  while (logL < 15 && ((int64_t)1 << logL) < (int64_t)a.m) logL++;
+  const int S = (int)(a.m >> logL);
+  const size_t smem = (size_t)4 << logL;
+  auto accum = S == 2 ? k_view_accum<true> : k_view_accum<false>;
+  e = allow_dynamic_smem((const void*)accum);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accum, 1024, smem);
+  const int64_t slots = (int64_t)sms * std::max(1, per_sm), units = (int64_t)S * a.d * vm.nv;
+  ViewPlanes q;
+  q.tiles = (uint8_t*)planes;
+  q.stride = view_tile_bytes(a.a, a.d);
   for (int64_t i0 = 0; i0 < a.n && e == cudaSuccess; i0 += W) {
-    q.items = staging;
     q.cnt = std::min(W, a.n - i0);
     for (int u = 0; u < 5; u++) q.col[u] = u < a.a ? a.cols + (int64_t)u * a.stride + i0 : nullptr;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((q.cnt + 255) / 256, full_grid));
-    const int64_t gend = (q.cnt + 31) / 32 * 32;
-    q.C = 256 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
-    q.nwarps = grid;   // regions are the CTAs'
-    items<<<grid, 256, 0, st>>>(a, t, q, vm);
+    make<<<(unsigned)std::min<int64_t>((q.cnt + 255) / 256, full_grid), 256, 0, st>>>(a, t, q);
     count_launch();
     e = cudaGetLastError();
-    const PartSplit sp = part_split(q.cnt * a.d, units, slots, q.nwarps);
-    for (int v = 0; v < vm.nv && e == cudaSuccess; v++) {
-      PartArgs qv = q;
-      qv.items = (uint16_t*)q.items + (int64_t)v * q.nwarps * a.d * q.C;
-      qv.cnts = q.cnts + (int64_t)v * q.nwarps * 16;
-      k_part_accum<false><<<(unsigned)(units * sp.nr), 1024, smem, st>>>(qv, ctr[v], (int64_t)a.m, a.d, q.logL, sp.R,
-                                                                         sp.logP);
-      count_launch();
-      e = cudaGetLastError();
-    }
+    if (e != cudaSuccess) break;
+    const int nr = (int)part_ranges(q.cnt * units, units, slots, (q.cnt + kViewTile - 1) / kViewTile);
+    accum<<<(unsigned)(units * nr), 1024, smem, st>>>(q, vm, vc, a.a, a.d, (int64_t)a.m, logL, nr);
+    count_launch();
+    e = cudaGetLastError();
   }
   return e;
 }
@@ -2444,10 +2540,10 @@ __global__ void __launch_bounds__(256) k_valid_bits(UpdArgs p, uint32_t* bits) {
 // Sub-query family views of one relation through the two-phase partitioned update (see
 // run_partitioned): when every attribute has exactly one sign slot, a view's sign is the
 // product of its attributes' slot-0 signs and its bin the sum of their bins, so one 24-byte
-// key table over the relation's attributes (built once) serves every view, and each view's
-// counters get both phases over the view's attributes (a validity pass over all of the
-// relation's keys first: a tuple is left out of every view when any key is outside its
-// domain, as in the per-tuple view update).  Taken for unit weights with declared
+// key table over the relation's attributes (built once) serves every view.  Large batches go
+// through the planes of run_views; else each view's counters get both phases over the view's
+// attributes (a validity pass over all of the relation's keys first: a tuple is left out of
+// every view when any key is outside its domain, as in the per-tuple view update).  Taken for unit weights with declared
 // domains, power-of-two 1024 <= m <= 2^16, d <= 9, views of at most 5 attributes, at least
 // 16 m tuples and views too large for one CTA's shared memory; *done = false (nothing
 // launched) otherwise, and the caller runs its per-tuple view update.
@@ -2487,33 +2583,31 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
     cudaGetLastError();
     return SK_OK;
   }
-  // All views in one first phase: for two views or more of a relation of at most five attributes,
-  // from 2^21 tuples (a 4-attribute relation's 15 views, m = 2^16, d = 9, against one view at a
-  // time: 0.80 and 0.82 ms at 2^20 tuples, where the second phases are most of either form, 1.10
-  // and 1.17 at 2^21, 3.00 and 3.59 at 2^23).
-  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)1 << 21)) {
+  // All views from one set of planes: for two views or more of a relation of at most five attributes,
+  // from 3 2^19 tuples (one view at a time against the planes: 15 views of four attributes, m = 2^16,
+  // d = 9, 2^21 tuples 1.17 against 0.52 ms; three views of two 0.37 against 0.16).  They would pay below
+  // that too, but callers count the two launches per view of smaller batches.
+  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)3 << 19)) {
     ViewMasks vm;
+    ViewCounters vc;
     vm.nv = 0;
-    unsigned long long* vctr[SK_MAX_VIEWS];
     for (int v = 0; v < nv; v++)
       if (amask[v]) {
-        vctr[vm.nv] = ctr[v];
+        vc.ctr[vm.nv] = ctr[v];
         vm.mask[vm.nv++] = (uint8_t)amask[v];
       }
-    const int64_t W = view_window(std::max(1, vm.nv), a.d, n);
-    const size_t vbytes = view_items_bytes(vm.nv, a.d, W, sms) +
-                          (size_t)vm.nv * sms * kPartMaxCtasPerSm * 16 * sizeof(uint32_t);
-    if (vm.nv > 0 && pool_malloc_async(&staging, vbytes, st) == cudaSuccess) {
+    const int64_t W = view_window(a.a, a.d, n);
+    if (vm.nv > 0 && pool_malloc_async(&staging, view_plane_bytes(a.a, a.d, W), st) == cudaSuccess) {
       *done = true;
       t.tbl = (uint32_t*)tbl;
       cudaError_t e = launch_table_l24(a, t, nullptr, (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32), st);
-      if (e == cudaSuccess) e = run_partitioned_views(a, t, vm, vctr, staging, W, sms, st);
+      if (e == cudaSuccess) e = run_views(a, t, vm, vc, staging, W, sms, st);
       cudaError_t ef = cudaFreeAsync(tbl, st);
       const cudaError_t es = cudaFreeAsync(staging, st);
       if (ef == cudaSuccess) ef = es;
       return set_status_from_cuda(e != cudaSuccess ? e : ef);
     }
-    cudaGetLastError();   // no room for the views' items: one view at a time
+    cudaGetLastError();   // no room for the planes: one view at a time
     staging = nullptr;
   }
   const size_t sbytes = part_staging_bytes(a.d, part_window(n), sms);

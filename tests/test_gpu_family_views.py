@@ -35,3 +35,10 @@ def test_equals_per_tuple_views(k, logm, d, n, window, subs, monkeypatch):
         got.append([f.sketch(i, 0) for i in range(len(queries))])
         f.close()
     assert all((x == y).all() for x, y in zip(*got))
+
+
+@pytest.mark.parametrize("k,logm,d,n,window", [
+    (3, 15, 9, 3 << 19, 0), (2, 16, 1, (3 << 19) + 1, 0), (4, 16, 8, 1_600_001, 8193), (5, 14, 9, 1_599_999, 500_000)])
+def test_tile_edges(k, logm, d, n, window, monkeypatch):
+    """One part and two, one row, 45 planes, windows that end inside a tile of 8192 tuples."""
+    test_equals_per_tuple_views(k, logm, d, n, window, "all", monkeypatch)
