@@ -2937,7 +2937,8 @@ sk_status ntt_groups(sk_set** sets, const std::map<int64_t, std::vector<int>>& g
     const int64_t** h_rows = (const int64_t**)meta.data();
     uint8_t* h_dirs = (uint8_t*)(meta.data() + b_rows);
     ntt::Out* h_outs = (ntt::Out*)(meta.data() + b_rows + b_dirs);
-    size_t v_words = 0, o = 0;
+    size_t v_words = 0, v_one = 0, o = 0;
+    int most = kFuMaxPrimes;   // primes at once
     for (Group& g : gs) {
       for (Member& mb : g.sets) {
         const sk_set* s = sets[mb.i];
@@ -2976,11 +2977,19 @@ sk_status ntt_groups(sk_set** sets, const std::map<int64_t, std::vector<int>>& g
       }
       const size_t words = (size_t)g.nvec_at[0] * g.M;
       if (words) v_words = std::max(v_words, words * ntt_primes_at_once(words, g.np));
+      v_one = std::max(v_one, words);
     }
     if (!v_words) return SK_OK;
     SK_CK(cudaMemcpyAsync(blk, meta.data(), meta.size(), cudaMemcpyHostToDevice, st));
     SK_CK(cudaMemsetAsync(d_sums, 0, b_sums, st));
-    SK_CK(pool_malloc_async((void**)&V, v_words * sizeof(uint32_t), st));
+    cudaError_t ea = pool_malloc_async((void**)&V, v_words * sizeof(uint32_t), st);
+    if (ea == cudaErrorMemoryAllocation && v_one < v_words) {   // little room: one prime at a time
+      cudaGetLastError();
+      most = 1;
+      ea = pool_malloc_async((void**)&V, v_one * sizeof(uint32_t), st);
+    }
+    if (ea != cudaSuccess) V = nullptr;
+    SK_CK(ea);
     for (const Group& g : gs) {
       if (!g.np) continue;
       ntt::ColArgs ca;
@@ -3003,7 +3012,7 @@ sk_status ntt_groups(sk_set** sets, const std::map<int64_t, std::vector<int>>& g
         ca.nvec[i] = g.nvec_at[i];
         ra.nout[i] = g.nout_at[i];
       }
-      const int at_once = ntt_primes_at_once((size_t)ca.stride * g.M, g.np);
+      const int at_once = std::min(most, ntt_primes_at_once((size_t)ca.stride * g.M, g.np));
       for (int i = 0; i < g.np; i += at_once) {
         ca.prime0 = ra.prime0 = i;
         SK_CK(ntt::cols(ca, g.nvec_at[i], std::min(at_once, g.np - i), st));
