@@ -1864,8 +1864,9 @@ bool fu_eligible(const sk_set* s, unsigned long long* negmask) {
 }
 
 // Fills the current device's root tables of sk_ntt.cuh (about 1.3 MB, a few milliseconds of
-// host arithmetic, once per device and process).
-cudaError_t ntt_constants() {
+// host arithmetic, once per device and process).  Stream-ordered on st; the host data are
+// pageable, so they are read before each call returns.
+cudaError_t ntt_constants(cudaStream_t st) {
   const std::vector<FuPrime>& pr = fu_primes();
   constexpr int NP = ntt::kMaxPrimes, NL = ntt::kMaxLog - ntt::kMinLog + 1;
   static_assert(NP == kFuMaxPrimes, "one table per CRT prime");
@@ -1899,10 +1900,12 @@ cudaError_t ntt_constants() {
       for (int j = 0; j < 32; j++) pc[i].w64[dir][j] = factor(64 * j);
     }
   }
-  cudaError_t e = cudaMemcpyToSymbol(ntt::g_root, root.data(), root.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_low, low.data(), low.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::g_row, row.data(), row.size() * sizeof(ntt::Factor));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(ntt::c_prime, pc.data(), pc.size() * sizeof(ntt::PrimeConst));
+  constexpr cudaMemcpyKind up = cudaMemcpyHostToDevice;
+  cudaError_t e = cudaMemcpyToSymbolAsync(ntt::g_root, root.data(), root.size() * 4, 0, up, st);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(ntt::g_low, low.data(), low.size() * 4, 0, up, st);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(ntt::g_row, row.data(), row.size() * sizeof(ntt::Factor), 0, up, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(ntt::c_prime, pc.data(), pc.size() * sizeof(ntt::PrimeConst), 0, up, st);
   return e;
 }
 
@@ -1926,8 +1929,11 @@ std::mutex g_fu_const_mutex;
 bool g_fu_const_ready[64] = {false};
 
 // Uploads the primes' constants to the current device once; *ready false when the fused
-// form cannot run here (fewer primes than needed, device index beyond the table).
-cudaError_t fu_constants(bool* ready) {
+// form cannot run here (fewer primes than needed, device index beyond the table).  The first
+// call waits for its copies on st: what reads the constants may run on any stream, the estimate
+// workers' non-blocking ones included, and a copy from pageable memory can return before its
+// last bytes are on the device.
+cudaError_t fu_constants(bool* ready, cudaStream_t st) {
   *ready = false;
   const std::vector<FuPrime>& pr = fu_primes();
   if ((int)pr.size() < kFuMaxPrimes) return cudaSuccess;
@@ -1941,9 +1947,10 @@ cudaError_t fu_constants(bool* ready) {
       ps[i] = pr[i].p;
       pis[i] = pr[i].pinv;
     }
-    cudaError_t e = cudaMemcpyToSymbol(c_fu_p, ps, sizeof(ps));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_fu_pinv, pis, sizeof(pis));
-    if (e == cudaSuccess) e = ntt_constants();
+    cudaError_t e = cudaMemcpyToSymbolAsync(c_fu_p, ps, sizeof(ps), 0, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_fu_pinv, pis, sizeof(pis), 0, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = ntt_constants(st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
     g_fu_const_ready[dev] = true;
   }
@@ -2366,7 +2373,7 @@ sk_status run_estimate_crt(sk_set* s, sk_estimate* out, cudaStream_t st, bool* d
 sk_status run_estimate_fused(sk_set* s, sk_estimate* out, cudaStream_t st, bool* done) {
   *done = false;
   bool ready = false;
-  SK_CK(fu_constants(&ready));
+  SK_CK(fu_constants(&ready, st));
   if (!ready) return SK_OK;
   SK_CK_ST(run_estimate_pairwise(s, out, st, done));
   if (*done) return SK_OK;
@@ -3053,7 +3060,7 @@ sk_status run_estimate_many(sk_set** sets, int n, sk_estimate* out, cudaStream_t
   // fused groups by width, on the caller's stream
   std::map<int64_t, std::vector<int>> groups;
   bool ready = false;
-  SK_CK(fu_constants(&ready));
+  SK_CK(fu_constants(&ready, st));
   for (int i = 0; i < n; i++) {
     sk_set* s = sets[i];
     unsigned long long nm = 0;
