@@ -310,12 +310,28 @@ __device__ __forceinline__ void add_tuple_key(const UpdArgs& p, const uint64_t* 
   }
 }
 
+// Sum of delta over the lanes of `same` (each lane's own group), modulo 2^64: one ballot per bit
+// of the warp's largest magnitude, positive and negative lanes counted apart.  The cost is the
+// same whatever the groups are; a reduction instruction per group runs the groups one after another
+// (1e7 uniform 64-bit keys with weights +-1, m = 10^6, d = 5: 542 us, 394 without any merging).
+__device__ __forceinline__ int64_t group_sum(unsigned same, int64_t delta) {
+  const uint64_t mag = delta < 0 ? 0ull - (uint64_t)delta : (uint64_t)delta;
+  const unsigned neg = __ballot_sync(0xffffffffu, delta < 0);
+  const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(mag >> 32));
+  const int bits = hi ? 64 - __clz(hi) : 32 - __clz(__reduce_or_sync(0xffffffffu, (uint32_t)mag));
+  uint64_t sum = 0;
+  for (int b = 0; b < bits; b++) {
+    const unsigned set = __ballot_sync(0xffffffffu, (mag >> b) & 1ull) & same;
+    sum += (uint64_t)(int64_t)(__popc(set) - 2 * __popc(set & neg)) << b;
+  }
+  return (int64_t)sum;
+}
+
 // Algorithm 2 for one warp's 32 consecutive tuples of a one-attribute relation into the int64
 // counters: lanes with the same key (field element) have the same bins and signs, so their
 // weights are added first and one lane hashes and updates for all.  Skewed keys otherwise queue
 // at their counters in L2: 1e6 skewed tuples, m = 10^6, d = 5, 56 us against 150; uniform keys
 // 29 against 33 (m = 2^16, d = 9: 69 against 170 and 44 against 43; a match on 64-bit values only: 45).
-// Weights of 2^25 and more in the warp: every lane for itself (the sum is 32 bits).
 template <bool POW2, bool DEG1>
 __device__ __forceinline__ void update_warp_key(const UpdArgs& p, const uint64_t* s_coef, int64_t i, bool live) {
   const int64_t key = live ? ld_key_stream(p.cols + i) : 0;
@@ -327,15 +343,10 @@ __device__ __forceinline__ void update_warp_key(const UpdArgs& p, const uint64_t
   const unsigned same = __all_sync(0xffffffffu, ok && (x >> 32) == 0)
                             ? __match_any_sync(0xffffffffu, (uint32_t)x)
                             : __match_any_sync(0xffffffffu, ok ? x : kP61 + lane);   // field elements are below p
-  if (!p.w) {
-    delta = __popc(same);
-  } else if (__all_sync(0xffffffffu, delta < (1 << 25) && delta > -(1 << 25))) {
-    delta = __reduce_add_sync(same, (int)delta);
-  } else {
-    add_tuple_key<POW2, DEG1>(p, s_coef, x, delta, ok);
-    return;
-  }
-  add_tuple_key<POW2, DEG1>(p, s_coef, x, delta, ok && lane == (unsigned)(__ffs(same) - 1));
+  const bool first = lane == (unsigned)(__ffs(same) - 1);
+  if (!p.w) delta = __popc(same);
+  else if (!__all_sync(0xffffffffu, first)) delta = group_sum(same, delta);   // else all keys differ
+  add_tuple_key<POW2, DEG1>(p, s_coef, x, delta, ok && first);
 }
 
 // Record of attribute u for key x (< 2^31: the field element is the key itself).
