@@ -68,16 +68,51 @@ __global__ void __launch_bounds__(256) k_update(UpdArgs p, const int* unless) {
   }
 }
 
+// Whether a weighted batch's weights suit the items: set by the table kernel, which runs before
+// both phases, from 1024 tuples of the batch.
+struct PartChoice {
+  int direct;   // most weights are beyond wmax: every tuple straight to the counters
+};
+
+struct WeightSample {
+  const int64_t* w;        // nullptr: unit weights
+  int64_t n;
+  int64_t wmax;            // the largest |Delta| an item holds
+  PartChoice* choice;
+};
+
+// By the table kernel's last CTA (of 256 threads), which then has no keys.  Weights beyond wmax cost
+// their reductions and what the items of the others cost besides; with few of them the items win:
+// 7e7 tuples of two columns, m = 2^16, d = 9: 2090 us with none, 2110 with a tenth, 3460 with three
+// quarters, 4180 with nearly all, against 3720 for reductions alone.  The line is at 0.7.
+__device__ __forceinline__ void choose_path(const WeightSample& s) {
+  bool far[4];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const int64_t j = 256 * k + threadIdx.x;
+    const int64_t w = __ldg(s.w + (s.n >> 10) * j + (((s.n & 1023) * j) >> 10));
+    far[k] = w > s.wmax || w < -s.wmax;
+  }
+  int beyond = 0;
+#pragma unroll
+  for (int k = 0; k < 4; k++) beyond += __syncthreads_count(far[k]);
+  if (threadIdx.x == 0) s.choice->direct = beyond > 717;
+}
+
 // Key-table records for every declared domain key of every attribute (one thread per key).
 template <bool POW2, bool DEG1>
-__global__ void __launch_bounds__(256) k_key_table(UpdArgs p, TabArgs t) {
+__global__ void __launch_bounds__(256) k_key_table(UpdArgs p, TabArgs t, WeightSample ws) {
+  if (ws.w && blockIdx.x == gridDim.x - 1) {
+    choose_path(ws);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* s_coef = (uint64_t*)smem_raw;
   const int ncoef = p.d * p.row_len;
   for (int i = threadIdx.x; i < ncoef; i += blockDim.x) s_coef[i] = p.coef[i];
   __syncthreads();
   const int64_t total = t.base[p.a];
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t step = (int64_t)(gridDim.x - (ws.w ? 1u : 0u)) * blockDim.x;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
     int u = 0;
     while (u + 1 < p.a && g >= t.base[u + 1]) u++;
@@ -156,6 +191,7 @@ struct PartArgs {
   const uint32_t* vbits;         // nullptr, or bit (i mod 32) of word i / 32: window tuple i is kept
   const int64_t* wts;            // weighted: Delta of the window's first tuple (items are uint32_t)
   int64_t wmax;                  // weighted: |Delta| <= wmax < 2^16 goes into an item
+  PartChoice* choice;            // weighted
   const int* go;                 // nullptr, or both phases return at once when it reads 0
 };
 
@@ -181,14 +217,18 @@ __device__ __forceinline__ int64_t ld_key_policy(const int64_t* ptr, uint64_t po
 
 // Key-table records in the 20-bit lane format above (d <= 9, one thread per domain key).
 template <bool DEG1>
-__global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t) {
+__global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t, WeightSample ws) {
+  if (ws.w && blockIdx.x == gridDim.x - 1) {
+    choose_path(ws);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* s_coef = (uint64_t*)smem_raw;
   const int ncoef = p.d * p.row_len;
   for (int i = threadIdx.x; i < ncoef; i += blockDim.x) s_coef[i] = p.coef[i];
   __syncthreads();
   const int64_t total = t.base[p.a];
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t step = (int64_t)(gridDim.x - (ws.w ? 1u : 0u)) * blockDim.x;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += step) {
     int u = 0;
     while (u + 1 < p.a && g >= t.base[u + 1]) u++;
@@ -230,8 +270,13 @@ struct FoundDomains {
 // the first 8 bytes hold word 2 and the aligned pair after it words 0 and 1, so a reader
 // always takes words 0 and 1 with one 16-byte load and word 2 with one 8-byte load.
 template <bool DEG1>
-__global__ void __launch_bounds__(256) k_key_table_l24(UpdArgs p, TabArgs t, const FoundDomains* found) {
+__global__ void __launch_bounds__(256) k_key_table_l24(UpdArgs p, TabArgs t, const FoundDomains* found,
+                                                       WeightSample ws) {
   if (found && !found->go) return;
+  if (ws.w && blockIdx.x == gridDim.x - 1) {
+    choose_path(ws);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* s_coef = (uint64_t*)smem_raw;
   const int ncoef = p.d * p.row_len;
@@ -243,7 +288,7 @@ __global__ void __launch_bounds__(256) k_key_table_l24(UpdArgs p, TabArgs t, con
     total = 0;
     for (int u = 0; u < p.a; u++) total += (int64_t)found->top[u] + 1;
   }
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t step = (int64_t)(gridDim.x - (ws.w ? 1u : 0u)) * blockDim.x;
   uint64_t* tbl = (uint64_t*)t.tbl;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
     int u = 0;
@@ -281,6 +326,78 @@ __device__ __forceinline__ void ld_record24(const uint64_t* tbl, uint64_t k, uin
   asm("ld.global.nc.u64 %0, [%1];" : "=l"(w2) : "l"(r + 2 - 2 * odd));
 }
 
+// A weighted window's tuples straight to the int64 counters, from k_tab_items' records (FMT as
+// there).  The grid has direct_ctas CTAs for each resident one: with resident CTAs alone, each with a
+// fixed share, the SMs whose reductions take longest hold up the rest (2e7 tuples of five uniform
+// columns, m = 2^16, d = 9: 1450 us, with four 1275 and with a CTA per 256 tuples 1250; the occupancy
+// makes no difference, and claims from a counter wait behind the reductions).  Batches that have
+// items pay for the CTAs that return at once, 1 us per 2000.
+template <int A, int FMT>
+__device__ __forceinline__ void add_direct(const UpdArgs& p, const TabArgs& t, const PartArgs& q) {
+  const uint32_t mask = (uint32_t)p.m - 1u;
+  const int d = p.d;
+  const int64_t step = (int64_t)gridDim.x * 256;
+  for (int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x; g < q.cnt; g += step) {
+    int64_t key[A];
+#pragma unroll
+    for (int u = 0; u < A; u++) key[u] = ld_key_stream(q.col[u] + g);
+    const int64_t delta = ld_key_stream(q.wts + g);
+    bool ok = true;
+#pragma unroll
+    for (int u = 0; u < A; u++) ok = ok && (uint64_t)key[u] < (uint64_t)p.dom[u];
+    if (!ok) {
+      record(p.status, SK_ERR_KEY_OUT_OF_DOMAIN);
+      continue;
+    }
+    auto put = [&](int j, uint32_t bin, bool neg) {
+      red_add_global(p.ctr + (int64_t)j * p.m + (bin & mask), (unsigned long long)(neg ? -delta : delta));
+    };
+    if constexpr (FMT == 1) {
+      uint32_t b2[7] = {0, 0, 0, 0, 0, 0, 0}, sg = 0;   // two rows per word, halves without carry
+#pragma unroll
+      for (int u = 0; u < A; u++) {
+        uint32_t w[8];
+        ld_record32((const uint4*)t.tbl + (uint64_t)(t.base[u] + key[u]) * 2, w);
+        sg ^= w[7];
+#pragma unroll
+        for (int j = 0; j < 7; j++) b2[j] = add16x2(b2[j], w[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 14; j++) {
+        if (j >= d) break;
+        put(j, b2[j >> 1] >> (16 * (j & 1)), (sg >> j) & 1u);
+      }
+    } else {
+      constexpr int B = FMT == 2 ? 22 : 20;   // bits per row of a record word
+      uint64_t acc[3] = {0, 0, 0};
+      uint32_t sg = 0;
+#pragma unroll
+      for (int u = 0; u < A; u++) {
+        if constexpr (FMT == 2) {
+          uint64_t w0, w1, w2;
+          ld_record24((const uint64_t*)t.tbl, (uint64_t)(t.base[u] + key[u]), w0, w1, w2);
+          acc[0] += w0;
+          acc[1] += w1;
+          acc[2] += w2;
+        } else {
+          uint32_t w[8];
+          ld_record32((const uint4*)t.tbl + (uint64_t)(t.base[u] + key[u]) * 2, w);
+          acc[0] += ((uint64_t)w[1] << 32) | w[0];
+          acc[1] += ((uint64_t)w[3] << 32) | w[2];
+          acc[2] += ((uint64_t)w[5] << 32) | w[4];
+          sg ^= w[7];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 9; j++) {
+        if (j >= d) break;
+        const uint32_t x = (uint32_t)(acc[j / 3] >> (B * (j % 3)));
+        put(j, x, FMT == 2 ? (x >> 19) & 1u : (sg >> j) & 1u);
+      }
+    }
+  }
+}
+
 // FMT 0: 20-bit lane records (d <= 9); FMT 2: 24-byte records (d <= 9, k_key_table_l24);
 // FMT 1: narrow 16-bit records of 32 bytes (d <= 14):
 // per record word holding the bins of rows 2j and 2j + 1, lo[j] adds the low halves (below
@@ -304,13 +421,16 @@ __device__ __forceinline__ void ld_record24(const uint64_t* tbl, uint64_t k, uin
 // records need.
 //
 // WT (weighted batches): items are 32 bits, the bin's offset in bits 0..14 and Delta times the
-// sign above; a tuple with |Delta| > wmax goes to the int64 counters directly.
+// sign above; a tuple with |Delta| > wmax goes to the int64 counters directly, and every tuple
+// does when the batch's sample says that most have such weights (choose_path, add_direct).
 template <int A, int FMT, bool WT>
 __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, PartArgs q) {
   if (q.go && !*q.go) return;
+  const bool direct = WT && q.choice->direct != 0;
+  if (WT && (int)blockIdx.x * 8 >= q.nwarps && !direct) return;   // a CTA for add_direct only
   using Item = typename std::conditional<WT, uint32_t, uint16_t>::type;
   constexpr bool HELD = WT && FMT != 1;
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t step = (int64_t)q.nwarps * 32;
   const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
   const uint32_t mask = (uint32_t)p.m - 1u;
   const uint32_t low = (1u << q.logL) - 1u;
@@ -340,6 +460,12 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
     kx[u] = kin ? (uint32_t)k : 0u;
   }
   if (WT && g < q.cnt) wn = ld_key_policy(q.wts + g, pol);
+  if constexpr (WT) {
+    if (direct) {   // asked after the first keys' loads: the answer arrives with them
+      add_direct<A, FMT>(p, t, q);
+      return;
+    }
+  }
   for (; g < gend; g += step) {
     const bool in = g < q.cnt;
     const bool whole = in && okm == (1u << A) - 1u && (!q.vbits || ((q.vbits[g >> 5] >> lane) & 1u));
@@ -399,7 +525,11 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
         }
       }
       if (WT && whole && !ok) {
-        for (int j = 0; j < d; j++) far(j, (uint32_t)(acc[j / 3] >> (20 * (j % 3))), ((sg >> j) & 1u) << 15);
+#pragma unroll
+        for (int j = 0; j < 9; j++) {
+          if (j >= d) break;
+          far(j, (uint32_t)(acc[j / 3] >> (20 * (j % 3))), ((sg >> j) & 1u) << 15);
+        }
         acc[0] = acc[1] = acc[2] = 0;
       }
 #pragma unroll
@@ -534,6 +664,7 @@ __global__ void __launch_bounds__(1024) k_part_accum(PartArgs q, unsigned long l
                                                      int logL, int R, int logP) {
   constexpr int LI = WT ? 2 : 3, I = 1 << LI;   // items per 16-byte chunk
   if (q.go && !*q.go) return;
+  if (WT && q.choice->direct) return;   // no items
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int* cnt = (int*)smem_raw;
   const int S = (int)(m >> logL);
@@ -891,8 +1022,11 @@ size_t part_items_bytes(int d, int64_t W, int sms, bool weighted) {
   return ((size_t)d * (size_t)(W + threads) * (weighted ? sizeof(uint32_t) : sizeof(uint16_t)) + 255) & ~(size_t)255;
 }
 
+size_t part_counts_bytes(int sms) { return (size_t)sms * kPartMaxCtasPerSm * 8 * 16 * sizeof(uint32_t); }
+
+// Items, the warps' counts, and for weighted batches a PartChoice.
 size_t part_staging_bytes(int d, int64_t W, int sms, bool weighted = false) {
-  return part_items_bytes(d, W, sms, weighted) + (size_t)sms * kPartMaxCtasPerSm * 8 * 16 * sizeof(uint32_t);
+  return part_items_bytes(d, W, sms, weighted) + part_counts_bytes(sms) + (weighted ? 256 : 0);
 }
 
 // Phase 2 over the regions of a window: R and the pieces per region follow from part_ranges.
@@ -918,56 +1052,102 @@ PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps) {
   return p;
 }
 
+// The kernels and the launch shape of both phases for one relation.
+struct PartPlan {
+  TabItemsKernel items;
+  void (*accum)(PartArgs, unsigned long long*, int64_t, int, int, int, int);
+  int64_t W;           // tuples per window
+  int64_t full_grid;   // phase-1 CTAs, all resident
+  int64_t units;       // (row, part) pairs
+  int64_t slots;       // resident phase-2 CTAs
+  int logL;
+  size_t smem;
+};
+
+cudaError_t part_plan(const UpdArgs& a, int fmt, int sms, int64_t most, PartPlan* pl) {
+  const bool weighted = a.w != nullptr;
+  pl->items = tab_items_kernel(a.a, fmt, weighted);
+  pl->accum = weighted ? k_part_accum<true> : k_part_accum<false>;
+  int per_sm = 1;
+  cudaError_t e = tab_items_per_sm(pl->items, &per_sm);
+  if (e != cudaSuccess) return e;
+  pl->full_grid = (int64_t)sms * per_sm;
+  pl->W = part_window(a.n, most);
+  int logm = 0;
+  while (((int64_t)1 << logm) < (int64_t)a.m) logm++;
+  pl->logL = std::min(logm, 15);
+  pl->smem = (size_t)4 << pl->logL;
+  e = allow_dynamic_smem((const void*)pl->accum);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pl->accum, 1024, pl->smem);
+  pl->slots = (int64_t)sms * std::max(1, per_sm);
+  pl->units = (int64_t)(a.m >> pl->logL) * a.d;
+  return e;
+}
+
+// Phase-1 grid and regions of a window of cnt tuples, its phase-2 split and the largest |Delta|
+// of an item: a phase-2 counter sums at most R C items, below 2^31 in magnitude.
+int part_regions(const PartPlan& pl, int d, int64_t cnt, PartArgs* q, PartSplit* sp) {
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((cnt + 255) / 256, pl.full_grid));
+  const int64_t gend = (cnt + 31) / 32 * 32;
+  q->cnt = cnt;
+  q->C = 32 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
+  q->nwarps = grid * 8;
+  *sp = part_split(cnt * d, pl.units, pl.slots, q->nwarps);
+  q->wmax = std::min<int64_t>(65535, 0x7fffffff / ((int64_t)sp->R * q->C));
+  return grid;
+}
+
+// CTAs of a weighted window per resident one (add_direct): one per 400 000 tuples, 4 to 20.
+int direct_ctas(int64_t cnt) { return (int)std::min<int64_t>(20, std::max<int64_t>(4, cnt / 400000)); }
+
+// What the table kernel samples of a weighted batch (of its first window's limit; a shorter last
+// window's is larger).
+cudaError_t weight_sample(const UpdArgs& a, int fmt, void* staging, int sms, int64_t most, WeightSample* ws) {
+  *ws = {nullptr, a.n, 0, nullptr};
+  if (!a.w) return cudaSuccess;
+  PartPlan pl;
+  const cudaError_t e = part_plan(a, fmt, sms, most, &pl);
+  if (e != cudaSuccess) return e;
+  PartArgs q;
+  PartSplit sp;
+  part_regions(pl, a.d, std::min(pl.W, a.n), &q, &sp);
+  *ws = {a.w, a.n, q.wmax,
+         (PartChoice*)((char*)staging + part_items_bytes(a.d, pl.W, sms, true) + part_counts_bytes(sms))};
+  return cudaSuccess;
+}
+
 // Both phases over every window of the batch; staging (part_staging_bytes) is caller-owned.
 // colp: the first tuple's key of each of the a.a attributes (nullptr: a.cols + u a.stride).
 // vbits: nullptr, or one bit per batch tuple (bit i mod 32 of word i / 32) that must be set
-// for the tuple to be added.  most: tuples per window at most.  go: see PartArgs.
+// for the tuple to be added.  most: tuples per window at most.  go: see PartArgs.  A weighted batch's
+// table kernel has been given weight_sample's.
 cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* staging, int sms, cudaStream_t st,
                             const int64_t* const* colp = nullptr, const uint32_t* vbits = nullptr,
                             int64_t most = (int64_t)1 << 30, const int* go = nullptr) {
   const int64_t n = a.n;
   const bool weighted = a.w != nullptr;
-  TabItemsKernel items = tab_items_kernel(a.a, fmt, weighted);
-  auto accum = weighted ? k_part_accum<true> : k_part_accum<false>;
-  int tab_per_sm = 1;
-  cudaError_t e = tab_items_per_sm(items, &tab_per_sm);
+  PartPlan pl;
+  cudaError_t e = part_plan(a, fmt, sms, most, &pl);
   if (e != cudaSuccess) return e;
-  const int64_t full_grid = (int64_t)sms * tab_per_sm;
-  const int64_t W = part_window(n, most);
   PartArgs q;
   q.go = go;
   q.items = staging;
-  q.cnts = (uint32_t*)((char*)staging + part_items_bytes(a.d, W, sms, weighted));
-  q.W = W;
-  int logm = 0;
-  while (((int64_t)1 << logm) < (int64_t)a.m) logm++;
-  const int logL = std::min(logm, 15);
-  q.logL = logL;
-  const int S = (int)(a.m >> logL);
-  const size_t smem = (size_t)4 << logL;
-  e = allow_dynamic_smem((const void*)accum);
-  int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accum, 1024, smem);
-  const int64_t slots = (int64_t)sms * std::max(1, per_sm);
-  const int64_t units = (int64_t)S * a.d;
-  for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += W) {
-    q.cnt = std::min(W, n - i0);
+  q.cnts = (uint32_t*)((char*)staging + part_items_bytes(a.d, pl.W, sms, weighted));
+  q.choice = weighted ? (PartChoice*)((char*)q.cnts + part_counts_bytes(sms)) : nullptr;
+  q.W = pl.W;
+  q.logL = pl.logL;
+  for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += pl.W) {
+    PartSplit sp;
+    const int grid = part_regions(pl, a.d, std::min(pl.W, n - i0), &q, &sp);
     for (int u = 0; u < 5; u++)
       q.col[u] = u < a.a ? (colp ? colp[u] : a.cols + (int64_t)u * a.stride) + i0 : nullptr;
     q.vbits = vbits ? vbits + i0 / 32 : nullptr;   // windows start at multiples of 256
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((q.cnt + 255) / 256, full_grid));
-    const int64_t gend = (q.cnt + 31) / 32 * 32;
-    q.C = 32 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
-    q.nwarps = grid * 8;
-    const PartSplit sp = part_split(q.cnt * a.d, units, slots, q.nwarps);
-    // a phase-2 counter sums at most R C weighted items: below 2^31 in magnitude
     q.wts = weighted ? a.w + i0 : nullptr;
-    q.wmax = std::min<int64_t>(65535, 0x7fffffff / ((int64_t)sp.R * q.C));
-    items<<<grid, 256, 0, st>>>(a, t, q);
+    pl.items<<<weighted ? grid * direct_ctas(q.cnt) : grid, 256, 0, st>>>(a, t, q);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
-    accum<<<(unsigned)(units * sp.nr), 1024, smem, st>>>(q, a.ctr, (int64_t)a.m, a.d, logL, sp.R, sp.logP);
+    pl.accum<<<(unsigned)(pl.units * sp.nr), 1024, pl.smem, st>>>(q, a.ctr, (int64_t)a.m, a.d, pl.logL, sp.R, sp.logP);
     count_launch();
     e = cudaGetLastError();
   }
@@ -2089,12 +2269,13 @@ bool in_device_memory(const int64_t* cols) {
 }
 
 // 24-byte key records of the declared domains, or of the found ones.
-cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDomains* found, int grid, cudaStream_t st) {
+cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDomains* found, int grid, cudaStream_t st,
+                             const WeightSample& ws = {}) {
   auto kern = all_deg1(a) ? k_key_table_l24<true> : k_key_table_l24<false>;
   const size_t smem = (size_t)a.d * a.row_len * sizeof(uint64_t);
   const cudaError_t e = fit_dynamic_smem((const void*)kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, 256, smem, st>>>(a, t, found);
+  kern<<<grid + (ws.w ? 1 : 0), 256, smem, st>>>(a, t, found, ws);
   count_launch();
   return cudaGetLastError();
 }
@@ -2217,7 +2398,9 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   }
   count_launch(2);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_table_l24(a, t, f, sms * 32, st);
+  WeightSample ws = {};
+  if (e == cudaSuccess) e = weight_sample(a, 2, buf, sms, (int64_t)1 << 26, &ws);
+  if (e == cudaSuccess) e = launch_table_l24(a, t, f, sms * 32, st, ws);
   if (e == cudaSuccess) e = run_partitioned(a, t, 2, buf, sms, st, nullptr, nullptr, (int64_t)1 << 26, &f->go);
   // a fixed grid, whose CTAs return at once in the dense case: 1e7 dense tuples 538 us in all with
   // 32 CTAs per SM, 552 with a tuple per thread; sparse ones measured the same
@@ -2345,15 +2528,17 @@ sk_status launch_update(sk_set* s, int relation, int64_t n, const int64_t* cols,
         a.smem_wmax = 0;
         const bool d1 = all_deg1(a);
         const int bgrid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sms * 32);
-        if (part && part_fmt == 2) {
-          e = launch_table_l24(a, t, nullptr, bgrid, st);
-        } else {
+        WeightSample ws = {};
+        e = part ? weight_sample(a, part_fmt, staging, sms, part_most(weights), &ws) : cudaSuccess;
+        if (e == cudaSuccess && part && part_fmt == 2) {
+          e = launch_table_l24(a, t, nullptr, bgrid, st, ws);
+        } else if (e == cudaSuccess) {
           auto kb = (part && part_fmt == 0) ? (d1 ? k_key_table_l20<true> : k_key_table_l20<false>)
                     : pow2 ? (d1 ? k_key_table<true, true> : k_key_table<true, false>)
                            : (d1 ? k_key_table<false, true> : k_key_table<false, false>);
           e = fit_dynamic_smem((const void*)kb, coef_bytes);
           if (e == cudaSuccess) {
-            kb<<<bgrid, 256, coef_bytes, st>>>(a, t);
+            kb<<<bgrid + (ws.w ? 1 : 0), 256, coef_bytes, st>>>(a, t, ws);
             count_launch();
             e = cudaGetLastError();
           }
