@@ -250,11 +250,12 @@ __global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t, Wei
   }
 }
 
-// The largest key of each attribute of a batch whose domains were not declared.
+// What the kernels find out about a batch whose domains were not declared.
 struct FoundDomains {
-  unsigned long long top[5];
-  int go;        // every key is dense enough for the tables
-  int blocks;    // CTAs of the scan that are done
+  unsigned long long top[5];   // the largest key of each attribute
+  float spread[5];             // distinct keys among 1024 of the batch, as a share
+  int go;                      // the tables serve
+  int blocks;                  // CTAs of the scan that are done
 };
 
 // Key-table records of 24 bytes (d <= 9, one thread per domain key): rows 3w .. 3w + 2 in
@@ -981,18 +982,24 @@ int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps)
   return std::max<int64_t>(1, std::min<int64_t>(nr, nwarps));
 }
 
-// SK_PART_UPDATE=0 keeps the single-phase k_update_tab (and the per-tuple update) for batches
-// the partitioned updates could take; =2 gives the wide partitioned update every batch whose
-// width, rows, arity and weights it accepts, whatever the sketch's size and the batch length.
-// SK_PART_WINDOW caps the tuples per window (default and largest: 2^30, which keeps every
-// shared-memory counter of k_part_accum below 2^31 in magnitude; 2^24 for the wide update).
-// SK_UNDECLARED_LEAST: the fewest tuples for which update_undeclared looks for dense keys.
+// SK_UNDECLARED_LEAST: the fewest tuples for which update_undeclared looks for dense keys; given, it
+// takes the tables for them whatever they gain.
 int64_t undeclared_least() {
   const char* v = std::getenv("SK_UNDECLARED_LEAST");
   const long long x = v ? std::atoll(v) : 0;
   return x > 0 ? (int64_t)x : (int64_t)1 << 22;
 }
 
+bool undeclared_least_given() {
+  const char* v = std::getenv("SK_UNDECLARED_LEAST");
+  return v && std::atoll(v) > 0;
+}
+
+// SK_PART_UPDATE=0 keeps the single-phase k_update_tab (and the per-tuple update) for batches
+// the partitioned updates could take; =2 gives the wide partitioned update every batch whose
+// width, rows, arity and weights it accepts, whatever the sketch's size and the batch length.
+// SK_PART_WINDOW caps the tuples per window (default and largest: 2^30, which keeps every
+// shared-memory counter of k_part_accum below 2^31 in magnitude; 2^24 for the wide update).
 int part_update_mode() {
   const char* v = std::getenv("SK_PART_UPDATE");
   return (v && v[0] == '0') ? 0 : ((v && v[0] == '2') ? 2 : 1);
@@ -2284,25 +2291,92 @@ cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDoma
 // Batches whose domains were not declared.  Hashing every tuple costs 36 a Horner steps for nine
 // rows; most key columns are dense codes, for which the tables serve as well as declared
 // domains do, but only the data tells.  So, without the host waiting for it: k_dom_probe looks at
-// 1024 tuples (sparse keys are seen there, and the scan is spared); k_dom_scan finds each column's
-// largest key; and either the tables and both phases of the partitioned update run, when every
-// key is below cap records per attribute, or the per-tuple update does: the kernels of the other
-// way return at once on the flag.  Counters are the same either way.
+// 1024 tuples (sparse keys, and domains too wide to pay for, are seen there and the scan is spared);
+// k_dom_scan finds each column's largest key; and either the tables and both phases of the partitioned
+// update run, or the per-tuple update does: the kernels of the other way return at once on the flag.
+// Counters are the same either way.
+//
+// What either way costs (UndeclaredCost), in picoseconds per tuple, fitted to n = 2^22, 1e7 and 3e7
+// tuples of 2, 3 and 5 columns, d = 5 and 9, m = 2^16, keys uniform or Zipf over n / 64 to n / 5:
+//   hashing        2 a d + 1.6 d + 3
+//   tables         1.4 d (2.2 d with weights), and per column a gather: 4.5 from L1 to 7 from L2
+//                  and 20 more beyond L2, which holds about 80 MB of records (both dies keep what both
+//                  read); how many go there, the share of distinct keys in the sample tells: for
+//                  uniform keys (all distinct) the records' share beyond 80 MB, for Zipf exponents of 0.8
+//                  (0.9 distinct) and 1 (0.7) about 0.38 and 0.25 of that
+//   and per batch  2.3 d + 4 per key to build, and 35 us beyond what turning back to hashing costs
+// Without it every dense batch took the tables: 3e7 tuples of five uniform columns over 6e6 keys, d = 5,
+// 4800 us against 1884 for hashing (d = 9: 5370 and 3248); over 4.7e5 keys 1283 (1454).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, uint64_t cap) {
+struct UndeclaredCost {
+  float n;
+  int a, d;
+  bool weighted, always;
+
+  // gain in ps per tuple with `keys` records in the tables and the columns' spreads given
+  __host__ __device__ float gain(float keys, const float* spread) const {
+    const float beyond = fmaxf(0.f, 1.f - 80e6f / fmaxf(24.f * keys, 1.f));
+    float t = (weighted ? 2.2f : 1.4f) * d + (keys * (2.3f * d + 4.f) + 35e6f) / n;
+    for (int u = 0; u < a; u++) {
+      const float l2 = fminf(fmaxf(spread[u] * 2.f - 1.f, 0.f), 1.f);
+      float far = fmaxf((spread[u] - 0.3f) * 0.62f, 0.f);
+      if (spread[u] > 0.965f) far = fminf(1.f, far + (spread[u] - 0.965f) * 30.f);   // uniform: 0.985 and up
+      t += 4.5f + 2.5f * l2 + 20.f * beyond * far;
+    }
+    return 2.f * a * d + 1.6f * d + 3.f - t;
+  }
+  __device__ bool pays(const FoundDomains& f, uint64_t cap) const {
+    float keys = 0.f;
+    bool dense = true;
+    for (int u = 0; u < a; u++) {
+      const unsigned long long top = *(const volatile unsigned long long*)&f.top[u];
+      dense = dense && top < cap;
+      keys += (float)top + 1.f;
+    }
+    return dense && (always || gain(keys, f.spread) > 0.f);
+  }
+};
+
+__global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, uint64_t cap, UndeclaredCost cost) {
+  __shared__ uint32_t s_seen[5][2048];   // 65536 bits per column
   const int64_t i = p.n / 1024 * threadIdx.x;
-  bool dense = true;
-  for (int u = 0; u < p.a; u++) dense = dense && (uint64_t)p.cols[(int64_t)u * p.stride + i] < cap;
-  dense = __syncthreads_and(dense);
+  uint64_t key[5];
+#pragma unroll
+  for (int u = 0; u < 5; u++) key[u] = u < p.a ? (uint64_t)p.cols[(int64_t)u * p.stride + i] : 0ull;
+  for (int k = threadIdx.x; k < 5 * 2048; k += 1024) (&s_seen[0][0])[k] = 0;
   if (threadIdx.x < 5) f->top[threadIdx.x] = 0;
+  bool dense = true;
+#pragma unroll
+  for (int u = 0; u < 5; u++) dense = dense && key[u] < cap;
+  dense = __syncthreads_and(dense);
+  if (!dense) {
+    if (threadIdx.x == 0) f->go = 0;
+    return;
+  }
+  bool fresh[5];
+#pragma unroll
+  for (int u = 0; u < 5; u++) {
+    const uint32_t h = ((uint32_t)key[u] * 2654435761u) >> 16;
+    fresh[u] = u < p.a && !(atomicOr(&s_seen[u][h >> 5], 1u << (h & 31u)) >> (h & 31u) & 1u);
+    if (u < p.a) {
+      const uint32_t top = __reduce_max_sync(0xffffffffu, (uint32_t)key[u]);   // cap is at most 2^31
+      if ((threadIdx.x & 31u) == 0) atomicMax(&f->top[u], (unsigned long long)top);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 5; u++) {
+    const int distinct = __syncthreads_count(fresh[u]);
+    if (threadIdx.x == 0) f->spread[u] = distinct / 1024.f;
+  }
   if (threadIdx.x == 0) {
-    f->go = dense ? 1 : 0;
+    f->go = cost.pays(*f, cap) ? 1 : 0;
     f->blocks = 0;
   }
 }
 
 template <int A>
-__global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, uint64_t cap) {
+__global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, uint64_t cap,
+                                                  UndeclaredCost cost) {
   __shared__ unsigned long long s_top[A];
   if (!f->go) return;
   if (threadIdx.x < A) s_top[threadIdx.x] = 0;
@@ -2341,18 +2415,16 @@ __global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, ui
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(&f->blocks, 1) == (int)gridDim.x - 1) {   // the last CTA decides
     __threadfence();
-    bool dense = true;
-    for (int u = 0; u < A; u++) dense = dense && *(volatile unsigned long long*)&f->top[u] < cap;
-    f->go = dense ? 1 : 0;
+    f->go = cost.pays(*f, cap) ? 1 : 0;
   }
 }
 
 // *done = false (nothing launched) unless the batch is one the partitioned update would take with
-// declared domains, of two attributes or more and at least 2^22 tuples.  Five columns, m = 2^16,
-// d = 9: dense keys 254 against 458 us at 2^22 tuples and 670 against 1810 at 2^24 (1e7
-// tuples 1080 -> 538 us); sparse keys, which pay for the kernels that
-// return, 961 against 938 and 3745 against 3730.  One attribute is left to update_warp_key.
-// Captured streams keep the per-tuple update, which allocates nothing.
+// declared domains, of two attributes or more and at least 2^22 tuples, and keys as kind as can be (few
+// and skewed) would gain 25 us: the probe and the kernels that return cost others 16 to 20 us.  Five columns, m = 2^16,
+// d = 9: dense keys 254 against 458 us at 2^22 tuples and 670 against 1810 at 2^24 (1e7 tuples 1080 ->
+// 538 us).  One attribute is left to update_warp_key.  Captured streams keep the per-tuple
+// update, which allocates nothing.
 cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int sms, cudaStream_t st, bool* done) {
   *done = false;
   const int64_t n = a0.n;
@@ -2364,8 +2436,12 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   if (e != cudaSuccess || cap_st != cudaStreamCaptureStatusNone || !in_device_memory(a0.cols)) return e;
   // records per attribute: a quarter of the tuples (the rule for declared domains), within the
   // tables' limit
-  const int64_t cap = std::min<int64_t>(n / 4, (int64_t)(key_table_max_bytes() / 24) / a0.a);
+  const int64_t cap =
+      std::min<int64_t>({n / 4, (int64_t)(key_table_max_bytes() / 24) / a0.a, ((int64_t)1 << 31) - 1});
   if (cap < 1) return cudaSuccess;
+  const UndeclaredCost cost = {(float)n, a0.a, a0.d, a0.w != nullptr, undeclared_least_given()};
+  const float kind[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  if (!cost.always && (float)n * cost.gain(0.f, kind) < 25e6f) return cudaSuccess;
   const int64_t W = part_window(n, (int64_t)1 << 26);
   const size_t b_part = part_staging_bytes(a0.d, W, sms, a0.w != nullptr), b_tab = ((size_t)a0.a * cap * 24 + 255) & ~(size_t)255;
   char* buf = nullptr;
@@ -2388,13 +2464,13 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   t.rvec = 2;
   t.narrow = 1;
   t.tbl = (uint32_t*)(buf + b_part);
-  k_dom_probe<<<1, 1024, 0, st>>>(a, f, (uint64_t)cap);
+  k_dom_probe<<<1, 1024, 0, st>>>(a, f, (uint64_t)cap, cost);
   const int grid = sms * 8;
   switch (a.a) {
-    case 2: k_dom_scan<2><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
-    case 3: k_dom_scan<3><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
-    case 4: k_dom_scan<4><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
-    default: k_dom_scan<5><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap); break;
+    case 2: k_dom_scan<2><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap, cost); break;
+    case 3: k_dom_scan<3><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap, cost); break;
+    case 4: k_dom_scan<4><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap, cost); break;
+    default: k_dom_scan<5><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap, cost); break;
   }
   count_launch(2);
   e = cudaGetLastError();
