@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(256, 4) k_tab_items(UpdArgs p, TabArgs t, Part
   if (WT && (int)blockIdx.x * 8 >= q.nwarps && !direct) return;   // a CTA for add_direct only
   using Item = typename std::conditional<WT, uint32_t, uint16_t>::type;
   constexpr bool HELD = WT && FMT != 1;
-  const int64_t step = (int64_t)q.nwarps * 32;
+  const int64_t step = WT ? (int64_t)q.nwarps * 32 : (int64_t)gridDim.x * blockDim.x;
   const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
   const uint32_t mask = (uint32_t)p.m - 1u;
   const uint32_t low = (1u << q.logL) - 1u;
