@@ -253,7 +253,8 @@ __global__ void __launch_bounds__(256) k_key_table_l20(UpdArgs p, TabArgs t, Wei
 // What the kernels find out about a batch whose domains were not declared.
 struct FoundDomains {
   unsigned long long top[5];   // the largest key of each attribute
-  float spread[5];             // distinct keys among 1024 of the batch, as a share
+  float spread[5];             // distinct keys among 1024 tuples of the batch, as a share
+  float far;                   // of their weights, the share that no item holds
   int go;                      // the tables serve
   int blocks;                  // CTAs of the scan that are done
 };
@@ -1104,8 +1105,11 @@ int part_regions(const PartPlan& pl, int d, int64_t cnt, PartArgs* q, PartSplit*
   return grid;
 }
 
-// CTAs of a weighted window per resident one (add_direct): one per 400 000 tuples, 4 to 20.
-int direct_ctas(int64_t cnt) { return (int)std::min<int64_t>(20, std::max<int64_t>(4, cnt / 400000)); }
+// CTAs of a weighted window per resident one (add_direct): one per 400 000 tuples, 4 to 20; four
+// when the whole phase may have to return at once (go).
+int direct_ctas(int64_t cnt, const int* go) {
+  return go ? 4 : (int)std::min<int64_t>(20, std::max<int64_t>(4, cnt / 400000));
+}
 
 // What the table kernel samples of a weighted batch (of its first window's limit; a shorter last
 // window's is larger).
@@ -1150,7 +1154,7 @@ cudaError_t run_partitioned(const UpdArgs& a, const TabArgs& t, int fmt, void* s
       q.col[u] = u < a.a ? (colp ? colp[u] : a.cols + (int64_t)u * a.stride) + i0 : nullptr;
     q.vbits = vbits ? vbits + i0 / 32 : nullptr;   // windows start at multiples of 256
     q.wts = weighted ? a.w + i0 : nullptr;
-    pl.items<<<weighted ? grid * direct_ctas(q.cnt) : grid, 256, 0, st>>>(a, t, q);
+    pl.items<<<weighted ? grid * direct_ctas(q.cnt, go) : grid, 256, 0, st>>>(a, t, q);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
@@ -2304,7 +2308,9 @@ cudaError_t launch_table_l24(const UpdArgs& a, const TabArgs& t, const FoundDoma
 //                  read); how many go there, the share of distinct keys in the sample tells: for
 //                  uniform keys (all distinct) the records' share beyond 80 MB, for Zipf exponents of 0.8
 //                  (0.9 distinct) and 1 (0.7) about 0.38 and 0.25 of that
-//   and per batch  2.3 d + 4 per key to build, and 35 us beyond what turning back to hashing costs
+//                  weights that no item holds cost 2.9 d, or when the batch goes straight to the
+//                  counters (add_direct) 6 d + 2.2 a in place of the 2.2 d and the gathers
+//   and per batch  2.3 d + 4 per key to build, and 30 us beyond what turning back to hashing costs
 // Without it every dense batch took the tables: 3e7 tuples of five uniform columns over 6e6 keys, d = 5,
 // 4800 us against 1884 for hashing (d = 9: 5370 and 3248); over 4.7e5 keys 1283 (1454).
 // ---------------------------------------------------------------------------
@@ -2313,36 +2319,42 @@ struct UndeclaredCost {
   int a, d;
   bool weighted, always;
 
-  // gain in ps per tuple with `keys` records in the tables and the columns' spreads given
-  __host__ __device__ float gain(float keys, const float* spread) const {
+  // gain in ps per tuple with `keys` records in the tables, the columns' spreads and the share of
+  // weights that no item holds
+  __host__ __device__ float gain(float keys, const float* spread, float heavy) const {
     const float beyond = fmaxf(0.f, 1.f - 80e6f / fmaxf(24.f * keys, 1.f));
-    float t = (weighted ? 2.2f : 1.4f) * d + (keys * (2.3f * d + 4.f) + 35e6f) / n;
+    const bool direct = heavy > 0.7f;
+    float t = (keys * (2.3f * d + 4.f) + 30e6f) / n;
+    t += direct ? 6.f * d + 2.2f * a : (weighted ? 2.2f : 1.4f) * d + 2.9f * d * heavy;
     for (int u = 0; u < a; u++) {
       const float l2 = fminf(fmaxf(spread[u] * 2.f - 1.f, 0.f), 1.f);
       float far = fmaxf((spread[u] - 0.3f) * 0.62f, 0.f);
       if (spread[u] > 0.965f) far = fminf(1.f, far + (spread[u] - 0.965f) * 30.f);   // uniform: 0.985 and up
-      t += 4.5f + 2.5f * l2 + 20.f * beyond * far;
+      t += (direct ? 0.f : 4.5f + 2.5f * l2) + 20.f * beyond * far;
     }
     return 2.f * a * d + 1.6f * d + 3.f - t;
   }
-  __device__ bool pays(const FoundDomains& f, uint64_t cap) const {
+  // slack: factor on the keys up to the largest (a sample does not show it)
+  __device__ bool pays(const FoundDomains& f, uint64_t cap, float slack) const {
     float keys = 0.f;
     bool dense = true;
     for (int u = 0; u < a; u++) {
       const unsigned long long top = *(const volatile unsigned long long*)&f.top[u];
       dense = dense && top < cap;
-      keys += (float)top + 1.f;
+      keys += slack * ((float)top + 1.f);
     }
-    return dense && (always || gain(keys, f.spread) > 0.f);
+    return dense && (always || gain(keys, f.spread, f.far) > 0.f);
   }
 };
 
-__global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, uint64_t cap, UndeclaredCost cost) {
+__global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, uint64_t cap, UndeclaredCost cost,
+                                                    int64_t wmax) {
   __shared__ uint32_t s_seen[5][2048];   // 65536 bits per column
   const int64_t i = p.n / 1024 * threadIdx.x;
   uint64_t key[5];
 #pragma unroll
   for (int u = 0; u < 5; u++) key[u] = u < p.a ? (uint64_t)p.cols[(int64_t)u * p.stride + i] : 0ull;
+  const int64_t w = p.w ? __ldg(p.w + i) : 0;
   for (int k = threadIdx.x; k < 5 * 2048; k += 1024) (&s_seen[0][0])[k] = 0;
   if (threadIdx.x < 5) f->top[threadIdx.x] = 0;
   bool dense = true;
@@ -2368,8 +2380,10 @@ __global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, 
     const int distinct = __syncthreads_count(fresh[u]);
     if (threadIdx.x == 0) f->spread[u] = distinct / 1024.f;
   }
+  const int far = __syncthreads_count(w > wmax || w < -wmax);
   if (threadIdx.x == 0) {
-    f->go = cost.pays(*f, cap) ? 1 : 0;
+    f->far = far / 1024.f;
+    f->go = cost.pays(*f, cap, 1.25f) ? 1 : 0;
     f->blocks = 0;
   }
 }
@@ -2415,7 +2429,7 @@ __global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, ui
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(&f->blocks, 1) == (int)gridDim.x - 1) {   // the last CTA decides
     __threadfence();
-    f->go = cost.pays(*f, cap) ? 1 : 0;
+    f->go = cost.pays(*f, cap, 1.f) ? 1 : 0;
   }
 }
 
@@ -2441,7 +2455,7 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   if (cap < 1) return cudaSuccess;
   const UndeclaredCost cost = {(float)n, a0.a, a0.d, a0.w != nullptr, undeclared_least_given()};
   const float kind[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  if (!cost.always && (float)n * cost.gain(0.f, kind) < 25e6f) return cudaSuccess;
+  if (!cost.always && (float)n * cost.gain(0.f, kind, 0.f) < 25e6f) return cudaSuccess;
   const int64_t W = part_window(n, (int64_t)1 << 26);
   const size_t b_part = part_staging_bytes(a0.d, W, sms, a0.w != nullptr), b_tab = ((size_t)a0.a * cap * 24 + 255) & ~(size_t)255;
   char* buf = nullptr;
@@ -2464,7 +2478,13 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   t.rvec = 2;
   t.narrow = 1;
   t.tbl = (uint32_t*)(buf + b_part);
-  k_dom_probe<<<1, 1024, 0, st>>>(a, f, (uint64_t)cap, cost);
+  WeightSample ws = {};
+  e = weight_sample(a, 2, buf, sms, (int64_t)1 << 26, &ws);
+  if (e != cudaSuccess) {
+    cudaFreeAsync(buf, st);
+    return e;
+  }
+  k_dom_probe<<<1, 1024, 0, st>>>(a, f, (uint64_t)cap, cost, ws.wmax);
   const int grid = sms * 8;
   switch (a.a) {
     case 2: k_dom_scan<2><<<grid, 256, 0, st>>>(a, f, (uint64_t)cap, cost); break;
@@ -2474,8 +2494,6 @@ cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int s
   }
   count_launch(2);
   e = cudaGetLastError();
-  WeightSample ws = {};
-  if (e == cudaSuccess) e = weight_sample(a, 2, buf, sms, (int64_t)1 << 26, &ws);
   if (e == cudaSuccess) e = launch_table_l24(a, t, f, sms * 32, st, ws);
   if (e == cudaSuccess) e = run_partitioned(a, t, 2, buf, sms, st, nullptr, nullptr, (int64_t)1 << 26, &f->go);
   // a fixed grid, whose CTAs return at once in the dense case: 1e7 dense tuples 538 us in all with
