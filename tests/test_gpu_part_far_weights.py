@@ -43,10 +43,11 @@ def test_equals_single_phase(far, a, logm, d, n, window, record, monkeypatch):
     assert torch.equal(*got)
 
 
-@pytest.mark.parametrize("a,logm,d,n", [(1, 14, 5, 2_000_000), (5, 16, 9, 1 << 20), (1, 16, 9, 4_000_000)])
-def test_no_dearer_than_single_phase(a, logm, d, n, monkeypatch):
-    """Amounts up to 10^6, uniform keys: within 1.22 times the single-phase update, whose reductions
-    they cost (with items and reductions both paid for: 1.34, 1.31 and 1.27 times)."""
+@pytest.mark.parametrize("a,logm,d,n,took", [(1, 14, 5, 2_000_000, 1.34), (5, 16, 9, 1 << 20, 1.31),
+                                             (1, 16, 9, 4_000_000, 1.27)])
+def test_no_dearer_than_single_phase(a, logm, d, n, took, monkeypatch):
+    """Amounts up to 10^6, uniform keys: the single-phase update's reductions and little more (with items
+    and reductions both paid for, `took` times as much): less than half of the excess is left."""
     g = torch.Generator(device="cuda").manual_seed(4)
     cols = torch.randint(0, 100_000, (a, n), generator=g, device="cuda")
     w = torch.randint(1, 1_000_001, (n,), generator=g, device="cuda")
@@ -58,4 +59,4 @@ def test_no_dearer_than_single_phase(a, logm, d, n, monkeypatch):
 
     two, one = best_times([lambda: update("1"), lambda: update("0")])
     s.close()
-    assert two <= 1.22 * one, (two, one)
+    assert two <= (1 + took) / 2 * one, (two, one)
