@@ -2334,16 +2334,16 @@ struct UndeclaredCost {
     }
     return 2.f * a * d + 1.6f * d + 3.f - t;
   }
-  // slack: factor on the keys up to the largest (a sample does not show it)
-  __device__ bool pays(const FoundDomains& f, uint64_t cap, float slack) const {
+  // scanned: 1.2 a of the tables' cost are the scan, which is behind
+  __device__ bool pays(const FoundDomains& f, uint64_t cap, bool scanned) const {
     float keys = 0.f;
     bool dense = true;
     for (int u = 0; u < a; u++) {
       const unsigned long long top = *(const volatile unsigned long long*)&f.top[u];
       dense = dense && top < cap;
-      keys += slack * ((float)top + 1.f);
+      keys += (float)top + 1.f;
     }
-    return dense && (always || gain(keys, f.spread, f.far) > 0.f);
+    return dense && (always || gain(keys, f.spread, f.far) + (scanned ? 1.2f * a : 0.f) > 0.f);
   }
 };
 
@@ -2383,7 +2383,7 @@ __global__ void __launch_bounds__(1024) k_dom_probe(UpdArgs p, FoundDomains* f, 
   const int far = __syncthreads_count(w > wmax || w < -wmax);
   if (threadIdx.x == 0) {
     f->far = far / 1024.f;
-    f->go = cost.pays(*f, cap, 1.25f) ? 1 : 0;
+    f->go = cost.pays(*f, cap, false) ? 1 : 0;
     f->blocks = 0;
   }
 }
@@ -2429,7 +2429,7 @@ __global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, ui
   __syncthreads();
   if (threadIdx.x == 0 && atomicAdd(&f->blocks, 1) == (int)gridDim.x - 1) {   // the last CTA decides
     __threadfence();
-    f->go = cost.pays(*f, cap, 1.f) ? 1 : 0;
+    f->go = cost.pays(*f, cap, true) ? 1 : 0;
   }
 }
 
