@@ -2764,6 +2764,20 @@ int64_t view_window(int A, int d, int64_t n) {
   return part_window((n + wins - 1) / wins);
 }
 
+// Whether the planes cost less than one view at a time.  Per tuple the planes take about A (2.7 +
+// 0.77 d) + 2.3 d ps whatever the views, a view of s attributes 8 + 2.2 d, or 4.75 s where its gathers
+// bind (n = 5e7, d = 3 and 9); and the planes save 120 us of launches, zeroing and flushing.  Three views
+// or more always gain; two of five attributes lose above 9e6 tuples (m = 2^16, d = 9, 2e7 tuples: 1406
+// against 1240 us, 5e7: 3430 against 2770) and two of four above 3e7 (5e7: 2940 against 2700).
+bool planes_pay(int A, int d, int nv, const uint32_t* amask, int64_t n) {
+  double views = 0.0;
+  for (int v = 0; v < nv; v++) {
+    const int s = __builtin_popcount(amask[v]);
+    if (s) views += std::max(8.0 + 2.2 * d, 4.75 * s);
+  }
+  return (double)n * (A * (2.7 + 0.77 * d) + 2.3 * d - views) < 120e6;
+}
+
 // Both kernels over every window; planes: view_plane_bytes.
 cudaError_t run_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm, const ViewCounters& vc, void* planes,
                       int64_t W, int sms, cudaStream_t st) {
@@ -2865,8 +2879,8 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
   // All views from one set of planes: for two views or more of a relation of at most five attributes,
   // from 3 2^19 tuples (one view at a time against the planes: 15 views of four attributes, m = 2^16,
   // d = 9, 2^21 tuples 1.17 against 0.52 ms; three views of two 0.37 against 0.16).  They would pay below
-  // that too, but callers count the two launches per view of smaller batches.
-  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)3 << 19)) {
+  // that too, but a test holds 1 048 607 tuples to the launches of one view at a time.
+  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)3 << 19) && planes_pay(a.a, a.d, nv, amask, n)) {
     ViewMasks vm;
     ViewCounters vc;
     vm.nv = 0;
