@@ -752,12 +752,12 @@ struct ViewCounters {
   unsigned long long* ctr[SK_MAX_VIEWS];   // [d][m] each
 };
 
-template <int A, bool ALL9>
+template <int A>
 __global__ void __launch_bounds__(256, A <= 4 ? 4 : 3) k_view_planes(UpdArgs p, TabArgs t, ViewPlanes q) {
   const int64_t step = (int64_t)gridDim.x * 256;
   const int64_t gend = (q.cnt + 31) & ~(int64_t)31;
   const unsigned lane = threadIdx.x & 31u;
-  const int d = ALL9 ? 9 : p.d;
+  const int d = p.d;
   const uint64_t pol = policy_evict_first();
   int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
   uint32_t kx[A], okm = 0;   // the thread's next tuple, see k_tab_items
@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(256, A <= 4 ? 4 : 3) k_view_planes(UpdArgs p, 
     uint32_t sb[2] = {0, 0};   // lane l: the sign bits of plane l, of plane 32 + l
 #pragma unroll
     for (int j = 0; j < 9; j++) {
-      if (!ALL9 && j >= d) break;
+      if (j >= d) break;
 #pragma unroll
       for (int u = 0; u < A; u++) {
         const uint32_t x = (uint32_t)(rec[u][j / 3] >> (22 * (j % 3)));   // sign: bit 19
@@ -2738,14 +2738,12 @@ namespace {
 
 using ViewPlanesKernel = void (*)(UpdArgs, TabArgs, ViewPlanes);
 
-template <bool ALL9>
-ViewPlanesKernel view_planes_kernel(int A) {
+ViewPlanesKernel view_planes_kernel(int A) {   // two attributes or more: one has one view
   switch (A) {
-    case 1: return k_view_planes<1, ALL9>;
-    case 2: return k_view_planes<2, ALL9>;
-    case 3: return k_view_planes<3, ALL9>;
-    case 4: return k_view_planes<4, ALL9>;
-    default: return k_view_planes<5, ALL9>;
+    case 2: return k_view_planes<2>;
+    case 3: return k_view_planes<3>;
+    case 4: return k_view_planes<4>;
+    default: return k_view_planes<5>;
   }
 }
 
@@ -2781,7 +2779,7 @@ bool planes_pay(int A, int d, int nv, const uint32_t* amask, int64_t n) {
 // Both kernels over every window; planes: view_plane_bytes.
 cudaError_t run_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm, const ViewCounters& vc, void* planes,
                       int64_t W, int sms, cudaStream_t st) {
-  ViewPlanesKernel make = a.d == 9 ? view_planes_kernel<true>(a.a) : view_planes_kernel<false>(a.a);
+  ViewPlanesKernel make = view_planes_kernel(a.a);
   int per_sm = 0;
   cudaError_t e = cudaFuncSetAttribute((const void*)make, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, make, 256, 0);
@@ -2880,7 +2878,7 @@ sk_status family_partitioned_update(const UpdArgs& a, int nv, const uint32_t* am
   // from 3 2^19 tuples (one view at a time against the planes: 15 views of four attributes, m = 2^16,
   // d = 9, 2^21 tuples 1.17 against 0.52 ms; three views of two 0.37 against 0.16).  They would pay below
   // that too, but a test holds 1 048 607 tuples to the launches of one view at a time.
-  if (nv >= 2 && a.a <= 5 && n >= ((int64_t)3 << 19) && planes_pay(a.a, a.d, nv, amask, n)) {
+  if (nv >= 2 && a.a >= 2 && a.a <= 5 && n >= ((int64_t)3 << 19) && planes_pay(a.a, a.d, nv, amask, n)) {
     ViewMasks vm;
     ViewCounters vc;
     vm.nv = 0;
