@@ -964,8 +964,9 @@ cudaError_t tab_items_per_sm(TabItemsKernel kern, int* per_sm) {
 // Phase-2 split of nwarps regions (`units` (row, part) pairs, `slots` resident CTAs): the number
 // of ranges of regions per pair.  A wave of CTAs costs its share of the items plus a fixed
 // zeroing and flush of 2^15 counters (about 9 us on a GB300 SM, as long as 125 000 items take),
-// so few waves.
-int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps) {
+// so few waves.  uneven: by how much the longest CTAs' shares exceed the others': where one key's
+// items queue at one counter, the part that holds it takes longer, and only more and smaller CTAs spread it.
+int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps, double uneven) {
   double best = 0.0;
   int64_t nr = 1;
   // The star's 18 pairs take one wave of 144 CTAs (star step 3.41 ms, with at least two waves 3.43;
@@ -974,7 +975,8 @@ int64_t part_ranges(int64_t items, int64_t units, int64_t slots, int64_t nwarps)
   for (int64_t k = 1; k <= 16; k++) {
     const int64_t r = std::max<int64_t>(1, k * slots / units);
     const double waves = std::ceil((double)(r * units) / (double)slots);
-    const double cost = waves * ((double)items / (double)(r * units) + 125000.0);
+    const double share = (double)items / (double)(r * units);
+    const double cost = waves * (share + 125000.0) + uneven * share;
     if (best == 0.0 || cost < best) {
       best = cost;
       nr = r;
@@ -1044,9 +1046,9 @@ struct PartSplit {
   int logP;     // pieces per region, log2: a CTA's 32 warps get equal shares
 };
 
-PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps) {
+PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps, double uneven) {
   PartSplit p;
-  p.nr = part_ranges(items, units, slots, nwarps);
+  p.nr = part_ranges(items, units, slots, nwarps, uneven);
   p.R = (int)((nwarps + p.nr - 1) / p.nr);
   p.nr = (nwarps + p.R - 1) / p.R;
   p.logP = 5;
@@ -1064,6 +1066,7 @@ PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps) {
 struct PartPlan {
   TabItemsKernel items;
   void (*accum)(PartArgs, unsigned long long*, int64_t, int, int, int, int);
+  int attrs;
   int64_t W;           // tuples per window
   int64_t full_grid;   // phase-1 CTAs, all resident
   int64_t units;       // (row, part) pairs
@@ -1079,6 +1082,7 @@ cudaError_t part_plan(const UpdArgs& a, int fmt, int sms, int64_t most, PartPlan
   int per_sm = 1;
   cudaError_t e = tab_items_per_sm(pl->items, &per_sm);
   if (e != cudaSuccess) return e;
+  pl->attrs = a.a;
   pl->full_grid = (int64_t)sms * per_sm;
   pl->W = part_window(a.n, most);
   int logm = 0;
@@ -1100,7 +1104,9 @@ int part_regions(const PartPlan& pl, int d, int64_t cnt, PartArgs* q, PartSplit*
   q->cnt = cnt;
   q->C = 32 * ((gend + (int64_t)grid * 256 - 1) / ((int64_t)grid * 256));
   q->nwarps = grid * 8;
-  *sp = part_split(cnt * d, pl.units, pl.slots, q->nwarps);
+  // One attribute's bins are as skewed as its keys; sums of several are not.  With one wave as for
+  // several, 5e7 Zipf (1.1) tuples took 1667 us at m = 2^16, d = 9, now 1322; uniform ones 1033, now 1087.
+  *sp = part_split(cnt * d, pl.units, pl.slots, q->nwarps, pl.attrs == 1 && pl.units > d ? 0.6 : 0.0);
   q->wmax = std::min<int64_t>(65535, 0x7fffffff / ((int64_t)sp->R * q->C));
   return grid;
 }
@@ -2803,7 +2809,7 @@ cudaError_t run_views(const UpdArgs& a, const TabArgs& t, const ViewMasks& vm, c
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
-    const int nr = (int)part_ranges(q.cnt * units, units, slots, (q.cnt + kViewTile - 1) / kViewTile);
+    const int nr = (int)part_ranges(q.cnt * units, units, slots, (q.cnt + kViewTile - 1) / kViewTile, 0.0);
     accum<<<(unsigned)(units * nr), 1024, smem, st>>>(q, vm, vc, a.a, a.d, (int64_t)a.m, logL, nr);
     count_launch();
     e = cudaGetLastError();
