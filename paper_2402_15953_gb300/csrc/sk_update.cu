@@ -1043,16 +1043,20 @@ size_t part_staging_bytes(int d, int64_t W, int sms, bool weighted = false) {
 struct PartSplit {
   int64_t nr;   // ranges per (row, part)
   int R;        // regions per range
-  int logP;     // pieces per region, log2: a CTA's 32 warps get equal shares
+  int logP;     // pieces per region, log2: a CTA's 32 warps get equal shares, a lane of each a chunk or more
 };
 
-PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps, double uneven) {
+// chunks: of 16 bytes, a region has for one part about.  Pieces of fewer chunks than a warp has lanes
+// only idle them (2^20 tuples, m = 2^16, d = 3, 13 chunks: four pieces 66 us, whole 60).
+PartSplit part_split(int64_t items, int64_t units, int64_t slots, int nwarps, int64_t chunks, double uneven) {
   PartSplit p;
   p.nr = part_ranges(items, units, slots, nwarps, uneven);
   p.R = (int)((nwarps + p.nr - 1) / p.nr);
   p.nr = (nwarps + p.R - 1) / p.R;
-  p.logP = 5;
-  for (int lp = 0; lp < 5; lp++) {
+  int most = 0;
+  while (most < 5 && (chunks >> (most + 1)) >= 32) most++;
+  p.logP = most;
+  for (int lp = 0; lp < most; lp++) {
     const int64_t pcs = (int64_t)p.R << lp;
     if ((pcs + 31) / 32 * 32 * 100 <= pcs * 105) {
       p.logP = lp;
@@ -1067,6 +1071,7 @@ struct PartPlan {
   TabItemsKernel items;
   void (*accum)(PartArgs, unsigned long long*, int64_t, int, int, int, int);
   int attrs;
+  bool weighted;
   int64_t W;           // tuples per window
   int64_t full_grid;   // phase-1 CTAs, all resident
   int64_t units;       // (row, part) pairs
@@ -1083,6 +1088,7 @@ cudaError_t part_plan(const UpdArgs& a, int fmt, int sms, int64_t most, PartPlan
   cudaError_t e = tab_items_per_sm(pl->items, &per_sm);
   if (e != cudaSuccess) return e;
   pl->attrs = a.a;
+  pl->weighted = weighted;
   pl->full_grid = (int64_t)sms * per_sm;
   pl->W = part_window(a.n, most);
   int logm = 0;
@@ -1106,7 +1112,8 @@ int part_regions(const PartPlan& pl, int d, int64_t cnt, PartArgs* q, PartSplit*
   q->nwarps = grid * 8;
   // One attribute's bins are as skewed as its keys; sums of several are not.  With one wave as for
   // several, 5e7 Zipf (1.1) tuples took 1667 us at m = 2^16, d = 9, now 1322; uniform ones 1033, now 1087.
-  *sp = part_split(cnt * d, pl.units, pl.slots, q->nwarps, pl.attrs == 1 && pl.units > d ? 0.6 : 0.0);
+  const int64_t chunks = q->C * d / (pl.weighted ? 4 : 8) / pl.units;
+  *sp = part_split(cnt * d, pl.units, pl.slots, q->nwarps, chunks, pl.attrs == 1 && pl.units > d ? 0.6 : 0.0);
   q->wmax = std::min<int64_t>(65535, 0x7fffffff / ((int64_t)sp->R * q->C));
   return grid;
 }
