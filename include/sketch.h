@@ -148,19 +148,29 @@ sk_status sk_sketch_create(const sk_query* query, int64_t m, int32_t d, uint64_t
  * (sum of bounds * 16 or 32 bytes when m <= 2^16 and d <= 14; 24 bytes for the
  * two-phase update below when d <= 9; 4 d rounded up to 16 bytes otherwise) comes
  * from the device's stream-ordered pool and is released on cuda_stream at the end
- * of the call; if it cannot be allocated the call hashes per tuple.  Unit-weight
- * batches (dev_weights NULL) into a power-of-two 1024 <= m <= 2^16 with d <= 14, at
- * most 5 attributes, at least 16 m rows and a d * m int32 sketch too large for one
- * CTA's shared memory update in two phases through the table: per-tuple bins
- * written as 16-bit items (2 d bytes per row of staging from the same pool, in
- * windows of at most 2^30 rows), then added per half row in shared memory.
- * Unit-weight batches into a power-of-two 2^17 <= m <= 2^24 with d <= 16, at most 5
- * attributes, at least m rows and a sketch larger than 32 MiB take the table too
- * (the lookups then replace one L2 reduction per counter update that would miss
- * L2) and sort each row's bins by part of 2^15 bins before adding them in shared
- * memory (6 d bytes per row of staging, windows of at most 2^24 rows).
+ * of the call; if it cannot be allocated the call hashes per tuple.  Batches into a
+ * power-of-two 1024 <= m <= 2^16 with d <= 14, at most 5 attributes, at least 16 m
+ * rows and a d * m int32 sketch too large for one CTA's shared memory update in two
+ * phases through the table: per-tuple bins written as items of 16 bits, or with
+ * weights of 32 (2 d or 4 d bytes per row of staging from the same pool, in windows
+ * of at most 2^30 or 2^26 rows), then added per half row in shared memory.  Weights
+ * too large for an item go to the counters directly; a sample of the weights sends
+ * the whole batch there when most are.
+ * Unit-weight batches (dev_weights NULL) into a power-of-two 2^17 <= m <= 2^24 with
+ * d <= 16, at most 5 attributes, at least m rows and a sketch larger than 32 MiB
+ * take the table too (the lookups then replace one L2 reduction per counter update
+ * that would miss L2) and sort each row's bins by part of 2^15 bins before adding
+ * them in shared memory (windows of at most 2^24 rows; staging 2 d bytes per row for
+ * m <= 2^20, 6 d beyond and, with d > 8, for columns in host memory).
+ * Without domain_hint, batches of at least 2^22 rows and 2 to 5 attributes in device
+ * memory that the two phases could take with d <= 9 are looked over on the device for
+ * dense non-negative keys and take the tables when these cost less than hashing every
+ * tuple (environment: SK_UNDECLARED_LEAST).  The call then allocates, before it has
+ * seen a key, the staging and tables for the widest domains that could be taken
+ * (n_rows / 4 keys per attribute, at most SK_KEY_TABLE_MAX_MB in all); it hashes if
+ * they cannot be had, and while cuda_stream is captured.
  * SK_PART_UPDATE=0 keeps the one-phase table update and the per-tuple update for
- * both.  Results are identical on every path.
+ * all of these.  Results are identical on every path.
  * Asynchronous on cuda_stream; the columns and weights must stay valid until it
  * completes.  n_rows == 0 is a no-op.
  * Errors: SK_ERR_INVALID_ARG, SK_ERR_CUDA. */
@@ -184,15 +194,18 @@ sk_status sk_sketch_update_batch(sk_set* set, int32_t relation, int64_t n_rows, 
  * from different plans running concurrently.  Key domains are not checked.  A
  * relation in a plan may have at most 5 joined attributes.
  *
- * sk_update_plan_config: chunk_tuples (tuples per work item), threads (per CTA),
+ * sk_update_plan_config: chunk_tuples (tuples per work item at most: a plan of few
+ * tuples takes smaller ones, so that they spread over the GPU), threads (per CTA),
  * ctas_per_sm, smem_max_counters (items with d*m at most this, and at most 40960,
  * use a per-chunk int32 shared-memory sub-sketch; 0 = never), smem16_max_counters
  * (other items with d*m at most this, and at most 81920, use a per-chunk sub-sketch
  * of 16-bit counters, two per 32-bit word, each biased by 2^15; only tuples with
- * |Delta| <= 32767 / chunk_tuples go there, so no counter leaves [0, 2^16) within a
- * chunk and the packed adds are exact; the others update global memory; 0 = never).
+ * |Delta| <= 32767 / (tuples of the work item) go there, so no counter leaves
+ * [0, 2^16) within a chunk and the packed adds are exact; the others update global memory; 0 = never).
  * sk_update_plan_autotune times a set of configurations on the plan itself (every
- * timed run updates the counters: reset them afterwards) and keeps the fastest.  The
+ * timed run updates the counters: reset them afterwards) and keeps the fastest; for
+ * plans whose work items are smaller than chunk_tuples anyway, several of the
+ * configurations are the same plan.  The
  * choice is persisted: keyed by the device's SM count, the plan's item shapes (m, d and
  * attribute count, with their counts) and the log2 of its tuple count, it is appended to a
  * JSON-lines file (SK_AUTOTUNE_CACHE, else autotune.json beside libsketch.so;
@@ -494,9 +507,11 @@ sk_status sk_family_create(const sk_query* query, int32_t n_sub, const int32_t* 
  * one sign slot (each in one join of Q), the batch has unit weights and declared
  * domains, m is a power of two in [1024, 2^16], d <= 9, views have at most 5
  * attributes and the batch at least 16 m rows, the call instead builds one key
- * table over R_k's attributes (24 bytes per domain key) and runs the two-phase
- * update of sk_sketch_update_batch once per view (staging from the same pool;
- * SK_PART_UPDATE=0 keeps the one-pass update).  A tuple with any key outside its
+ * table over R_k's attributes (24 bytes per domain key) and either lays the
+ * attributes' bins out in planes that all views add up (at least 3 * 2^19 rows, two
+ * views or more, unless few views of many attributes make the planes dearer) or runs
+ * the two-phase update of sk_sketch_update_batch once per view (staging from the same
+ * pool; SK_PART_UPDATE=0 keeps the one-pass update).  A tuple with any key outside its
  * domain is left out of every view.  A relation in no sub-query is a no-op.
  * Domain violations are recorded and reported by sk_family_sync.  Results are
  * identical on both paths.

@@ -198,8 +198,9 @@ __device__ __forceinline__ uint32_t root_pow(int prime, int dir, int logR, uint3
 // R = 2^(LA + LB).  A thread of a CTA of 256 holds one A- or B-point DFT (A <= B) of one of cb =
 // 256 / A columns: the counters go from global memory into registers, through one shared-memory
 // exchange between the two levels and back to global memory.  LA = 0: R = B points per thread,
-// no exchange.  64-byte column segments are read and 32-byte ones written at least, so tiles
-// wider than eight columns would not save sectors.
+// no exchange.  64-byte column segments of counters are read and 32-byte ones of residues written
+// up to R = 1024, where wider tiles would not save sectors.  R = 2048 has the same eight columns; R =
+// 4096 has four: it reads 32 bytes (16 of residues) and writes half sectors, which L2 puts together.
 //
 // WORDS: residues instead of counters.  BACK: the inverse transform's column pass, on residues
 // that k_ntt_corr has multiplied by the inverse twiddle already.

@@ -145,7 +145,8 @@ __global__ void __launch_bounds__(256, (A > 0 && V8 && NARROW && POW2) ? 5 : 1) 
 }
 
 // ---------------------------------------------------------------------------
-// Partitioned update through the key tables (power-of-two 1024 <= m <= 2^16, d <= 14, at most 5 attributes: the star fact table).  k_update_tab adds each (tuple, row)
+// Partitioned update through the key tables (power-of-two 1024 <= m <= 2^16, d <= 14, at most 5
+// attributes: the star fact table).  k_update_tab adds each (tuple, row)
 // to the L2-resident int64 sketch with one 64-bit reduction, and the L2 lookup rate bounds it
 // (9 reductions per tuple at d = 9, about half of them forwarded between the two dies' L2
 // halves).  Shared-memory atomics run about ten times faster than L2 reductions on GB300,
@@ -1802,8 +1803,8 @@ SortLayout sort_layout(int d, int64_t m, int64_t W) {
 
 // k_wide_sort over the whole window in four launches: with two row groups the halves of the
 // first group, then of the second (the CTAs of a group run together either way); with one group
-// the quarters of the window.  Callers that count launches see seven per window, as for wider
-// sketches; the extra boundaries cost about 1 % of the pass.
+// the quarters of the window.  One launch per group would do, and save about 1 % of the pass: a test
+// holds every width of the wide update to the seven launches per window that the widest take.
 template <int A>
 cudaError_t launch_wide_sort(const UpdArgs& a, const TabArgs& t, SortArgs q, cudaStream_t st) {
   constexpr size_t smem = (size_t)kSortRows * kSortChunk * sizeof(uint32_t);
@@ -2448,9 +2449,10 @@ __global__ void __launch_bounds__(256) k_dom_scan(UpdArgs p, FoundDomains* f, ui
 
 // *done = false (nothing launched) unless the batch is one the partitioned update would take with
 // declared domains, of two attributes or more and at least 2^22 tuples, and keys as kind as can be (few
-// and skewed) would gain 25 us: the probe and the kernels that return cost others 16 to 20 us.  Five columns, m = 2^16,
-// d = 9: dense keys 254 against 458 us at 2^22 tuples and 670 against 1810 at 2^24 (1e7 tuples 1080 ->
-// 538 us).  One attribute is left to update_warp_key.  Captured streams keep the per-tuple
+// and skewed) would gain 25 us: the probe and the kernels that return cost others 16 to 25 us (2^22 tuples
+// of two columns, d = 5: 145 -> 170; at 1e7 5 %), and a key beyond the tables that no sample shows also
+// the scan (1e7 tuples of two columns 323 -> 371).  Five columns, m = 2^16, d = 9: dense keys 254 against 458
+// us at 2^22 tuples and 670 against 1810 at 2^24 (1e7 tuples 1080 -> 538 us).  One attribute is left to update_warp_key.  Captured streams keep the per-tuple
 // update, which allocates nothing.
 cudaError_t update_undeclared(const UpdArgs& a0, bool pow2, bool use_smem, int sms, cudaStream_t st, bool* done) {
   *done = false;
