@@ -437,7 +437,10 @@ def run_ours(args, world, rank, local):
     achieved_gbs = fact_bytes / (fact_ms / 1e3) / 1e9
     mulmods_per_fact_tuple = wl.d * 5 * (1 + 3 * 1)
     fact_s = fact_ms / 1e3
-    tables = not args.no_domains
+    # without declared domains, batches of 2^22 rows and more are looked over for dense keys, which
+    # these are, and take the tables all the same
+    found = args.no_domains and args.fact_rows >= 1 << 22
+    tables = found or not args.no_domains
     if tables:
         # The fact-table update call is three launches, timed together: k_key_table_l24 hashes
         # the 5 x 1e6 declared domain keys once (9 rows each, 24-byte records), k_tab_items
@@ -446,17 +449,21 @@ def run_ours(args, world, rank, local):
         # adds them into a half-row int32 sketch in shared memory, flushing each counter once
         # (phase 2).
         # HBM roofline: algorithmic bytes = the 40 key bytes per tuple.  traffic = DRAM bytes
-        # of one ncu capture of both phases at 2e7 rows (k_tab_items 1.4755 GB read + 0.4119 GB
-        # written, k_part_accum 0.3665 + 0.0002 GB: key stream, record misses and the items'
-        # round trip) scaled to this row count, plus the table write (5e6 x 24 B).
-        # L2 roofline beside it: L2 requests per tuple from the same capture (5.71: 5.21 in
-        # phase 1, 0.50 in phase 2; 16.35 with one 64-bit reduction per counter update).
-        # The bound phase 1 meets is the L1 data pipe: 5.97 wavefronts per tuple (one per
+        # of one ncu capture of both phases at 2e7 rows (k_tab_items 1.4789 GB read + 0.4134 GB
+        # written, k_part_accum 0.3665 + 0.0034 GB: key stream, record misses and the items'
+        # round trip) scaled to this row count, plus the table write (5e6 x 24 B) and, without
+        # declared domains, the scan's second read of the keys.
+        # L2 roofline beside it: L2 requests per tuple from the same capture (5.48: 5.16 in
+        # phase 1, 0.32 in phase 2; 16.35 with one 64-bit reduction per counter update).
+        # The bound phase 1 meets is the L1 data pipe: 5.90 wavefronts per tuple (one per
         # record gather and lane, plus the key loads and item stores), 82 % of its peak of one
         # wavefront per clock and SM in that capture.
-        traffic = (1.4755 + 0.4119 + 0.3665 + 0.0002) * args.fact_rows / 2e7 + 5 * 1_000_000 * 24 / 1e9
+        traffic = (1.4789 + 0.4134 + 0.3665 + 0.0034) * args.fact_rows / 2e7 + 5 * 1_000_000 * 24 / 1e9
         kernel = "k_key_table_l24 + k_tab_items<5,24B> + k_part_accum (fact table F, two-phase)"
-        l2_req_per_tuple = 5.71
+        if found:
+            traffic += fact_bytes / 1e9
+            kernel = "k_dom_probe + k_dom_scan + " + kernel
+        l2_req_per_tuple = 5.48
         l2_peak = 188 * 2.016e9
         l2_rate = l2_req_per_tuple * args.fact_rows / fact_s
         roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
@@ -468,11 +475,11 @@ def run_ours(args, world, rank, local):
                                  "unit": "G requests/s", "frac": l2_rate / l2_peak,
                                  "per_tuple": l2_req_per_tuple, "kernel": kernel,
                                  "source": "ncu lts__t_requests of k_tab_items + k_part_accum (2e7 rows)"},
-                 "roofline_l1_phase1": {"bound": "l1_data_pipe_wavefronts", "per_tuple": 5.97,
-                                        "frac_ncu": 0.824, "kernel": "k_tab_items<5,24B>",
+                 "roofline_l1_phase1": {"bound": "l1_data_pipe_wavefronts", "per_tuple": 5.90,
+                                        "frac_ncu": 0.820, "kernel": "k_tab_items<5,24B>",
                                         "source": "ncu l1tex__data_pipe_lsu_wavefronts (2e7 rows)"}}
     else:
-        # Per-tuple hashing (no declared domains): integer-ALU roofline, algorithmic work =
+        # Per-tuple hashing (no declared domains, short batches): integer-ALU roofline, algorithmic work =
         # GF(2^61-1) Horner multiply-add steps (1 per bin hash, 3 per sign hash), peak = the
         # step rate of the same arithmetic without loads, atomics or combination (6.4 steps
         # per clock per SM measured) x 152 SMs x 2.07 GHz.  traffic: DRAM bytes of one ncu
