@@ -1515,9 +1515,9 @@ __global__ void __launch_bounds__(1024) k_wide_accum(WideArgs q, unsigned long l
 //      a piece whatever the segments' lengths.
 // Per tuple and row 2 bytes are written and read once (the sorted form above: 8 written, 8
 // read), and each item passes one atomic with a returned value instead of two.  Inner chain
-// relation of 1e7 tuples, m = 2^20, d = 16: 758 us against 1063 us (table 88, k_wide_sort 420,
+// relation of 1e7 tuples, m = 2^20, d = 16: 758 us against 1063 us (table 89, k_wide_sort 427,
 // bound by the L1 data pipe at 77 %: two record gathers and 12 shared-memory wavefronts per warp
-// and row; k_wide_gather 230, waiting on the pieces it loads; 352 + 152 us before its list was
+// and row; k_wide_gather 217, waiting on the pieces it loads; 352 + 152 us before its list was
 // ordered for the SMs).
 // ---------------------------------------------------------------------------
 constexpr int kSortLog = 11;
