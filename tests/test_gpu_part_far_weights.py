@@ -43,8 +43,7 @@ def test_equals_single_phase(far, a, logm, d, n, window, record, monkeypatch):
     assert torch.equal(*got)
 
 
-@pytest.mark.parametrize("a,logm,d,n,took", [(1, 14, 5, 2_000_000, 1.34), (5, 16, 9, 1 << 20, 1.31),
-                                             (1, 16, 9, 4_000_000, 1.27)])
+@pytest.mark.parametrize("a,logm,d,n,took", [(1, 14, 5, 2_000_000, 1.34), (5, 16, 9, 20_000_000, 1.2)])
 def test_no_dearer_than_single_phase(a, logm, d, n, took, monkeypatch):
     """Amounts up to 10^6, uniform keys: the single-phase update's reductions and little more (with items
     and reductions both paid for, `took` times as much): less than half of the excess is left."""
